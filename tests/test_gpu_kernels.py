@@ -1,0 +1,90 @@
+"""Kernel edges: sizes at which a kernel changes its layout, word count or path."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2511_20317_gb300 import tfg
+from paper_2511_20317_gb300.tfg import WALKER_INFO_DTYPE
+from paper_2511_20317_gb300.workloads import naive_start
+from test_gpu_walk import THREADS, assert_parity, gpu  # noqa: F401  (gpu: the module's set-up fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _up(x):
+    return (x + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("fmt", [(4, 5, 5), (5, 6, 9)])
+def test_verify_sums_beyond_8_bits(fmt):
+    """Eq. (1) on the device when an entry's partial sums leave 8 bits: 130 copies of
+    a term followed by 130 of its negative cancel (valid), one more copy does not;
+    a checkpoint blob carries the planted best schemes (three 64-bit words per sign)."""
+    n, extra = 6, 262
+    start = naive_start(*fmt)
+    r0 = start.shape[0]
+    W = tfg.Walkers([(fmt, 0, start, n)], seed=1, params=tfg.tfg_default_params(r_slack=extra))
+    blob = np.frombuffer(W.checkpoint(), dtype=np.uint8).copy()
+    info = blob[: n * WALKER_INFO_DTYPE.itemsize].view(WALKER_INFO_DTYPE)
+    R = W.pop[0]["r_max"]
+    per = R * 2 * 3 * 8
+    off = _up(n * WALKER_INFO_DTYPE.itemsize) + _up(n * per)
+    best = blob[off: off + n * per].view(np.uint64).reshape(n, R, 2, 3)
+    for w, (plus, minus) in enumerate([(130, 130), (131, 130), (130, 131), (0, 0), (127, 127), (1, 0)]):
+        t = best[w, 3].copy()                      # one of the naive terms
+        neg = t.copy()
+        neg[1, 2], neg[0, 2] = t[0, 2], 0          # w negated
+        best[w, r0: r0 + plus] = t
+        best[w, r0 + plus: r0 + plus + minus] = neg
+        info["best_r"][w] = r0 + plus + minus
+    W.restore(blob.tobytes())
+    assert W.verify_all() == 3                     # the walkers with one copy too many
+    W.close()
+
+
+@pytest.mark.parametrize("mode", [tfg.TFG_MODE_ZT, tfg.TFG_MODE_Z2])
+@pytest.mark.parametrize("fmt,slack,nw,policy", [
+    ((2, 2, 2), 3, 45, 0), ((2, 3, 4), 8, 60, 0),                         # rows, 32-bit terms, 32 slots
+    ((1, 5, 5), 7, 40, 0), ((1, 5, 5), 8, 70, 0),                         # 64-bit terms, 32 and 33 slots
+    ((3, 4, 5), 4, 40, 0), ((3, 4, 5), 5, 33, 1), ((3, 3, 4), 28, 40, 1),  # 64 and 65 slots; 64 in use
+    ((4, 4, 5), 8, 50, 0), ((4, 4, 5), 8, 33, 2),                         # 88 slots
+    ((4, 4, 5), 3, 20001, 0), ((3, 3, 4), 6, 45001, 1),                   # more than reside at once: terms in device memory
+])
+def test_class_walker_edges(fmt, slack, nw, policy, mode):
+    """The thread-per-walker kernel at the edges of its slot words (32 / 33, 64 / 65,
+    88 slots), both places of the packed terms, the three walk policies."""
+    start = naive_start(*fmt)
+    if mode == tfg.TFG_MODE_Z2:
+        start = np.abs(start).astype(np.int8)
+    steps, L = (700, 120) if nw < 1000 else (400, 120)
+    kw = dict(plateau_len=L if policy == 0 else 10**6, walk_policy=policy, r_slack=slack,
+              expand_thresh=int(0.03 * 2**32) if policy == 1 else 0)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=12, params=tfg.tfg_default_params(mapping=1, **kw))
+    W.walk(steps // 3).walk(steps - steps // 3).sync()
+    take = np.unique(np.linspace(0, nw - 1, 40).astype(int))
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=12, mode=mode, plateau_len=kw["plateau_len"], r_slack=slack, policy=policy,
+                         expand_thresh=kw["expand_thresh"]).walk(steps, THREADS)
+    assert (ref.info["accepted"] > 0).any()
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} slack {slack} policy {policy} mode {mode}")
+    assert W.verify_all() == 0
+    W.close()
+
+
+@pytest.mark.parametrize("nw", [1, 255, 257, 70001])
+def test_stats_equal_the_records(nw):
+    """Counters, extremes and histogram against the records themselves, below, at and
+    above one block of records and beyond the launch's blocks."""
+    W = tfg.Walkers([((2, 2, 2), 1, naive_start(2, 2, 2), nw)], seed=4, params=tfg.tfg_default_params(plateau_len=100))
+    W.walk(300).sync()
+    info, _, _ = W.read_walkers(0, nw, slots=False, best=False)
+    st, hist = W.stats(0, hist_len=64)
+    assert st["walkers"] == nw and st["steps"] == info["t"].sum()
+    for k in ("accepted", "rejected", "nocand", "drops", "merges", "plus", "reductions"):
+        assert st[k] == info[k].sum(), k
+    assert st["min_best_r"] == info["best_r"].min() and st["max_best_r"] == info["best_r"].max()
+    assert np.array_equal(hist, np.bincount(info["best_r"], minlength=64)[:64])
+    W.close()
