@@ -1,4 +1,5 @@
-// Thread-per-walker walk kernel variants (zt32), 128 threads per block.
+// Thread-per-walker variants: Z_T, terms of at most 32 coefficients.
+#include "walk_link.cuh"
 #include "walk_solo.cuh"
 
 #ifndef TFG_SLICED_ZT_BLOCK
@@ -8,10 +9,10 @@
 namespace tfg {
 const WalkVariant *walk_variants_solo_zt32(int *n) {
     static const WalkVariant v[] = {
-        TFG_SOLO_VARIANT(TFG_MODE_ZT, uint32_t, 32, 12, 128),
-        TFG_SOLO_VARIANT(TFG_MODE_ZT, uint32_t, 32, 16, 128),
-        TFG_SOLO_VARIANT(TFG_MODE_ZT, uint32_t, 32, 24, 128),
-        TFG_SOLO_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, 128),
+        TFG_LINK_VARIANT(TFG_MODE_ZT, uint32_t, 32, 12, 32),
+        TFG_LINK_VARIANT(TFG_MODE_ZT, uint32_t, 32, 16, 32),
+        TFG_LINK_VARIANT(TFG_MODE_ZT, uint32_t, 32, 24, 32),
+        TFG_LINK_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, 32),
         TFG_SOLO_SLICED_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, TFG_SLICED_ZT_BLOCK, 9, false),
         TFG_SOLO_SLICED_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, TFG_SLICED_ZT_BLOCK, 9, true),
     };
