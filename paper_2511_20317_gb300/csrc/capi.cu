@@ -1241,7 +1241,27 @@ static int window_steps(tfg_ctx *ctx, int64_t steps, int32_t policy, const void 
     }
     const int H = lg.horizon;
     int32_t *status = &ctx->aux()->status;
-    for (int64_t st = 0; st < steps; ++st) {
+    auto segment_log = [&](const Segment &s) {
+        tfg_log_spec ls = lg;   // the segment's walkers' rings
+        if (H > 1) {
+            ls.d_ring = lg.d_ring + (size_t)s.first * H * 32;
+            ls.d_ring_step = lg.d_ring_step + (size_t)s.first * H;
+        }
+        return ls;
+    };
+    // uniform: all steps but the last in one launch per population and 2^30 steps; the last one
+    // leaves its window in the scratch
+    int64_t done = 0;
+    while (policy == 0 && done < steps - 1) {
+        const int32_t chunk = (int32_t)std::min<int64_t>(steps - 1 - done, 1 << 30);
+        for (const Segment &s : ctx->segs)
+            tfg::launch_window_walk(ctx->desc(s), chunk, d_choices ? d_choices + (size_t)done * N + s.first : nullptr, N,
+                                    segment_log(s), ctx->stream);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "window walk launch");
+        done += chunk;
+    }
+    for (int64_t st = done; st < steps; ++st) {
         for (const Segment &s : ctx->segs)
             tfg::launch_window(ctx->desc(s), nullptr, desc + (size_t)s.first * W, kwin + s.first, ctx->stream);
         if (policy == 1)
@@ -1250,13 +1270,8 @@ static int window_steps(tfg_ctx *ctx, int64_t steps, int32_t policy, const void 
                                          score + (size_t)s.first * W, status, ctx->stream);
         for (const Segment &s : ctx->segs) {
             int32_t *ch = d_choices ? d_choices + (size_t)st * N + s.first : nullptr;
-            tfg_log_spec ls = lg;   // the segment's walkers' rings
-            if (H > 1) {
-                ls.d_ring = lg.d_ring + (size_t)s.first * H * 32;
-                ls.d_ring_step = lg.d_ring_step + (size_t)s.first * H;
-            }
             tfg::launch_window_apply(ctx->desc(s), desc + (size_t)s.first * W, kwin + s.first,
-                                     score + (size_t)s.first * W, policy, eps_thresh, ch, ls, ctx->stream);
+                                     score + (size_t)s.first * W, policy, eps_thresh, ch, segment_log(s), ctx->stream);
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "window step launch");

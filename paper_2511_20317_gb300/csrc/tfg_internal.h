@@ -108,6 +108,8 @@ void launch_window_score(const SegDesc &d, const void *params, const uint2 *desc
                          int *err, cudaStream_t st);
 int launch_window_apply(const SegDesc &d, const uint2 *desc, const int *kwin, const float *score, int policy,
                         uint32_t eps, int32_t *choices, const WindowLog &log, cudaStream_t st);
+void launch_window_walk(const SegDesc &d, int32_t steps, int32_t *choices, int64_t stride, const WindowLog &log,
+                        cudaStream_t st);
 size_t mlp_param_bytes();
 int launch_mlp_score(const void *params, const void *x, int64_t n, float *out, int *err, cudaStream_t st);
 void set_first_wait_limit(int64_t polls);   // test hook of tfg_test_set_wait_limit

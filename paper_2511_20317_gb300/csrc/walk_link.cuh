@@ -21,7 +21,8 @@
 // lane's words side by side: a thread's accesses at a row of its own never
 // conflict with another lane's.  GM: the packed terms stay in the walker's
 // device-memory slots.  PG: the walk policy is read from the descriptor (policies 1
-// and 2); without it the plateau policy is compiled in alone.
+// and 2); without it the plateau policy is compiled in alone.  CNT (window mode): lists
+// at any capacity, and every slot's number of matches (u, v and w) is kept too.
 //
 // What bounds it: the latency of a warp's step (550 to 1300 instructions, most of
 // them in the accepting lanes' short dependent loops, at 35% of the issue rate
@@ -56,17 +57,20 @@ __device__ __forceinline__ uint32_t sign_spread(uint32_t x) {
     return r;
 }
 
-template <int MODE, class Wd, int NW, bool GM, bool PG>
+template <int MODE, class Wd, int NW, bool GM, bool PG, bool CNT = false>
 struct LinkWalker {
     static constexpr bool ZT = (MODE == TFG_MODE_ZT);
     static constexpr int NWS = ZT ? 2 : 1;   // words per slot
-    static constexpr bool ROWS = NW == 1;
+    static constexpr bool ROWS = NW == 1 && !CNT;
+    static constexpr bool kCounts = CNT;
     using T = PTerm<Wd, 1, ZT>;
     using O = Ops<Wd, 1, ZT>;
     using M = Masks<Wd, 1>;
 
     Wd *sm;           // slot k at sm[k * RS]: this thread's shared-memory column, or (GM) the walker's own slots
     uint32_t *ix;     // ROWS: row of slot k, factor f at ix[(3 k + f) * kLane]; lists: next of (k, f) = byte f of ix[k * kLane]
+    uint32_t *cn;     // CNT: matches of slots 2k and 2k + 1 in the halves of cn[k * kLane]
+    int matches;      // CNT: their sum
     uint32_t *hs;     // hash slices: bit b of factor f, word q at hs[((f * 8 + b) * NW + q) * kLane]
     M mk;
     int r, best_r, R;
@@ -83,7 +87,8 @@ struct LinkWalker {
 
     // words of shared memory of a thread
     __host__ __device__ static constexpr size_t thread_bytes(int R) {
-        return (GM ? (size_t)0 : (size_t)R * NWS * sizeof(Wd)) + (size_t)R * (ROWS ? 12 : 4) + (size_t)3 * kHashBits * NW * 4;
+        return (GM ? (size_t)0 : (size_t)R * NWS * sizeof(Wd)) + (size_t)R * (ROWS ? 12 : 4) +
+               (CNT ? (size_t)(R + 1) / 2 * 4 : (size_t)0) + (size_t)3 * kHashBits * NW * 4;
     }
 
     __device__ __forceinline__ static int popc_word(Wd x) {
@@ -127,6 +132,13 @@ struct LinkWalker {
     __device__ __forceinline__ uint32_t &row(int k, int f) const { return ix[(3 * k + f) * kLane]; }
     __device__ __forceinline__ uint8_t &next(int k, int f) const { return reinterpret_cast<uint8_t *>(ix)[k * (kLane * 4) + f]; }
 
+    // CNT: slot k's number of matches changes by n
+    __device__ __forceinline__ void count(int k, int n) {
+        if constexpr (CNT) {
+            reinterpret_cast<uint16_t *>(cn)[(k >> 1) * (kLane * 2) + (k & 1)] += (uint16_t)n;
+            matches += n;
+        }
+    }
     // f(k) for every other slot of slot s's class of factor fc
     template <class F>
     __device__ __forceinline__ void each_match(int s, int fc, F f) const {
@@ -237,7 +249,7 @@ struct LinkWalker {
     // dependent loops.  ROWS: returns the new classes.
     template <bool TWO>
     __device__ __forceinline__ void relink_pair(int sa, int fa, const T &va, int sb, int fb, const T &vb, uint32_t &ea,
-                                                uint32_t &eb) const {
+                                                uint32_t &eb) {
         const Wd ma = mk.of(fa, 0), mb = TWO ? mk.of(fb, 0) : Wd(0);
         uint32_t ca[NW], cb[NW];
         scan(sa, fa, factor_hash(va, ma), ca);
@@ -306,8 +318,8 @@ struct LinkWalker {
             int pa = sa, qa = oa, pb = sb, qb = ob;   // q = next of p
 #pragma unroll 1
             while (qa != sa || (TWO && qb != sb)) {
-                if (qa != sa) { pa = qa; qa = next(pa, fa); }
-                if (TWO && qb != sb) { pb = qb; qb = next(pb, fb); }
+                if (qa != sa) { pa = qa; count(pa, -1); count(sa, -1); qa = next(pa, fa); }
+                if (TWO && qb != sb) { pb = qb; count(pb, -1); count(sb, -1); qb = next(pb, fb); }
             }
             next(pa, fa) = (uint8_t)oa;
             if (TWO) next(pb, fb) = (uint8_t)ob;
@@ -325,14 +337,21 @@ struct LinkWalker {
             next(pa, fa) = (uint8_t)sa;
             next(sa, fa) = (uint8_t)qa;
             if (TWO) { next(pb, fb) = (uint8_t)sb; next(sb, fb) = (uint8_t)qb; }
+            if constexpr (CNT) {
+#pragma unroll 1
+                while (qa != sa || (TWO && qb != sb)) {
+                    if (qa != sa) { count(qa, 1); count(sa, 1); qa = next(qa, fa); }
+                    if (TWO && qb != sb) { count(qb, 1); count(sb, 1); qb = next(qb, fb); }
+                }
+            }
         }
     }
-    __device__ __forceinline__ void relink(int s, int f, const T &v) const {
+    __device__ __forceinline__ void relink(int s, int f, const T &v) {
         uint32_t ea, eb;
         relink_pair<false>(s, f, v, s, f, v, ea, eb);
     }
     // take slot s out of its class of factor f (it becomes a class of its own)
-    __device__ __forceinline__ void unlink(int s, int f) const {
+    __device__ __forceinline__ void unlink(int s, int f) {
         if constexpr (ROWS) {
             uint32_t ch = row(s, f);
             const uint32_t sb = 1u << s;
@@ -345,9 +364,14 @@ struct LinkWalker {
         } else {
             const int n = next(s, f);
             if (n != s) {
-                int p = n;
+                int p = s, q = n;
 #pragma unroll 1
-                for (int q; (q = next(p, f)) != s;) p = q;
+                while (q != s) {
+                    p = q;
+                    count(p, -1);
+                    count(s, -1);
+                    q = next(p, f);
+                }
                 next(p, f) = (uint8_t)n;
                 next(s, f) = (uint8_t)s;
             }
@@ -570,6 +594,10 @@ struct LinkWalker {
             if constexpr (ROWS) row(k, 0) = row(k, 1) = row(k, 2) = 0u;
             else ix[k * kLane] = (uint32_t)k * 0x010101u;
         }
+        if constexpr (CNT) {
+            matches = 0;
+            for (int k = 0; k < (R + 1) / 2; ++k) cn[k * kLane] = 0u;
+        }
 #pragma unroll
         for (int q = 0; q < 3 * kHashBits * NW; ++q) hs[q * kLane] = 0u;
         // the slots enter their classes one after another
@@ -682,6 +710,104 @@ struct LinkWalker {
         }
     }
 
+    // What a step did: the candidate it drew and what became of it.
+    struct Step {
+        int action, i, j, X, rho, sneg;
+    };
+
+    // ---- the flip (Section 3.3.1) of candidate (X, j, rho) on term i = s.i with the
+    // ternary validity test; on acceptance the terms are normalised and stored,
+    // zero terms are removed, and terms that may share a pair of factors with
+    // another slot are queued for the cascade.
+    __device__ __forceinline__ void flip(const T &ti, const T &tj, int policy, Step &s) {
+        const int i = s.i, j = s.j, X = s.X;
+        // (Y, Z) cyclic after X, rho swaps; Y_i += Y_j, Z_j -= s Z_i
+        const int X1 = X == 2 ? 0 : X + 1, X2 = X == 0 ? 2 : X - 1;
+        const int Y = s.rho ? X2 : X1, Z = s.rho ? X1 : X2;
+        s.sneg = (ZT && X == 2) ? (int)(((ti.p[0] ^ tj.p[0]) & mk.m[2][0]) != Wd(0)) : 0;
+        T ti2, tj2;
+        bool ok = O::add(ti, tj, Y, false, mk, ti2);
+        ok &= O::add(tj, ti, Z, s.sneg == 0, mk, tj2);
+        s.action = ok ? kAccept : kReject;
+        if (!ok) return;
+        const bool zi = O::zero(ti2, Y, mk);
+        const bool zj = O::zero(tj2, Z, mk);
+        if (policy == 2) nnz += (zi ? 0u : nnz_of(ti2)) + (zj ? 0u : nnz_of(tj2)) - nnz_of(ti) - nnz_of(tj);
+        canon_factor(ti2, Y);
+        canon_factor(tj2, Z);
+        st(i, ti2);
+        st(j, tj2);
+        // of the other factors the normalisation changes the sign of w at most
+        uint32_t e1, e3;
+        relink_pair<true>(i, Y, ti2, j, Z, tj2, e1, e3);
+        if (zi || zj) {
+            q_push(i);
+            q_push(j);
+            const int hi = i > j ? i : j, lo = i > j ? j : i;
+            const bool zhi = (hi == i) ? zi : zj, zlo = (lo == i) ? zi : zj;
+            if (zhi) { drop(hi); c_drp += 1; }
+            if (zlo) { drop(lo); c_drp += 1; }
+            if (policy == 2) qlen = 0;   // no reduction edges
+        } else if (policy != 2) {
+            // A third slot shares a pair with i' = (X_i, Y_i + Y_j, Z_i) iff it is in two of
+            // its classes x, e1, z, and with j' = (X_j, Y_j, Z_j - s Z_i), X_j = +-X_i, iff in
+            // two of x, e2, e3.  i' and j' share X and never another factor: that
+            // would need Y_i = 0, or Z_j equal to 0 or to +-2 Z_i.
+            if constexpr (ROWS) {
+                const uint32_t cx = row(i, X) & ~(1u << j), cz = row(i, Z), e2 = row(j, Y);
+                if ((cx & cz) | (e1 & (cx | cz)) | (e2 & (cx | e3)) | (cx & e3)) { q_push(i); q_push(j); }
+            } else {
+                // sets of members modulo 32 (a superset test: the cascade checks exactly)
+                uint32_t cx = 0u, cz = 0u, a1 = 0u, a2 = 0u, a3 = 0u;
+                int px = next(i, X), pz = next(i, Z), p1 = next(i, Y), p2 = next(j, Y), p3 = next(j, Z);
+#pragma unroll 1
+                while ((px ^ i) | (pz ^ i) | (p1 ^ i) | (p2 ^ j) | (p3 ^ j)) {
+                    if (px != i) { cx |= px != j ? 1u << (px & 31) : 0u; px = next(px, X); }
+                    if (pz != i) { cz |= 1u << (pz & 31); pz = next(pz, Z); }
+                    if (p1 != i) { a1 |= 1u << (p1 & 31); p1 = next(p1, Y); }
+                    if (p2 != j) { a2 |= 1u << (p2 & 31); p2 = next(p2, Y); }
+                    if (p3 != j) { a3 |= 1u << (p3 & 31); p3 = next(p3, Z); }
+                }
+                if ((cx & cz) | (a1 & (cx | cz)) | (a2 & (cx | a3)) | (cx & a3)) { q_push(i); q_push(j); }
+            }
+        }
+    }
+
+    // ---- rest of a step, warp-converged, after the cascade of its flip: digest, best
+    // scheme, plateau, expansion (and its cascade).  x2, x3: the step's third and
+    // fourth draw.  Returns whether any lane's scheme changed here.
+    __device__ __forceinline__ bool finish(const SegDesc &d, unsigned wmask, int lane, int nl, Wd *bestp, int policy,
+                                           uint32_t x2, uint32_t x3, const Step &s) {
+        dig = digest_mix(dig, ((uint64_t)((uint32_t)r << 8) << 32) |
+                                  ((uint32_t)s.action | ((uint32_t)s.X << 4) | ((uint32_t)s.rho << 6) |
+                                   ((uint32_t)s.sneg << 7) | ((uint32_t)s.i << 8) | ((uint32_t)s.j << 24)));
+        // walk policy 1: a failed try_flip expands and ends the step (no best update)
+        const bool failed = policy == 1 && s.action != kAccept;
+        // the best scheme is the one of least rank (policy 2: least (rank, non-zero coefficients))
+        const bool better = !failed && (r < best_r || (policy == 2 && r == best_r && nnz < best_nnz));
+        const bool again = !failed && r == best_r && (policy != 2 || nnz == best_nnz) && x2 < d.refresh_thresh;
+        bool expand;
+        if (policy == 0) expand = t >= t_exp;   // and more, below
+        else if (policy == 1) expand = failed || x3 < d.expand_thresh;
+        else expand = false;
+        if (!__any_sync(wmask, better | again | expand)) return false;
+        if (better) {
+            best_r = r;
+            if (policy == 2) best_nnz = nnz;
+            best_t = t;
+            restart(d);
+        }
+        coop_snapshot(wmask, lane, nl, better | again, bestp);
+        if (policy == 0) expand = d.plus_enabled && t >= t_exp;
+        expand = expand && r < R && r >= 2 && (failed || r <= best_r + 2);
+        if (!__any_sync(wmask, expand)) return false;
+        uint64_t rec = 0;
+        if (expand) rec = plus_setup(d);
+        cascade_all(wmask);
+        if (rec) dig = digest_mix(dig, rec | ((uint64_t)(uint32_t)r << 44));
+        return true;
+    }
+
     __device__ __forceinline__ void run(const SegDesc &d, int64_t w, int32_t steps) {
         load(d, w);
         Wd *bestp = reinterpret_cast<Wd *>(d.best) + (size_t)w * R * NWS;
@@ -699,115 +825,51 @@ struct LinkWalker {
             const int64_t tn = t + 1;
             const U4 xn = philox10((uint32_t)tn, (uint32_t)(tn >> 32), wid, 0u, key0, key1);   // the next step's draws
             // ---- try_flip (Algorithm 1): candidates X_j = +-X_i, ordered (X, slot, rho)
-            const int i = s.i, r_before = r;
-            int action = kNoCand, X = 0, j = 0, rho = 0, sneg = 0;
+            const int r_before = r;
+            Step did{kNoCand, s.i, 0, 0, 0, 0};
             Cand c;
             candidates(s, c);
             const int n01 = c.n0 + c.n1, K = 2 * (n01 + c.n2);
             if (K > 0) {
                 const int ch = (int)__umulhi(x.y, (uint32_t)K);
-                rho = ch & 1;
+                did.rho = ch & 1;
                 const int mi = ch >> 1;
-                X = (int)(mi >= c.n0) + (int)(mi >= n01);
-                j = member(s, X, mi - (X == 0 ? 0 : (X == 1 ? c.n0 : n01)), c);
-                const T ti = s.ti, tj = ld(j);
-                // (Y, Z) cyclic after X, rho swaps; Y_i += Y_j, Z_j -= s Z_i
-                const int X1 = X == 2 ? 0 : X + 1, X2 = X == 0 ? 2 : X - 1;
-                const int Y = rho ? X2 : X1, Z = rho ? X1 : X2;
-                sneg = (ZT && X == 2) ? (int)(((ti.p[0] ^ tj.p[0]) & mk.m[2][0]) != Wd(0)) : 0;
-                T ti2, tj2;
-                bool ok = O::add(ti, tj, Y, false, mk, ti2);
-                ok &= O::add(tj, ti, Z, sneg == 0, mk, tj2);
-                action = ok ? kAccept : kReject;
-                if (ok) {
-                    const bool zi = O::zero(ti2, Y, mk);
-                    const bool zj = O::zero(tj2, Z, mk);
-                    if (policy == 2) nnz += (zi ? 0u : nnz_of(ti2)) + (zj ? 0u : nnz_of(tj2)) - nnz_of(ti) - nnz_of(tj);
-                    canon_factor(ti2, Y);
-                    canon_factor(tj2, Z);
-                    st(i, ti2);
-                    st(j, tj2);
-                    // of the other factors the normalisation changes the sign of w at most
-                    uint32_t e1, e3;
-                    relink_pair<true>(i, Y, ti2, j, Z, tj2, e1, e3);
-                    if (zi || zj) {
-                        q_push(i);
-                        q_push(j);
-                        const int hi = i > j ? i : j, lo = i > j ? j : i;
-                        const bool zhi = (hi == i) ? zi : zj, zlo = (lo == i) ? zi : zj;
-                        if (zhi) { drop(hi); c_drp += 1; }
-                        if (zlo) { drop(lo); c_drp += 1; }
-                        if (policy == 2) qlen = 0;   // no reduction edges
-                    } else if (policy != 2) {
-                        // A third slot shares a pair with i' = (X_i, Y_i + Y_j, Z_i) iff it is in two of
-                        // its classes x, e1, z, and with j' = (X_j, Y_j, Z_j - s Z_i), X_j = +-X_i, iff in
-                        // two of x, e2, e3.  i' and j' share X and never another factor: that
-                        // would need Y_i = 0, or Z_j equal to 0 or to +-2 Z_i.
-                        if constexpr (ROWS) {
-                            const uint32_t cx = (X == 0 ? s.l[0] : (X == 1 ? s.l[1] : s.l[2])) & ~(1u << j);
-                            const uint32_t cz = Z == 0 ? s.l[0] : (Z == 1 ? s.l[1] : s.l[2]);
-                            const uint32_t e2 = row(j, Y);
-                            if ((cx & cz) | (e1 & (cx | cz)) | (e2 & (cx | e3)) | (cx & e3)) { q_push(i); q_push(j); }
-                        } else {
-                            // sets of members modulo 32 (a superset test: the cascade checks exactly)
-                            uint32_t cx = 0u, cz = 0u, a1 = 0u, a2 = 0u, a3 = 0u;
-                            int px = next(i, X), pz = next(i, Z), p1 = next(i, Y), p2 = next(j, Y), p3 = next(j, Z);
-#pragma unroll 1
-                            while ((px ^ i) | (pz ^ i) | (p1 ^ i) | (p2 ^ j) | (p3 ^ j)) {
-                                if (px != i) { cx |= px != j ? 1u << (px & 31) : 0u; px = next(px, X); }
-                                if (pz != i) { cz |= 1u << (pz & 31); pz = next(pz, Z); }
-                                if (p1 != i) { a1 |= 1u << (p1 & 31); p1 = next(p1, Y); }
-                                if (p2 != j) { a2 |= 1u << (p2 & 31); p2 = next(p2, Y); }
-                                if (p3 != j) { a3 |= 1u << (p3 & 31); p3 = next(p3, Z); }
-                            }
-                            if ((cx & cz) | (a1 & (cx | cz)) | (a2 & (cx | a3)) | (cx & a3)) { q_push(i); q_push(j); }
-                        }
-                    }
-                }
+                const int X = (int)(mi >= c.n0) + (int)(mi >= n01);
+                did.X = X;
+                did.j = member(s, X, mi - (X == 0 ? 0 : (X == 1 ? c.n0 : n01)), c);
+                flip(s.ti, ld(did.j), policy, did);
             }
-            c_acc += action == kAccept;
-            c_rej += action == kReject;
+            c_acc += did.action == kAccept;
+            c_rej += did.action == kReject;
             cascade_all(wmask);
-            // ---- the next step's term, unless this one still expands (below)
+            // ---- the next step's term, unless this one still expands
             fetch(xn.x, s);
-            // ---- digest, best scheme and plateau
             c_red += r < r_before;
-            dig = digest_mix(dig, ((uint64_t)((uint32_t)r << 8) << 32) |
-                                      ((uint32_t)action | ((uint32_t)X << 4) | ((uint32_t)rho << 6) | ((uint32_t)sneg << 7) |
-                                       ((uint32_t)i << 8) | ((uint32_t)j << 24)));
-            // walk policy 1: a failed try_flip expands and ends the step (no best update)
-            const bool failed = policy == 1 && action != kAccept;
-            // the best scheme is the one of least rank (policy 2: least (rank, non-zero coefficients))
-            const bool better = !failed && (r < best_r || (policy == 2 && r == best_r && nnz < best_nnz));
-            const bool again = !failed && r == best_r && (policy != 2 || nnz == best_nnz) && x.z < d.refresh_thresh;
-            bool expand;
-            if (policy == 0) expand = t >= t_exp;   // and more, below
-            else if (policy == 1) expand = failed || x.w < d.expand_thresh;
-            else expand = false;
-            if (__any_sync(wmask, better | again | expand)) {
-                if (better) {
-                    best_r = r;
-                    if (policy == 2) best_nnz = nnz;
-                    best_t = t;
-                    restart(d);
-                }
-                coop_snapshot(wmask, lane, nl, better | again, bestp);
-                if (policy == 0) expand = d.plus_enabled && t >= t_exp;
-                expand = expand && r < R && r >= 2 && (failed || r <= best_r + 2);
-                if (__any_sync(wmask, expand)) {
-                    uint64_t rec = 0;
-                    if (expand) rec = plus_setup(d);
-                    cascade_all(wmask);
-                    if (rec) dig = digest_mix(dig, rec | ((uint64_t)(uint32_t)r << 44));
-                    fetch(xn.x, s);
-                }
-            }
+            if (finish(d, wmask, lane, nl, bestp, policy, x.z, x.w, did)) fetch(xn.x, s);
             x = xn;
             t = tn;
         }
         store(d, w, (uint32_t)steps);
     }
 };
+
+// Rows of a thread's warp in shared memory: terms (unless in device memory), classes,
+// counts, slices.
+template <class LW, class Wd>
+__device__ __forceinline__ void link_rows(LW &wk, const SegDesc &d, int64_t w, bool in_device, unsigned char *smem) {
+    const int lane = threadIdx.x & 31;
+    unsigned char *at = smem + (size_t)(threadIdx.x >> 5) * (LW::thread_bytes(d.R) * 32);
+    if (in_device) {
+        wk.sm = reinterpret_cast<Wd *>(d.slots) + (size_t)w * d.R * LW::NWS;
+    } else {
+        wk.sm = reinterpret_cast<Wd *>(at) + lane * LW::NWS;
+        at += (size_t)d.R * 32 * LW::NWS * sizeof(Wd);
+    }
+    wk.ix = reinterpret_cast<uint32_t *>(at) + lane;
+    uint32_t *after = wk.ix + (size_t)d.R * 32 * (LW::ROWS ? 3 : 1);
+    wk.cn = after;
+    wk.hs = after + (LW::kCounts ? (size_t)(d.R + 1) / 2 * 32 : (size_t)0);
+}
 
 // Blocks of any whole number of warps (kLinkMaxBlock threads at most): a warp's
 // rows are its own.
@@ -819,16 +881,7 @@ __global__ void __launch_bounds__(kLinkMaxBlock, 3) walk_link_kernel(const SegDe
     if (w >= d.n_walkers) return;   // no block-wide barrier is used
     using LW = LinkWalker<MODE, Wd, NW, GM, PG>;
     LW wk;
-    const int lane = threadIdx.x & 31;
-    unsigned char *at = smem_raw + (size_t)(threadIdx.x >> 5) * (LW::thread_bytes(d.R) * 32);
-    if constexpr (GM) {
-        wk.sm = reinterpret_cast<Wd *>(d.slots) + (size_t)w * d.R * LW::NWS;
-    } else {
-        wk.sm = reinterpret_cast<Wd *>(at) + lane * LW::NWS;
-        at += (size_t)d.R * 32 * LW::NWS * sizeof(Wd);
-    }
-    wk.ix = reinterpret_cast<uint32_t *>(at) + lane;
-    wk.hs = wk.ix + (size_t)d.R * 32 * (LW::ROWS ? 3 : 1);
+    link_rows<LW, Wd>(wk, d, w, GM, smem_raw);
     wk.run(d, w, steps);
 }
 
@@ -862,19 +915,21 @@ void prepare_walk_link() {
 // resident) 9.2e9 / 7.0e9; (3,3,4) 40330 walkers (1.1 times what fits) 1.02e10 /
 // 1.24e10; (4,4,5) 80660 walkers (4.5 times) 5.3e9 / 9.5e9.  32-bit terms (at
 // most 32 slots of 8 bytes) always go to shared memory.
+inline bool link_terms_shared(size_t block_bytes, int64_t grid) {
+    if (block_bytes > (size_t)kLinkSmem) return false;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return grid <= (int64_t)sms * (int64_t)(kLinkSmem / (block_bytes + 1024));   // 1 KB a block is the system's
+}
+
 template <int MODE, class Wd, int NW>
 void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
     prepare_walk_link<MODE, Wd, NW>();
     using Shared = dev::LinkWalker<MODE, Wd, NW, false, false>;
     using Device = dev::LinkWalker<MODE, Wd, NW, true, false>;
     const size_t block_bytes = Shared::thread_bytes(d.R) * block;
-    bool shared = sizeof(Wd) == 4;
-    if (!shared && block_bytes <= (size_t)kLinkSmem) {
-        int dev = 0, sms = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        shared = (int64_t)grid <= (int64_t)sms * (int64_t)(kLinkSmem / (block_bytes + 1024));   // 1 KB a block is the system's
-    }
+    const bool shared = sizeof(Wd) == 4 || link_terms_shared(block_bytes, grid);
     const size_t smem = shared ? block_bytes : Device::thread_bytes(d.R) * block;
     if (shared) {
         if (d.walk_policy == 0) dev::walk_link_kernel<MODE, Wd, NW, false, false><<<grid, block, smem, st>>>(d, steps);

@@ -20,6 +20,7 @@
 #include <cuda_bf16.h>
 
 #include "mlp_pipe.cuh"
+#include "walk_link.cuh"
 #include "walk_solo.cuh"
 
 namespace tfg {
@@ -331,6 +332,145 @@ __device__ __forceinline__ void write_log_entry(const WindowLog &log, unsigned l
     e->pad = 0;
 }
 
+// Logs a step's chosen candidate: features lf (of the state before the flip), positive:
+// the step's reductions lowered the rank.
+__device__ __forceinline__ void log_step(const WindowLog &log, int64_t w, const uint32_t (&lf)[kFeat / 2], bool positive,
+                                         int64_t t_step, uint32_t wid, uint32_t key0, uint32_t key1) {
+    const int H = log.horizon > 1 ? log.horizon : 1;
+    bool keep0 = false;
+    if (!positive && log.neg_thresh) {
+        const U4 y = philox10((uint32_t)t_step, (uint32_t)(t_step >> 32), wid, 0x100u, key0, key1);
+        keep0 = y.x < log.neg_thresh;
+    }
+    if (H > 1) {
+        // this step's features into ring slot t mod H; a rank-lowering step appends the
+        // entries of steps t-H+1 .. t still in the ring (step order) and empties it
+        uint4 *ring = reinterpret_cast<uint4 *>(log.d_ring) + (size_t)w * H * (kFeat / 8);
+        uint32_t *rs = log.d_ring_step + (size_t)w * H;
+        const int kt = (int)(t_step % H);
+#pragma unroll
+        for (int k = 0; k < kFeat / 8; ++k)
+            ring[kt * (kFeat / 8) + k] = make_uint4(lf[4 * k], lf[4 * k + 1], lf[4 * k + 2], lf[4 * k + 3]);
+        rs[kt] = (uint32_t)t_step;
+        if (positive) {
+            int n = 0;
+            for (int dd = 0; dd < H && dd <= t_step; ++dd)
+                n += rs[(int)((t_step - dd) % H)] == (uint32_t)(t_step - dd);
+            unsigned long long slot = atomicAdd(reinterpret_cast<unsigned long long *>(log.d_count),
+                                                (unsigned long long)n);
+            for (int dd = H - 1; dd >= 0; --dd) {
+                if (dd > t_step) continue;
+                const int k = (int)((t_step - dd) % H);
+                if (rs[k] != (uint32_t)(t_step - dd)) continue;
+                if (slot < (unsigned long long)log.capacity) {
+                    uint32_t e16[kFeat / 2];
+#pragma unroll
+                    for (int q = 0; q < kFeat / 8; ++q) {
+                        const uint4 v = ring[k * (kFeat / 8) + q];
+                        e16[4 * q] = v.x; e16[4 * q + 1] = v.y; e16[4 * q + 2] = v.z; e16[4 * q + 3] = v.w;
+                    }
+                    write_log_entry(log, slot, e16, 1.f, wid, (uint32_t)(t_step - dd));
+                }
+                ++slot;
+            }
+            for (int k = 0; k < H; ++k) rs[k] = 0xFFFFFFFFu;
+        }
+    }
+    const bool keep = (H == 1 && positive) || keep0;
+    if (keep) {
+        const unsigned long long slot = atomicAdd(reinterpret_cast<unsigned long long *>(log.d_count), 1ull);
+        if (slot < (unsigned long long)log.capacity) write_log_entry(log, slot, lf, positive ? 1.f : 0.f, wid,
+                                                                     (uint32_t)t_step);
+    }
+}
+
+// Steps of uniform window walks, many per launch, one walker per thread, on the walker with
+// kept factor classes (walk_link.cuh).  Uniform choice needs of the window only its
+// size and the chosen row: with every slot's number of matches n_k kept
+// beside the classes, K = min(256, 2 sum n_k), and row c belongs to the first term
+// after i0 whose running sum of 2 n_k exceeds c.
+// Bound by the latency of a step, most of it the walk over the counts (two slots a
+// word, 15 to 33 words a step on (4,4,4)).  Measured on (4,4,4), 262144 walkers: 2.17 ms a
+// step with a window kernel that lists all 256 rows and an apply kernel per step,
+// now 0.1 ms (20 steps, the last one by those kernels: 43.6, now 4.1 ms);
+// 4096 logged walkers (the training data), 500 steps: 28.4 ms, now 2.6.
+template <class Wd, int NW, bool GM>
+__global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int32_t steps, int32_t *__restrict__ choices,
+                                                            int64_t choice_stride, WindowLog log) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= d.n_walkers) return;   // no block-wide barrier is used
+    using LW = LinkWalker<TFG_MODE_ZT, Wd, NW, GM, false, true>;
+    using T = typename LW::T;
+    LW wk;
+    link_rows<LW, Wd>(wk, d, w, GM, smem_raw);
+    wk.load(d, w);
+    Wd *bestp = reinterpret_cast<Wd *>(d.best) + (size_t)w * d.R * 2;
+    const unsigned wmask = __activemask();
+    const int lane = threadIdx.x & 31;
+    const int nl = __popc(wmask);
+    U4 x = philox10((uint32_t)wk.t, (uint32_t)(wk.t >> 32), wk.wid, 0u, wk.key0, wk.key1);
+#pragma unroll 1
+    for (int32_t step = 0; step < steps; ++step) {
+        const int64_t t_step = wk.t, tn = wk.t + 1;
+        const U4 xn = philox10((uint32_t)tn, (uint32_t)(tn >> 32), wk.wid, 0u, wk.key0, wk.key1);
+        const int r = wk.r, i0 = (int)__umulhi(x.x, (uint32_t)r);
+        typename LW::Step did{kNoCand, i0, 0, 0, 0, 0};
+        const int K = min(2 * wk.matches, kWin);
+        int c = -1;
+        uint32_t lf[kFeat / 2];   // logged features of the chosen candidate (state before the flip)
+        if (K > 0) {
+            c = (int)__umulhi(x.y, (uint32_t)K);
+            // the term of row c: skip c / 2 matches from i0 on (around the last slot)
+            const int nw = (r + 1) >> 1;
+            int left = c >> 1, wi = i0 >> 1;
+            uint32_t v = wk.cn[wi * kLane] & ((i0 & 1) ? 0xffff0000u : ~0u);
+#pragma unroll 1
+            for (int n = 0; n < nw; ++n) {
+                const int sum = (int)(v & 0xffffu) + (int)(v >> 16);
+                if (left < sum) break;
+                left -= sum;
+                wi = wi + 1 == nw ? 0 : wi + 1;
+                v = wk.cn[wi * kLane];
+            }
+            const int lo = (int)(v & 0xffffu), odd = (int)(left >= lo);
+            left -= odd ? lo : 0;
+            const int n_i = odd ? (int)(v >> 16) : lo;
+            typename LW::Sample s;
+            s.i = 2 * wi + odd;
+            s.ti = wk.ld(s.i);
+            s.l[0] = wk.ix[s.i * kLane];
+            did.i = s.i;
+            did.rho = c & 1;
+            typename LW::Cand cd;
+            wk.candidates(s, cd);
+            const int n01 = cd.n0 + cd.n1;
+            did.X = (int)(left >= cd.n0) + (int)(left >= n01);
+            did.j = wk.member(s, did.X, left - (did.X == 0 ? 0 : (did.X == 1 ? cd.n0 : n01)), cd);
+            const T tj = wk.ld(did.j);
+            if (log.d_entries) {
+                const int sneg = did.X == 2 ? (int)(((s.ti.p[0] ^ tj.p[0]) & wk.mk.m[2][0]) != Wd(0)) : 0;
+                const int q = s.i >= i0 ? s.i - i0 : s.i - i0 + r;
+                const uint32_t info = (uint32_t)min(2 * n_i, 64) | ((uint32_t)min(q, 64) << 8);
+                cand_features_bf16<Wd>(s.ti, tj, wk.mk, pack_cand(s.i, did.X, did.j, sneg, did.rho), info, r, wk.best_r, d.m,
+                                       d.n, d.p, lf);
+            }
+            wk.flip(s.ti, tj, 0, did);
+        }
+        wk.c_acc += did.action == kAccept;
+        wk.c_rej += did.action == kReject;
+        wk.cascade_all(wmask);
+        const bool lowered = wk.r < r;
+        wk.c_red += lowered;
+        if (choices) choices[(int64_t)step * choice_stride + w] = c;
+        if (log.d_entries && c >= 0) log_step(log, w, lf, lowered, t_step, wk.wid, wk.key0, wk.key1);
+        wk.finish(d, wmask, lane, nl, bestp, 0, x.z, x.w, did);
+        x = xn;
+        wk.t = tn;
+    }
+    wk.store(d, w, (uint32_t)steps);
+}
+
 // One window-mode step per thread (walker), on the solo walker's state machine.
 template <class Wd, int RMAX, int BT>
 __global__ void __launch_bounds__(BT) window_apply_kernel(const SegDesc d, const uint2 *__restrict__ desc,
@@ -388,55 +528,7 @@ __global__ void __launch_bounds__(BT) window_apply_kernel(const SegDesc d, const
     }
     wk.finish_step(d, wmask, lane, nl, bestp, x.z, x.w, r_before, action, X, rho, sneg, i, j, need_check, ti2, tj2);
     if (choices) choices[w] = c;
-    if (log.d_entries && c >= 0) {
-        const bool positive = wk.c_red > 0;   // the flip's reductions lowered the rank this step
-        const int H = log.horizon > 1 ? log.horizon : 1;
-        bool keep0 = false;
-        if (!positive && log.neg_thresh) {
-            const U4 y = philox10((uint32_t)t_step, (uint32_t)(t_step >> 32), wk.wid, 0x100u, wk.key0, wk.key1);
-            keep0 = y.x < log.neg_thresh;
-        }
-        if (H > 1) {
-            // this step's features into ring slot t mod H; a rank-lowering step appends the
-            // entries of steps t-H+1 .. t still in the ring (step order) and empties it
-            uint4 *ring = reinterpret_cast<uint4 *>(log.d_ring) + (size_t)w * H * (kFeat / 8);
-            uint32_t *rs = log.d_ring_step + (size_t)w * H;
-            const int kt = (int)(t_step % H);
-#pragma unroll
-            for (int k = 0; k < kFeat / 8; ++k)
-                ring[kt * (kFeat / 8) + k] = make_uint4(lf[4 * k], lf[4 * k + 1], lf[4 * k + 2], lf[4 * k + 3]);
-            rs[kt] = (uint32_t)t_step;
-            if (positive) {
-                int n = 0;
-                for (int dd = 0; dd < H && dd <= t_step; ++dd)
-                    n += rs[(int)((t_step - dd) % H)] == (uint32_t)(t_step - dd);
-                unsigned long long slot = atomicAdd(reinterpret_cast<unsigned long long *>(log.d_count),
-                                                    (unsigned long long)n);
-                for (int dd = H - 1; dd >= 0; --dd) {
-                    if (dd > t_step) continue;
-                    const int k = (int)((t_step - dd) % H);
-                    if (rs[k] != (uint32_t)(t_step - dd)) continue;
-                    if (slot < (unsigned long long)log.capacity) {
-                        uint32_t e16[kFeat / 2];
-#pragma unroll
-                        for (int q = 0; q < kFeat / 8; ++q) {
-                            const uint4 v = ring[k * (kFeat / 8) + q];
-                            e16[4 * q] = v.x; e16[4 * q + 1] = v.y; e16[4 * q + 2] = v.z; e16[4 * q + 3] = v.w;
-                        }
-                        write_log_entry(log, slot, e16, 1.f, wk.wid, (uint32_t)(t_step - dd));
-                    }
-                    ++slot;
-                }
-                for (int k = 0; k < H; ++k) rs[k] = 0xFFFFFFFFu;
-            }
-        }
-        const bool keep = (H == 1 && positive) || keep0;
-        if (keep) {
-            const unsigned long long slot = atomicAdd(reinterpret_cast<unsigned long long *>(log.d_count), 1ull);
-            if (slot < (unsigned long long)log.capacity) write_log_entry(log, slot, lf, positive ? 1.f : 0.f, wk.wid,
-                                                                         (uint32_t)t_step);
-        }
-    }
+    if (log.d_entries && c >= 0) log_step(log, w, lf, wk.c_red > 0, t_step, wk.wid, wk.key0, wk.key1);
     wk.store(d, w);
 }
 
@@ -512,6 +604,39 @@ int launch_window_apply(const SegDesc &d, const uint2 *desc, const int *kwin, co
         else return -1;
     }
     return 0;
+}
+
+template <class Wd, int NW>
+static void window_walk_variant(const SegDesc &d, int32_t steps, int32_t *choices, int64_t stride, const WindowLog &log,
+                                cudaStream_t st) {
+    using Shared = dev::LinkWalker<TFG_MODE_ZT, Wd, NW, false, false, true>;
+    using Device = dev::LinkWalker<TFG_MODE_ZT, Wd, NW, true, false, true>;
+    constexpr int kBlock = 64;
+    static bool attr = [] {
+        cudaFuncSetAttribute(dev::window_walk_kernel<Wd, NW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinkSmem);
+        if constexpr (sizeof(Wd) == 8)
+            cudaFuncSetAttribute(dev::window_walk_kernel<Wd, NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinkSmem);
+        return true;
+    }();
+    (void)attr;
+    const unsigned grid = (unsigned)((d.n_walkers + kBlock - 1) / kBlock);
+    const size_t bytes = Shared::thread_bytes(d.R) * kBlock;
+    if (sizeof(Wd) == 4 || link_terms_shared(bytes, grid)) {
+        dev::window_walk_kernel<Wd, NW, false><<<grid, kBlock, bytes, st>>>(d, steps, choices, stride, log);
+    } else if constexpr (sizeof(Wd) == 8) {
+        dev::window_walk_kernel<Wd, NW, true><<<grid, kBlock, Device::thread_bytes(d.R) * kBlock, st>>>(d, steps, choices,
+                                                                                                        stride, log);
+    }
+}
+
+// `steps` uniform window steps of a population that window_apply_capacity accepts.
+// choices (may be null): the first step's row of the population's walkers, `stride` apart.
+void launch_window_walk(const SegDesc &d, int32_t steps, int32_t *choices, int64_t stride, const WindowLog &log,
+                        cudaStream_t st) {
+    if (d.n_walkers <= 0 || steps <= 0) return;
+    if (d.word_bits == 32) window_walk_variant<uint32_t, 1>(d, steps, choices, stride, log, st);
+    else if (d.R <= 64) window_walk_variant<uint64_t, 2>(d, steps, choices, stride, log, st);
+    else window_walk_variant<uint64_t, 3>(d, steps, choices, stride, log, st);
 }
 
 }  // namespace tfg

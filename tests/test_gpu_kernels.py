@@ -88,3 +88,31 @@ def test_stats_equal_the_records(nw):
     assert st["min_best_r"] == info["best_r"].min() and st["max_best_r"] == info["best_r"].max()
     assert np.array_equal(hist, np.bincount(info["best_r"], minlength=64)[:64])
     W.close()
+
+
+@pytest.mark.parametrize("fmt,slack,nw,horizon", [((2, 2, 2), 3, 33, 1), ((3, 3, 3), 5, 64, 8), ((1, 5, 5), 8, 70, 1),
+                                                  ((3, 4, 5), 4, 40, 16), ((3, 4, 5), 5, 65, 1), ((4, 4, 5), 8, 40, 2),
+                                                  ((4, 4, 4), 3, 25001, 1)])
+def test_uniform_window_steps_in_one_launch(fmt, slack, nw, horizon):
+    """Uniform window steps run together equal the same steps called one at a time (a
+    window kernel and an apply kernel each): state, choices and the log, at the edges
+    of the slot words and with the terms in shared and in device memory."""
+    steps = 24 if nw > 1000 else 150
+    p = tfg.tfg_default_params(plateau_len=60, r_slack=slack)
+    A, B = (tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=8, params=p) for _ in range(2))
+    logs = [tfg.TransitionLog(nw * steps, neg_thresh=int(0.05 * 2**32), horizon=horizon) for _ in range(2)]
+    ca = A.walk_window(steps, policy=0, record_choices=True, log=logs[0])
+    cb = [B.walk_window(1, policy=0, record_choices=True, log=logs[1]) for _ in range(steps)]
+    A.sync()
+    assert np.array_equal(ca.cpu().numpy(), np.concatenate([c.cpu().numpy() for c in cb]))
+    take = np.unique(np.linspace(0, nw - 1, 64).astype(int))
+    ia, ib = (W.read_walkers(0, nw, slots=False, best=False)[0] for W in (A, B))
+    assert np.array_equal(ia, ib)
+    for w in take:
+        for a, b in zip(A.read_walkers(int(w), 1)[1:], B.read_walkers(int(w), 1)[1:]):
+            assert np.array_equal(a, b), w
+    ea, eb = (np.sort(log.read(), order=["walker_id", "step", "label"]) for log in logs)
+    assert len(ea) > 0 and np.array_equal(ea, eb)
+    assert np.array_equal(A.window_buffers()[2].cpu().numpy(), B.window_buffers()[2].cpu().numpy())   # last step's sizes
+    A.close()
+    B.close()
