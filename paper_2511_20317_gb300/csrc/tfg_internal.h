@@ -71,7 +71,7 @@ struct ResizePlan {
     int32_t nblk;
     int32_t lt_src, mn_src, np_src;   // source row layout (u | v | w)
     int32_t lt_out, mn_out, np_out;   // result row layout
-    int32_t lt_aux, aux_rank;
+    int32_t lt_aux, mn_aux, np_aux, aux_rank;   // aux row layout
     int32_t canon;       // Z_T: restore the sign normalisation
     int32_t drop_zero;   // remove terms with a zero factor
     int32_t use_best;    // source: best scheme instead of the live one
@@ -80,7 +80,6 @@ struct ResizePlan {
 };
 bool build_resize_plan(int op, int axis, int index, const tfg_format &src, const tfg_format *aux, int aux_rank,
                        tfg_format &out, ResizePlan &plan, std::vector<int16_t> &maps);
-size_t resize_smem_bytes(const ResizePlan &plan);
 void launch_resize(const SegDesc &src, int64_t src_first, const SegDesc &dst, int64_t dst_first, int64_t count,
                    const ResizePlan &plan, unsigned long long *d_skipped, cudaStream_t st);
 
