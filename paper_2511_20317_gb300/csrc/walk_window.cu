@@ -17,6 +17,7 @@
 //      (computed from the state before the flip) with the label "the step
 //      lowered the rank" for training.
 #include <cstdint>
+#include <type_traits>
 #include <cuda_bf16.h>
 
 #include "mlp_pipe.cuh"
@@ -28,7 +29,6 @@ namespace dev {
 
 constexpr int kWin = 256;         // window capacity: up to 256 candidate pairs per step (two tensor-core tiles of rows)
 constexpr int kFeat = 32;
-constexpr int kWinMaxSlots = 128; // slots per walker supported by the window kernel
 
 // candidate descriptor: i (10 bits) | X (2) | j (10) | sign (1) | rho (1)
 __device__ __forceinline__ uint32_t pack_cand(int i, int X, int j, int sneg, int rho) {
@@ -97,126 +97,194 @@ __device__ __forceinline__ void cand_features_bf16(const PTerm<Wd, 1, true> &a, 
     for (int k = 0; k < kFeat / 2; ++k) h[k] = mlp::pack_bf16x2(f[2 * k], f[2 * k + 1]);
 }
 
-// One warp per walker.  Phase 1: eight terms i0 + g (g = lane / 4, then the
-// next eight while the window has room); the four lanes of a group scan
-// consecutive quarters of the slots for the term's try_flip candidates, and
-// every candidate's descriptor goes to its window position in shared memory
-// (order: term, then factor, then slot, then rho).  Phase 2: the lanes write
-// the window rows l, l+32, ... (descriptor and info words), and, when `feat`
-// is given, their feature rows (coalesced 64-byte rows; rows past the window
-// are zero).
+// One warp per walker; lane l holds slots l, l + 32, ... (NCH of them, r <= 32 NCH).
+// Matches of all terms at once: the slots' 16-bit factor hashes are transposed by
+// ballots into words over the slots, and a lane compares each of its slots' hash
+// with all slots by one word operation per bit, chunk and factor.  The hash classes
+// are the factor classes when every slot equals the lowest slot of its hash class
+// on the full words (one comparison per slot and factor); a walker with a collision
+// (about 3% at 64 slots) drops the false members one by one.  Then the counts' prefix
+// sums in slot order, rotated to start at term i0, give every term's first window
+// row, the lanes write their terms' rows to shared memory (the two rows of a match
+// in one 16-byte store), and the warp copies the rows out.  With `feat` it also
+// writes their feature rows (coalesced 64-byte rows; rows past the window are zero).
+// Bound by integer issue.  The kernel it replaces compared eight terms a round with all
+// slots, a quarter of the slots per lane, until the window was full, which in a
+// long walk takes every term (about 3.5 candidates each): (3,4,5) 262144 walkers
+// 1.77 ms, (4,4,4) 2.04 ms; now 0.56 and 0.6 ms.
+constexpr int kWinHash = 16;
 template <class Wd>
-__global__ void __launch_bounds__(128) window_kernel(const SegDesc d, __nv_bfloat16 *__restrict__ feat,
-                                                     uint2 *__restrict__ desc, int *__restrict__ kwin) {
-    __shared__ __align__(16) Wd sp[4][kWinMaxSlots], sn[4][kWinMaxSlots];
-    __shared__ uint32_t sdesc[4][kWin], sinfo[4][kWin];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t w = (int64_t)blockIdx.x * 4 + warp;
-    if (w >= d.n_walkers) return;
+struct alignas(2 * sizeof(Wd)) WinSlot {
+    Wd p, n;
+};
+template <class Wd, int NCH>
+__device__ __forceinline__ void window_of(const SegDesc &d, int64_t w, int lane, WinSlot<Wd> *st, uint2 *srow,
+                                          __nv_bfloat16 *feat, uint2 *desc, int *kwin) {
     using T = PTerm<Wd, 1, true>;
-    using O = Ops<Wd, 1, true>;
+    using LW = LinkWalker<TFG_MODE_ZT, Wd, NCH, false, false>;   // hash and comparison of factors
+    using Slot = WinSlot<Wd>;
+    constexpr unsigned full = 0xffffffffu;
     Masks<Wd, 1> mk;
     mk.load(d);
     const tfg_walker_info &H = d.hdr[w];
     const int r = H.r, best_r = H.best_r;
     const U4 x = philox10((uint32_t)H.t, (uint32_t)(H.t >> 32), H.walker_id, 0u, d.key0, d.key1);
     const int i0 = (int)__umulhi(x.x, (uint32_t)r);
-    const Wd *src = reinterpret_cast<const Wd *>(d.slots) + (size_t)w * d.R * 2;
-    for (int k = lane; k < r; k += 32) {
-        sp[warp][k] = src[(size_t)k * 2];
-        sn[warp][k] = src[(size_t)k * 2 + 1];
+    const Slot *src = reinterpret_cast<const Slot *>(d.slots) + (size_t)w * d.R;
+    T own[NCH];
+    uint32_t live[NCH];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int k = 32 * c + lane;
+        Slot v{Wd(0), Wd(0)};
+        if (k < r) v = src[k];
+        own[c].p[0] = v.p;
+        own[c].n[0] = v.n;
+        st[k] = v;
+        const int lo = r - 32 * c;
+        live[c] = lo >= 32 ? full : (lo > 0 ? (1u << lo) - 1u : 0u);
     }
     __syncwarp();
-    // ---- phase 1: candidate descriptors in window order
-    const int g = lane >> 2, sub = lane & 3;
-    const int chunk = (r + 3) >> 2;                  // <= 32 slots per lane
-    const int jb = sub * chunk, je = min(r, jb + chunk);
-    int carry = 0;
-    for (int base = 0; base < r && carry < kWin; base += 8) {
-        const int q = base + g;
-        const bool has = q < r;
-        const int i = has ? (i0 + q) % r : 0;
-        T ti;
-        ti.p[0] = sp[warp][i];
-        ti.n[0] = sn[warp][i];
-        // bit (j - jb): slot j of this lane's quarter is a candidate of factor u / v / w (w negated)
-        uint32_t bu = 0, bv = 0, bw = 0, bn = 0;
-        if (has) {
-            for (int j = jb; j < je; ++j) {
-                if (j == i) continue;
-                T c;
-                c.p[0] = sp[warp][j];
-                c.n[0] = sn[warp][j];
-                bool eu, ev, ewp, ewn;
-                O::compare(c, ti, mk, eu, ev, ewp, ewn);
-                const uint32_t bit = 1u << (j - jb);
-                bu |= eu ? bit : 0u;
-                bv |= ev ? bit : 0u;
-                bw |= (ewp || ewn) ? bit : 0u;
-                bn |= ewn ? bit : 0u;
-            }
-        }
-        // per-factor counts: this lane, earlier lanes of the group, the whole term
-        const uint32_t own = (uint32_t)__popc(bu) | ((uint32_t)__popc(bv) << 8) | ((uint32_t)__popc(bw) << 16);
-        uint32_t gin = own;
+    // ---- m[f][c][e]: members of chunk e in the class of factor f of slot 32 c + lane (without it)
+    uint32_t m[3][NCH][NCH];
+    bool exact = true;
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, gin, o, 4);
-            if (sub >= o) gin += y;
+    for (int f = 0; f < 3; ++f) {
+        uint32_t h[NCH];
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+            h[c] = LW::factor_hash16(own[c], mk.m[f][0]);
+#pragma unroll
+            for (int e = 0; e < NCH; ++e) m[f][c][e] = 0u;
         }
-        const uint32_t gtot = __shfl_sync(0xffffffffu, gin, 3, 4);
-        const uint32_t gex = gin - own;
-        const int nU = (int)(gtot & 255u), nV = (int)((gtot >> 8) & 255u), nW = (int)(gtot >> 16);
-        const int ki = 2 * (nU + nV + nW);
-        // window offset of the term: counts of the earlier terms of this round
-        int incl = sub == 0 ? ki : 0;
+        // one top bit of every byte a round (rolled: the code is read once per walker)
+#pragma unroll 1
+        for (int round = 0; round < kWinHash / 4; ++round) {
+            auto bit = [&](auto byte) {
+                constexpr int B = decltype(byte)::value;
+                uint32_t word[NCH];
+#pragma unroll
+                for (int e = 0; e < NCH; ++e) word[e] = __ballot_sync(full, (h[e] >> (8 * B + 7)) & 1u);
+#pragma unroll
+                for (int c = 0; c < NCH; ++c) {
+                    const uint32_t sp = sign_spread<B>(h[c]);
+#pragma unroll
+                    for (int e = 0; e < NCH; ++e) m[f][c][e] |= word[e] ^ sp;
+                }
+            };
+            bit(std::integral_constant<int, 0>{});
+            bit(std::integral_constant<int, 1>{});
+            bit(std::integral_constant<int, 2>{});
+            bit(std::integral_constant<int, 3>{});
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) h[c] <<= 1;
+        }
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+            int first = 0;   // lowest live slot of the hash class
+#pragma unroll
+            for (int e = NCH - 1; e >= 0; --e) {
+                m[f][c][e] = ~m[f][c][e] & live[e];
+                first = m[f][c][e] ? 32 * e + __ffs(m[f][c][e]) - 1 : first;
+            }
+            const Slot v = st[first];
+            T t;
+            t.p[0] = v.p;
+            t.n[0] = v.n;
+            exact = exact && (LW::same(t, own[c], mk.m[f][0]) || 32 * c + lane >= r);
+            m[f][c][c] &= ~(1u << lane);
+        }
+    }
+    if (!__all_sync(full, exact)) {
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int c = 0; c < NCH; ++c)
+#pragma unroll
+                for (int e = 0; e < NCH; ++e) {
+                    uint32_t left = m[f][c][e];
+#pragma unroll 1
+                    while (left) {
+                        const uint32_t low = left & (0u - left);
+                        left ^= low;
+                        const Slot v = st[32 * e + __ffs(low) - 1];
+                        T t;
+                        t.p[0] = v.p;
+                        t.n[0] = v.n;
+                        if (!LW::same(t, own[c], mk.m[f][0])) m[f][c][e] ^= low;
+                    }
+                }
+    }
+    // ---- window offsets: candidates (two per match) of the terms before, from i0 on
+    int ki[NCH], pre[NCH], total = 0;
+    uint32_t wneg[NCH];   // slots whose w starts with -1
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        int n = 0;
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int e = 0; e < NCH; ++e) n += __popc(m[f][c][e]);
+        ki[c] = 32 * c + lane < r ? 2 * n : 0;
+        int incl = ki[c];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            const int y = __shfl_up_sync(full, incl, o);
             if (lane >= o) incl += y;
         }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        const int tpos = carry + incl - ki;
-        const uint32_t info = (uint32_t)(ki < 64 ? ki : 64) | ((uint32_t)(q < 64 ? q : 64) << 8);
-        // this lane's candidates: factor X, slot order, rho 0 then 1
-        for (int X = 0; X < 3; ++X) {
-            const int before = X == 0 ? 0 : (X == 1 ? nU : nU + nV);
-            const int lex = (int)((gex >> (8 * X)) & 255u);
-            int pos = tpos + 2 * (before + lex);
-            uint32_t bits = X == 0 ? bu : (X == 1 ? bv : bw);
-            while (bits && pos < kWin) {
-                const int o = __ffs(bits) - 1;
-                bits &= bits - 1u;
-                const int j = jb + o;
-                const int sneg = (X == 2) ? (int)((bn >> o) & 1u) : 0;
-                sdesc[warp][pos] = pack_cand(i, X, j, sneg, 0);
-                sinfo[warp][pos] = info;
-                if (pos + 1 < kWin) {
-                    sdesc[warp][pos + 1] = pack_cand(i, X, j, sneg, 1);
-                    sinfo[warp][pos + 1] = info;
-                }
-                pos += 2;
-            }
-        }
-        carry += total;
+        pre[c] = total + incl - ki[c];
+        total += __shfl_sync(full, incl, 31);
+        const Wd dw = (own[c].p[0] | own[c].n[0]) & mk.m[2][0];
+        wneg[c] = __ballot_sync(full, (own[c].n[0] & dw & (Wd(0) - dw)) != Wd(0));
     }
-    const int K = carry < kWin ? carry : kWin;
+    int start = 0;   // candidates of the slots before i0
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int y = __shfl_sync(full, pre[c], i0 & 31);
+        start = (i0 >> 5) == c ? y : start;
+    }
+    const int K = total < kWin ? total : kWin;
+    // ---- rows: term, then factor, then slot, then rho
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int i = 32 * c + lane;
+        int pos = pre[c] - start + (i < i0 ? total : 0);
+        const int q = i >= i0 ? i - i0 : i - i0 + r;
+        const uint32_t info = (uint32_t)(ki[c] < 64 ? ki[c] : 64) | ((uint32_t)(q < 64 ? q : 64) << 8);
+        const uint32_t mine = (wneg[c] >> lane) & 1u;
+        if (i >= r) pos = kWin;
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int e = 0; e < NCH; ++e) {
+                uint32_t left = m[f][c][e];
+#pragma unroll 1
+                while (left && pos < kWin) {   // pos is even, and so is kWin
+                    const int o = __ffs(left) - 1;
+                    left &= left - 1u;
+                    const uint32_t sneg = f == 2 ? ((wneg[e] >> o) & 1u) ^ mine : 0u;
+                    const uint32_t dc = pack_cand(i, f, 32 * e + o, (int)sneg, 0);
+                    reinterpret_cast<uint4 *>(srow)[pos >> 1] = make_uint4(dc, info, dc | (1u << 23), info);
+                    pos += 2;
+                }
+            }
+    }
     __syncwarp();
-    // ---- phase 2: window rows (and feature rows when asked for)
-    uint2 *dw = desc + (size_t)w * kWin;
-    for (int row = lane; row < K; row += 32) dw[row] = make_uint2(sdesc[warp][row], sinfo[warp][row]);
+    uint4 *dw = reinterpret_cast<uint4 *>(desc + (size_t)w * kWin);
+    const uint4 *sw = reinterpret_cast<const uint4 *>(srow);
+    for (int row = lane; row < K / 2; row += 32) dw[row] = sw[row];
     if (feat) {
         __nv_bfloat16 *fw = feat + (size_t)w * kWin * kFeat;
         for (int row = lane; row < kWin; row += 32) {
             uint4 *dst = reinterpret_cast<uint4 *>(fw + (size_t)row * kFeat);
             if (row < K) {
-                const uint32_t dc = sdesc[warp][row], in = sinfo[warp][row];
-                const int i = (int)(dc & 1023u), j = (int)((dc >> 12) & 1023u);
+                const uint32_t dc = srow[row].x, in = srow[row].y;
+                const Slot vi = st[dc & 1023u], vj = st[(dc >> 12) & 1023u];
                 T ti, tj;
-                ti.p[0] = sp[warp][i];
-                ti.n[0] = sn[warp][i];
-                tj.p[0] = sp[warp][j];
-                tj.n[0] = sn[warp][j];
+                ti.p[0] = vi.p;
+                ti.n[0] = vi.n;
+                tj.p[0] = vj.p;
+                tj.n[0] = vj.n;
                 uint32_t h[kFeat / 2];
                 cand_features_bf16<Wd>(ti, tj, mk, dc, in, r, best_r, d.m, d.n, d.p, h);
 #pragma unroll
@@ -228,6 +296,21 @@ __global__ void __launch_bounds__(128) window_kernel(const SegDesc d, __nv_bfloa
         }
     }
     if (lane == 0) kwin[w] = K;
+}
+
+// NCH: chunks of the slot capacity; a walker runs at the chunks of its rank.
+template <class Wd, int NCH>
+__global__ void __launch_bounds__(128) window_kernel(const SegDesc d, __nv_bfloat16 *__restrict__ feat,
+                                                     uint2 *__restrict__ desc, int *__restrict__ kwin) {
+    __shared__ WinSlot<Wd> st[4][32 * NCH];
+    __shared__ __align__(16) uint2 srow[4][kWin];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t w = (int64_t)blockIdx.x * 4 + warp;
+    if (w >= d.n_walkers) return;
+    const int r = d.hdr[w].r;
+    if (NCH > 2 && r > 64) window_of<Wd, NCH>(d, w, lane, st[warp], srow[warp], feat, desc, kwin);
+    else if (NCH > 1 && r > 32) window_of<Wd, NCH < 2 ? 1 : 2>(d, w, lane, st[warp], srow[warp], feat, desc, kwin);
+    else window_of<Wd, 1>(d, w, lane, st[warp], srow[warp], feat, desc, kwin);
 }
 
 // Producer of the fused scoring kernel: tile t is half t & 1 (rows 0-127 or
@@ -471,6 +554,48 @@ __global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int
     wk.store(d, w, (uint32_t)steps);
 }
 
+// Row of highest score (first on ties) of every lane's walker that asks for one, by the
+// warp: a walker's scores in two 16-byte loads per lane.  (A thread reading its own
+// walker's 256 scores touches 32 lines a load: 0.34 ms for 262144 walkers with the
+// rest of the step, now 0.22.)  As a scan from row 0 that moves on a greater score
+// does, a NaN is never chosen over another row, and one in row 0 stays chosen.
+__device__ __forceinline__ int best_row(unsigned wmask, int lane, int nl, bool ask, int K, const float *mine) {
+    // order-preserving integers of scores (-0 as +0); 0: no score
+    auto key = [](float f) -> uint32_t {
+        const uint32_t u = __float_as_uint(f + 0.f);
+        return f != f ? 1u : (u & 0x80000000u ? ~u : u | 0x80000000u);
+    };
+    int c = 0;
+    unsigned pend = __ballot_sync(wmask, ask);
+#pragma unroll 1
+    while (pend) {
+        const int a = __ffs(pend) - 1;
+        pend &= pend - 1u;
+        const int Ka = __shfl_sync(wmask, K, a);
+        const float4 *row = reinterpret_cast<const float4 *>(
+            __shfl_sync(wmask, reinterpret_cast<unsigned long long>(mine), a));
+        uint32_t top = 0u;
+        int at = 0;
+#pragma unroll 2
+        for (int k0 = 4 * lane; k0 < Ka; k0 += 4 * nl) {   // nl: live lanes, 0 .. nl - 1
+            const float4 v = row[k0 >> 2];
+            const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t u = key(f[q]);
+                if (k0 + q == 0 && u == 1u) u = 0xffffffffu;
+                u = k0 + q < Ka ? u : 0u;
+                at = u > top ? k0 + q : at;
+                top = max(u, top);
+            }
+        }
+        const uint32_t most = __reduce_max_sync(wmask, top);
+        const int first = (int)__reduce_min_sync(wmask, top == most ? (unsigned)at : 0xffffu);
+        if (lane == a) c = first;
+    }
+    return c;
+}
+
 // One window-mode step per thread (walker), on the solo walker's state machine.
 template <class Wd, int RMAX, int BT>
 __global__ void __launch_bounds__(BT) window_apply_kernel(const SegDesc d, const uint2 *__restrict__ desc,
@@ -503,16 +628,10 @@ __global__ void __launch_bounds__(BT) window_apply_kernel(const SegDesc d, const
     T ti2, tj2;
     ti2.p[0] = tj2.p[0] = 0;
     ti2.n[0] = tj2.n[0] = 0;
+    const bool greedy = K > 0 && policy != 0 && x.w >= eps_thresh;
+    const int top = policy != 0 ? best_row(wmask, lane, nl, greedy, K, score + (size_t)w * kWin) : 0;
     if (K > 0) {
-        if (policy == 0 || x.w < eps_thresh) {
-            c = (int)__umulhi(x.y, (uint32_t)K);
-        } else {
-            const float *sc = score + (size_t)w * kWin;
-            c = 0;
-            float best = sc[0];
-            for (int k = 1; k < K; ++k)
-                if (sc[k] > best) { best = sc[k]; c = k; }
-        }
+        c = greedy ? top : (int)__umulhi(x.y, (uint32_t)K);
         const uint2 dci = desc[(size_t)w * kWin + c];
         const uint32_t dc = dci.x;
         i = (int)(dc & 1023u);
@@ -537,14 +656,13 @@ __global__ void __launch_bounds__(BT) window_apply_kernel(const SegDesc d, const
 int window_cap() { return dev::kWin; }
 
 void launch_window(const SegDesc &d, void *feat, uint2 *desc, int *kwin, cudaStream_t st) {
-    const int64_t blocks = (d.n_walkers + 3) / 4;
-    if (blocks <= 0) return;
-    if (d.word_bits == 32)
-        dev::window_kernel<uint32_t><<<(unsigned)blocks, 128, 0, st>>>(d, reinterpret_cast<__nv_bfloat16 *>(feat),
-                                                                      desc, kwin);
-    else
-        dev::window_kernel<uint64_t><<<(unsigned)blocks, 128, 0, st>>>(d, reinterpret_cast<__nv_bfloat16 *>(feat),
-                                                                      desc, kwin);
+    const unsigned blocks = (unsigned)((d.n_walkers + 3) / 4);
+    if (d.n_walkers <= 0) return;
+    auto *fb = reinterpret_cast<__nv_bfloat16 *>(feat);
+    if (d.word_bits == 32) dev::window_kernel<uint32_t, 1><<<blocks, 128, 0, st>>>(d, fb, desc, kwin);
+    else if (d.R <= 32) dev::window_kernel<uint64_t, 1><<<blocks, 128, 0, st>>>(d, fb, desc, kwin);
+    else if (d.R <= 64) dev::window_kernel<uint64_t, 2><<<blocks, 128, 0, st>>>(d, fb, desc, kwin);
+    else dev::window_kernel<uint64_t, 3><<<blocks, 128, 0, st>>>(d, fb, desc, kwin);
 }
 
 template <class Wd>

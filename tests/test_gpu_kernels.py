@@ -116,3 +116,52 @@ def test_uniform_window_steps_in_one_launch(fmt, slack, nw, horizon):
     assert np.array_equal(A.window_buffers()[2].cpu().numpy(), B.window_buffers()[2].cpu().numpy())   # last step's sizes
     A.close()
     B.close()
+
+
+@pytest.mark.parametrize("net", ["random", "zero", "nan"])
+@pytest.mark.parametrize("nw", [1, 33, 200])
+def test_greedy_choice_is_the_first_best_row(nw, net):
+    """The learned policy's choice: the first row of highest score among the window's K,
+    in full and partial warps; with a network of zeros every score ties; NaN scores
+    compare false, so row 0 stays chosen when every score is one."""
+    import torch
+    from paper_2511_20317_gb300 import learned
+    fmt = (3, 4, 5)
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=6, params=tfg.tfg_default_params(plateau_len=500))
+    W.walk(150)
+    params = learned.init_params(3)
+    if net != "random":
+        params.zero_()
+    if net == "nan":
+        params[-16:-12].view(torch.float32).fill_(float("nan"))   # b3
+    ch = W.walk_window(1, policy=1, mlp_params=params, record_choices=True).cpu().numpy()[0]
+    W.sync()
+    _, score, K = (b.cpu().numpy() for b in W.window_buffers())
+    for w in range(nw):
+        s = score[w, : K[w]]
+        want = 0 if np.isnan(s[0]) else int(np.nanargmax(s))
+        assert ch[w] == want, w
+    W.close()
+
+
+@pytest.mark.parametrize("fmt,slack,steps", [((2, 2, 2), 3, 50), ((3, 3, 3), 5, 0), ((1, 5, 5), 8, 60), ((3, 4, 5), 6, 400),
+                                             ((4, 4, 4), 3, 300), ((4, 4, 5), 8, 500)])
+def test_window_rows_equal_the_oracle(fmt, slack, steps):
+    """Window rows and sizes at 1, 2 and 3 chunks of slots, full and sparse windows, on
+    walked states, against the oracle's window."""
+    nw = 40
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=2, params=tfg.tfg_default_params(plateau_len=40, r_slack=slack))
+    W.walk(steps).sync()
+    info, slots, _ = W.read_walkers(0, nw)
+    _, rows, sizes = W.window_dump(features=False)
+    rows, sizes = rows.cpu().numpy(), sizes.cpu().numpy()
+    for w in range(nw):
+        r, t = int(info["r"][w]), int(info["t"][w])
+        i0 = (int(oracle.philox4x32_10([t, 0, w, 0], [2, 0])[0]) * r) >> 32
+        feat, cand = oracle.window_features(fmt, slots[w, :r], int(info["best_r"][w]), i0)
+        assert sizes[w] == len(cand), w
+        d, i = rows[w, : sizes[w], 0].view(np.uint32), rows[w, : sizes[w], 1]
+        got = np.stack([d & 1023, (d >> 10) & 3, (d >> 12) & 1023, np.where((d >> 22) & 1, -1, 1), (d >> 23) & 1], 1)
+        assert np.array_equal(got, cand), w
+        assert np.array_equal(i & 255, feat[:, 18]) and np.array_equal(i >> 8, feat[:, 24]), w
+    W.close()
