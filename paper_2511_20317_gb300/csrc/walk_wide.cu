@@ -7,81 +7,69 @@
 // bits per factor and sign), so every operation of Section 3.5.2 works word
 // by word and needs no mask.
 //
-// Mapping.  One warp per walker; lane l owns the slots k*32 + l (strided, so
-// that runs of related terms spread over the lanes).  The walker's terms live
-// in shared memory together with 32-bit signatures of each factor (hashes of
-// u, v and of w up to sign, plus the sign of w).  The candidate search of
-// try_flip (Algorithm 1) compares signatures only and verifies every
-// signature hit against the full factor words, so the candidate list is
-// exact; the chosen candidate is located in slot order by a walk over the
-// per-pass ballots.  The reduction checks (Section 3.4.1) are filtered the
-// same way.  All walker-uniform bookkeeping is replicated in every lane.
-// The arithmetic of a flip, a merge or a plus transition works on one word
-// per lane (lane q < 3*FW holds word q, of factor q / FW, of each term
-// involved): additions, normalisation, signatures and stores are a handful of
-// lane-parallel instructions and ballots; __syncwarp orders the shared-memory
-// writes.
+// Mapping.  Eight lanes per walker, four walkers a warp, with the factor classes of walk_link.cuh kept in shared memory: per factor the
+// slots of equal factors (w up to sign) form a cyclic list in ascending order, and
+// the slots' 8-bit factor hashes are held bit-sliced.  A step reads the sampled
+// term's three lists (a lane each); an accepted flip moves two slots to other
+// classes: the lanes share the hash words of the new factor's scan, check the
+// hits on the full words, and one lane per moved slot relinks it.  The arithmetic
+// of a flip, a merge or a plus transition works on one word per lane (lane q < 3*FW
+// holds word q, of factor q / FW, of each term involved): additions and
+// normalisation are a handful of lane-parallel instructions and ballots.  All
+// walker-uniform bookkeeping is replicated in the walker's lanes.  The four walkers
+// of a warp stay converged: what only some of them do is entered when any does
+// and predicated on their lanes (`on`), since shuffles and ballots on the lanes of one
+// walker alone split the warp into four that run one after another (32 us
+// a step of 32768 walkers at 351 terms, converged 27, and 18 with the scan, the
+// snapshots and the build as they are now).
 //
-// Terms of large walkers (capacity >= 256 slots) stay in their HBM slots and
-// only the signatures sit in shared memory (more walkers resident per SM).
+// Bound by the latency of a step, the reads of terms from L2 and memory first; 3.3 KB
+// of shared memory per walker at 354 slots let 68 walkers reside on an SM (17 warps).
+// The kernel it replaces searched all slots' 32-bit signatures with a warp per walker in
+// every step (1186 instructions a walker-step at 351 terms, now 280).  Measured, Z_T, 32768
+// walkers, 400 steps (classes built at each launch), before / now: (4,5,12) 10.7 / 5.4 ms,
+// (5,6,10) 10.7 / 6.3, (6,7,9) 12.7 / 8.2, (4,5,5) 7.8 / 3.7; (9,8,2) 16384 walkers 5.9 / 3.1.
 //
 // The step contract (draws, candidate order, flip, rejection, removal,
 // normalisation, reduction cascade, best/plateau bookkeeping, plus
 // transitions, trajectory digest) is the one of the lane-group and
 // thread-per-walker kernels.
 #include <cstdint>
+#include <type_traits>
 
 #include "tfg_internal.h"
 #include "pterm.cuh"
+#include "walk_link.cuh"
 
 namespace tfg {
 namespace dev {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// FW 64-bit words per factor and sign: word h of factor f is word f*FW + h.
-template <bool ZT, int FW>
-struct FTerm {
-    uint64_t p[3 * FW];
-    uint64_t n[3 * FW];   // kept zero in Z_2
-};
-
-// x[q] for a runtime q, by selects (no local-memory indexing)
-template <int N>
-__device__ __forceinline__ uint64_t pick(const uint64_t (&x)[N], int q) {
-    uint64_t v = x[0];
-#pragma unroll
-    for (int a = 1; a < N; ++a) v = (q == a) ? x[a] : v;
-    return v;
-}
-
-// 32-bit signature of word h of one factor (p, n): a multiply-xor hash, upper
-// half.  The signature of a factor is the XOR over its words.
-__device__ __forceinline__ uint32_t fsig(uint64_t p, uint64_t n, int h) {
-    const uint64_t k = h ? 0xC2B2AE3D27D4EB4Full : 0x9E3779B97F4A7C15ull;
-    const uint64_t x = (p ^ (n * 0xD6E8FEB86659FD93ull)) * k;
-    return (uint32_t)(x >> 32);
-}
-
-// GW: the term words stay in the walker's HBM slots (only the signatures are
-// in shared memory), else they are staged in shared memory for the launch.
 // PG: the walk policy is read from the descriptor (policies 1 and 2); without
 // it the plateau policy is compiled in alone.
 // FW: 64-bit words per factor (1: factors of at most 64 coefficients, 2: at most 128).
-template <int MODE, bool GW, bool PG, int FW>
+// GM: the terms stay in the walker's device-memory slots, else they are staged in shared
+// memory for the launch.
+template <int MODE, bool PG, int FW, bool GM>
 struct WideWalker {
+    static constexpr int G = 8;   // lanes per walker
     static_assert(FW == 1 || FW == 2, "one or two words per factor");
+    static_assert(G >= 3 * FW && G >= 5 && G < 32, "a lane per word of a term and per list of the reduction test");
     static constexpr bool ZT = (MODE == TFG_MODE_ZT);
     __device__ __forceinline__ static int policy_of(const SegDesc &d) { return PG ? d.walk_policy : 0; }
     static constexpr int TW = 3 * FW;                          // words per sign
-    static constexpr int NWG = ZT ? 2 * TW : TW;               // words per slot in HBM (p words [n words])
-    static constexpr int NWS = ZT ? 2 * TW : (TW + 1) / 2 * 2; // words per slot in shared memory (16-byte rows)
+    static constexpr int NWG = ZT ? 2 * TW : TW;               // words per slot (p words [n words])
     static constexpr unsigned FM = (1u << FW) - 1u;            // a factor's lanes / words in a ballot
-    using T = FTerm<ZT, FW>;
+    static_assert(G >= kHashBits, "a lane per hash slice");
+    static constexpr int NL = 32 / G;                          // hash words per lane at 1023 slots
+    static constexpr int kNone = 1 << 20;
 
-    uint64_t *W;    // GW: HBM slots [R][NWG]; else shared [R][NWS]: Z_T (p_q n_q) pairs, Z_2 p words (padded)
-    uint4 *SG;      // [32 * KM] signatures (u, v, w up to sign, sign of w)
-    int lane, KM;
+    uint64_t *W;      // this walker's slots [R][NWG], in device (GM) or shared memory
+    uint16_t *nx;     // next of (k, f) = nx[f * R + k]
+    uint32_t *hs;     // hash slices: bit b of factor f, slots 32 q .. 32 q + 31 = hs[(f * 8 + b) * KW + q]
+    int lane, gb;     // lane within the walker's G lanes; the first of them
+    int KW;           // hash words: ceil(R / 32)
     int r, best_r, R;
     int64_t t, plateau, best_t;
     uint64_t dig;
@@ -90,78 +78,43 @@ struct WideWalker {
     int qlen, q0, q1, q2;
     uint32_t nnz, best_nnz;   // non-zero coefficients of the live (walk policy 2) / best scheme
 
-    // shared-memory word of HBM slot word g
-    __device__ __forceinline__ static int smem_word(int g) { return ZT ? (g < TW ? 2 * g : 2 * (g - TW) + 1) : g; }
+    __host__ __device__ static constexpr size_t walker_bytes(int R) {
+        return term_bytes(R) + (((size_t)R * 6 + 15) & ~(size_t)15) + (size_t)3 * kHashBits * ((R + 31) / 32) * 4;
+    }
+    __host__ __device__ static constexpr size_t term_bytes(int R) {   // in shared memory
+        return GM ? (size_t)0 : ((size_t)R * NWG * 8 + 15) & ~(size_t)15;
+    }
+    // slots: the walker's device-memory slots
+    __device__ __forceinline__ void attach(unsigned char *at, uint64_t *slots) {
+        W = GM ? slots : reinterpret_cast<uint64_t *>(at);
+        at += term_bytes(R);
+        nx = reinterpret_cast<uint16_t *>(at);
+        hs = reinterpret_cast<uint32_t *>(at + (((size_t)R * 6 + 15) & ~(size_t)15));
+    }
 
-    // ---- full-term comparisons (hit verification)
-    __device__ __forceinline__ static bool eq(const T &a, const T &b, int f) {
-        bool e = true;
-#pragma unroll
-        for (int h = 0; h < FW; ++h) e = e && a.p[f * FW + h] == b.p[f * FW + h] && (!ZT || a.n[f * FW + h] == b.n[f * FW + h]);
-        return e;
+    // ---- group communication
+    __device__ __forceinline__ unsigned vote(bool p) const {
+        return (__ballot_sync(kFull, p) >> gb) & ((1u << G) - 1u);
     }
-    __device__ __forceinline__ static bool eqneg(const T &a, const T &b, int f) {
-        bool e = ZT;
+    template <class V>
+    __device__ __forceinline__ V from(V v, int l) const { return __shfl_sync(kFull, v, gb + l); }
+    __device__ __forceinline__ static bool any(bool p) { return __any_sync(kFull, p); }
+
+    __device__ __forceinline__ static uint32_t sum(uint32_t v) {   // over the walker's lanes
 #pragma unroll
-        for (int h = 0; h < FW; ++h) e = e && a.p[f * FW + h] == b.n[f * FW + h] && a.n[f * FW + h] == b.p[f * FW + h];
-        return e;
-    }
-    __device__ __forceinline__ static bool sum_ok(const T &a, const T &b, int f, bool neg) {
-        if constexpr (ZT) {
-            uint64_t clash = 0ull;
-#pragma unroll
-            for (int h = 0; h < FW; ++h) {
-                const int q = f * FW + h;
-                const uint64_t bp = neg ? b.n[q] : b.p[q], bn = neg ? b.p[q] : b.n[q];
-                clash |= (a.p[q] & bp) | (a.n[q] & bn);
-            }
-            return clash == 0ull;
-        } else {
-            return true;
-        }
-    }
-    // the first non-zero coefficient of factor f is negative
-    __device__ __forceinline__ static bool lead_neg(const T &a, int f) {
-        bool ng = false;
-#pragma unroll
-        for (int h = FW - 1; h >= 0; --h) {
-            const uint64_t d = a.p[f * FW + h] | a.n[f * FW + h];
-            ng = d ? ((a.n[f * FW + h] & d & (0ull - d)) != 0ull) : ng;
-        }
-        return ng;
-    }
-    __device__ __forceinline__ static uint4 sig(const T &a) {
-        uint4 s = make_uint4(0u, 0u, 0u, 0u);
-        const bool ng = ZT && lead_neg(a, 2);
-#pragma unroll
-        for (int h = 0; h < FW; ++h) {
-            s.x ^= fsig(a.p[h], a.n[h], h);
-            s.y ^= fsig(a.p[FW + h], a.n[FW + h], h);
-            const uint64_t wp = a.p[2 * FW + h], wn = a.n[2 * FW + h];
-            s.z ^= fsig(ng ? wn : wp, ng ? wp : wn, h);
-        }
-        s.w = ng ? 1u : 0u;
-        return s;
+        for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+        return v;
     }
 
     // ---- one word per lane: lane q < 3*FW holds word q (factor q / FW) of each
-    // term involved; lanes 3*FW..31 mirror word 0 and never store
+    // term involved; the other lanes mirror word 0 and never store
     struct DF { uint64_t p, n; };
-    int fq;   // this lane's word (0 on lanes 3*FW..31)
+    int fq;   // this lane's word (0 on lanes past the words)
     __device__ __forceinline__ bool owns(int f) const { return (lane >> (FW - 1)) == f; }   // holds a word of factor f
-    __device__ __forceinline__ int fh() const { return FW == 1 ? 0 : lane & 1; }         // its word within the factor
     __device__ __forceinline__ bool fown() const { return lane < 3 * FW; }
 
-    __device__ __forceinline__ DF dof(const T &a) const { return DF{pick(a.p, fq), pick(a.n, fq)}; }
     __device__ __forceinline__ DF dget(int s) const {
-        if constexpr (GW) {
-            return DF{W[(size_t)s * NWG + fq], ZT ? W[(size_t)s * NWG + TW + fq] : 0ull};
-        } else if constexpr (ZT) {
-            const ulonglong2 a = reinterpret_cast<const ulonglong2 *>(W + (size_t)s * NWS)[fq];
-            return DF{a.x, a.y};
-        } else {
-            return DF{W[(size_t)s * NWS + fq], 0ull};
-        }
+        return DF{W[(size_t)s * NWG + fq], ZT ? W[(size_t)s * NWG + TW + fq] : 0ull};
     }
     // res = a with factor f := a_f + b_f (neg: a_f - b_f); false when a
     // coefficient leaves the coefficient set (Section 3.5.2)
@@ -177,10 +130,10 @@ struct WideWalker {
             res.p = me ? (a.p ^ b.p) : a.p;
             res.n = 0ull;
         }
-        return !__any_sync(kFull, bad);
+        return vote(bad) == 0u;
     }
     __device__ __forceinline__ bool dzero(const DF &a, int f) const {
-        return ((__ballot_sync(kFull, (a.p | a.n) == 0ull) >> (f * FW)) & FM) == FM;
+        return ((vote((a.p | a.n) == 0ull) >> (f * FW)) & FM) == FM;
     }
     __device__ __forceinline__ void dtake(DF &dst, const DF &src, int f) const {
         if (owns(f)) dst = src;
@@ -189,12 +142,12 @@ struct WideWalker {
     // returned ballot) is set when factor f's first non-zero coefficient is negative.
     __device__ __forceinline__ unsigned dlead(const DF &a) const {
         const uint64_t d = a.p | a.n;
-        const unsigned ng = __ballot_sync(kFull, (a.n & d & (0ull - d)) != 0ull);
+        const unsigned ng = vote((a.n & d & (0ull - d)) != 0ull);
         if constexpr (FW == 1) {
             return ng;
         } else {
             // a factor's second word decides only when its first word is zero
-            const unsigned nz = __ballot_sync(kFull, d != 0ull);
+            const unsigned nz = vote(d != 0ull);
             return (ng & nz & 0x15u) | ((ng >> 1) & ~nz & 0x15u);
         }
     }
@@ -211,120 +164,173 @@ struct WideWalker {
     // non-zero coefficients of a term held one word per lane
     __device__ __forceinline__ uint32_t dnnz(const DF &a) const {
         const uint32_t c = fown() ? (uint32_t)__popcll(a.p | a.n) : 0u;
-        return __reduce_add_sync(kFull, c);
+        return sum(c);
     }
     // w of a equals -w of b
     __device__ __forceinline__ bool dwneg(const DF &a, const DF &b) const {
-        return ZT && ((__ballot_sync(kFull, a.p == b.n && a.n == b.p) >> (2 * FW)) & FM) == FM;
+        return ZT && ((vote(a.p == b.n && a.n == b.p) >> (2 * FW)) & FM) == FM;
     }
-    __device__ __forceinline__ void dput(int s, const DF &a) {
-        uint64_t cp = a.p, cn = a.n;
-        uint32_t ng = 0u;
-        if constexpr (ZT) {
-            if constexpr (FW == 1) {
-                const uint64_t d = a.p | a.n;
-                ng = (lane == 2 && (a.n & d & (0ull - d)) != 0ull) ? 1u : 0u;   // read by lane 2 alone
-            } else {
-                ng = (dlead(a) >> (2 * FW)) & 1u;
-            }
-            if (ng && owns(2)) { cp = a.n; cn = a.p; }
-        }
-        uint32_t h = fsig(cp, cn, fh());
-        if constexpr (FW == 2) h ^= __shfl_xor_sync(kFull, h, 1);   // the factor's two words
-        if (fown()) {
-            if constexpr (GW) {
-                W[(size_t)s * NWG + lane] = a.p;
-                if constexpr (ZT) W[(size_t)s * NWG + TW + lane] = a.n;
-            } else if constexpr (ZT) {
-                reinterpret_cast<ulonglong2 *>(W + (size_t)s * NWS)[lane] = make_ulonglong2(a.p, a.n);
-            } else {
-                W[(size_t)s * NWS + lane] = a.p;
-            }
-            if (fh() == 0) {
-                uint32_t *g = reinterpret_cast<uint32_t *>(SG + s);
-                g[lane >> (FW - 1)] = h;
-                if (owns(2)) g[3] = ng;
-            }
+    __device__ __forceinline__ void dput(bool on, int s, const DF &a) {
+        if (on && fown()) {
+            W[(size_t)s * NWG + lane] = a.p;
+            if constexpr (ZT) W[(size_t)s * NWG + TW + lane] = a.n;
         }
         __syncwarp();
     }
 
-    // ---- term slots
-    __device__ __forceinline__ static void set_word(T &out, int g, uint64_t v) {
-        if (g < TW) out.p[g] = v;
-        else out.n[g - TW] = v;
+    // ---- factor classes
+    __device__ __forceinline__ uint16_t &next(int k, int f) const { return nx[f * R + k]; }
+    // symmetric in the two signs: w's class is up to sign
+    __device__ __forceinline__ static uint32_t fold(uint64_t x) {
+        const uint64_t a = (uint64_t)(uint32_t)x * 0x9E3779B1u + (uint64_t)(uint32_t)(x >> 32) * 0x85EBCA77u;
+        return (uint32_t)a ^ (uint32_t)(a >> 32);
     }
-    __device__ __forceinline__ T get(int s) const {
-        T out;
-        if constexpr (!ZT) {
-#pragma unroll
-            for (int q = 0; q < TW; ++q) out.n[q] = 0ull;
-        }
-        if constexpr (GW) {
-            const uint64_t *g = W + (size_t)s * NWG;
-            if constexpr (NWG % 2 == 0) {
-                const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(g);   // rows of 16-byte multiples
-#pragma unroll
-                for (int e = 0; e < NWG / 2; ++e) {
-                    const ulonglong2 a = q[e];
-                    set_word(out, 2 * e, a.x);
-                    set_word(out, 2 * e + 1, a.y);
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < NWG; ++e) set_word(out, e, g[e]);
-            }
-            return out;
-        }
-        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(W + (size_t)s * NWS);
-#pragma unroll
-        for (int e = 0; e < NWS / 2; ++e) {
-            const ulonglong2 a = src[e];
-            if constexpr (ZT) {
-                out.p[e] = a.x; out.n[e] = a.y;
-            } else {
-                out.p[2 * e] = a.x;
-                if (2 * e + 1 < TW) out.p[2 * e + 1] = a.y;
-            }
-        }
-        return out;
+    __device__ __forceinline__ static uint32_t word_hash(uint64_t p, uint64_t n, int h) {
+        const uint32_t x = fold(p) + (ZT ? fold(n) : 0u);
+        return h ? x * 0xC2B2AE35u : x;
     }
-    // factor f of slot s equals factor f of a (wneg: or its negation)
-    __device__ __forceinline__ bool fmatch(int s, int f, const T &a, bool wneg) const {
-        bool ep = true, en = ZT && wneg;
+    // hash of factor f of a term held one word per lane
+    __device__ __forceinline__ uint32_t dhash(const DF &a, int f) const {
+        const uint32_t x = word_hash(a.p, a.n, FW == 1 ? 0 : lane & 1);
+        uint32_t h = from(x, f * FW);
+        if constexpr (FW == 2) h += from(x, f * FW + 1);
+        return h;
+    }
+    // live slots of hash word q
+    __device__ __forceinline__ static uint32_t live_word(int r, int q) {
+        const int lo = r - 32 * q;
+        return lo >= 32 ? ~0u : (lo > 0 ? (1u << lo) - 1u : 0u);
+    }
+    __device__ __forceinline__ static void spreads(uint32_t h, uint32_t (&sp)[kHashBits]) {
+        sp[0] = sign_spread<0>(h); sp[1] = sign_spread<1>(h); sp[2] = sign_spread<2>(h); sp[3] = sign_spread<3>(h);
+        const uint32_t h1 = h << 1;
+        sp[4] = sign_spread<0>(h1); sp[5] = sign_spread<1>(h1); sp[6] = sign_spread<2>(h1); sp[7] = sign_spread<3>(h1);
+    }
+    // This lane's share (words lane, lane + G, ...) of the slots that may hold the factor f
+    // of hash h, slot s aside; s's own slices := the hash.
+    __device__ __forceinline__ void scan(bool on, int s, int f, uint32_t h, uint32_t (&c)[NL]) const {
+        uint32_t sp[kHashBits];
+        spreads(h, sp);
+        const uint32_t sb = 1u << (s & 31);
+        uint32_t *base = hs + f * kHashBits * KW;
+#pragma unroll
+        for (int a = 0; a < NL; ++a) c[a] = 0u;
+#pragma unroll
+        for (int a = 0; a < NL; ++a) {
+            if (a * G >= KW) break;   // the same for all lanes
+            const int q = a * G + lane;
+            if (on && q < KW) {
+                uint32_t dd = 0u;
+#pragma unroll
+                for (int b = 0; b < kHashBits; ++b) dd |= base[b * KW + q] ^ sp[b];
+                c[a] = ~dd & live_word(r, q) & (q == (s >> 5) ? ~sb : ~0u);
+            }
+        }
+        __syncwarp();
+        // a lane per slice
+        if (on && lane < kHashBits) {
+            uint32_t mine = sp[0];
+#pragma unroll
+            for (int b = 1; b < kHashBits; ++b) mine = lane == b ? sp[b] : mine;
+            uint32_t &w = base[lane * KW + (s >> 5)];
+            w = (w & ~sb) | (mine & sb);
+        }
+    }
+    // this lane's lowest slot of c, removed from it (-1: none)
+    __device__ __forceinline__ int take(uint32_t (&c)[NL]) const {
+        int k = -1;
+#pragma unroll
+        for (int a = 0; a < NL; ++a) {
+            const bool here = k < 0 && c[a] != 0u;
+            k = here ? 32 * (a * G + lane) + __ffs(c[a]) - 1 : k;
+            c[a] = here ? c[a] & (c[a] - 1u) : c[a];
+        }
+        return k;
+    }
+    // factor f of slot s of the slots w equals (vp, vn) up to sign
+    __device__ __forceinline__ static bool fsame(const uint64_t *w, int s, int f, const uint64_t (&vp)[FW],
+                                                 const uint64_t (&vn)[FW]) {
+        bool ep = true, en = ZT;
 #pragma unroll
         for (int h = 0; h < FW; ++h) {
-            const int q = f * FW + h;
-            uint64_t p, n;
-            if constexpr (GW) {
-                p = W[(size_t)s * NWG + q];
-                n = ZT ? W[(size_t)s * NWG + TW + q] : 0ull;
-            } else if constexpr (ZT) {
-                const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(W + (size_t)s * NWS)[q];
-                p = x.x; n = x.y;
-            } else {
-                p = W[(size_t)s * NWS + q];
-                n = 0ull;
-            }
-            ep = ep && p == a.p[q] && n == a.n[q];
-            en = en && p == a.n[q] && n == a.p[q];
+            const uint64_t p = w[(size_t)s * NWG + f * FW + h], n = ZT ? w[(size_t)s * NWG + TW + f * FW + h] : 0ull;
+            ep = ep && p == vp[h] && n == vn[h];
+            en = en && p == vn[h] && n == vp[h];
         }
         return ep || en;
     }
-    __device__ __forceinline__ void move(int from, int to) {
-        if constexpr (GW) {
-            if (lane < NWG) W[(size_t)to * NWG + lane] = W[(size_t)from * NWG + lane];
-            else if (lane == NWG) SG[to] = SG[from];
-            __syncwarp();
-            return;
+    // slot s out of its class of factor f, then into the class of slot `hit` (-1: a class of
+    // its own); by one lane
+    __device__ __forceinline__ void move_class(int s, int f, int hit) const {
+        const int o = next(s, f);
+        int p = s, q = o;
+#pragma unroll 1
+        for (int n = 0; n < R && q != s; ++n) {   // a class has at most R members
+            p = q;
+            q = next(q, f);
         }
-        if (lane < NWS / 2) {
-            const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(W + (size_t)from * NWS);
-            ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(W + (size_t)to * NWS);
-            dst[lane] = src[lane];
-        } else if (lane == NWS / 2) {
-            SG[to] = SG[from];
+        next(p, f) = (uint16_t)o;
+        p = hit >= 0 ? hit : s;
+        q = hit >= 0 ? (int)next(hit, f) : s;
+#pragma unroll 1
+        for (int n = 0; n < R && !(p < q ? (p < s && s < q) : (s >= p || s <= q)); ++n) {
+            p = q;
+            q = next(q, f);
         }
+        next(p, f) = (uint16_t)s;
+        next(s, f) = (uint16_t)q;
+    }
+    // One or (TWO) two slots change their class: slot sa's factor fa is now va's, slot sb's
+    // factor fb (fb != fa) now vb's (both stored already).
+    template <bool TWO>
+    __device__ __forceinline__ void relink(bool on, int sa, int fa, const DF &va, int sb, int fb, const DF &vb) const {
+        uint32_t ca[NL], cb[NL];
+        scan(on, sa, fa, dhash(va, fa), ca);
+        if constexpr (TWO) {
+            scan(on, sb, fb, dhash(vb, fb), cb);
+        } else {
+#pragma unroll
+            for (int a = 0; a < NL; ++a) cb[a] = 0u;
+        }
+        uint64_t ap[FW], an[FW], bp[FW], bn[FW];
+#pragma unroll
+        for (int h = 0; h < FW; ++h) {
+            ap[h] = from(va.p, fa * FW + h);
+            an[h] = ZT ? from(va.n, fa * FW + h) : 0ull;
+            bp[h] = TWO ? from(vb.p, fb * FW + h) : 0ull;
+            bn[h] = TWO && ZT ? from(vb.n, fb * FW + h) : 0ull;
+        }
+        int ha = -1, hb = -1;   // a slot of the new class
+#pragma unroll 1
+        for (int n = 0; n <= R; ++n) {
+            const int ka = ha < 0 ? take(ca) : -1, kb = TWO && hb < 0 ? take(cb) : -1;
+            if (!any(ka >= 0 || kb >= 0)) break;
+            const bool oa = ka >= 0 && fsame(W, ka, fa, ap, an);
+            const bool ob = TWO && kb >= 0 && fsame(W, kb, fb, bp, bn);
+            const unsigned ma = vote(oa);
+            const int fa2 = from(ka, ma ? __ffs(ma) - 1 : 0);
+            ha = ma ? fa2 : ha;
+            if constexpr (TWO) {
+                const unsigned mb = vote(ob);
+                const int fb2 = from(kb, mb ? __ffs(mb) - 1 : 0);
+                hb = mb ? fb2 : hb;
+            }
+        }
+        if constexpr (TWO) {
+            if (on && lane < 2) move_class(lane ? sb : sa, lane ? fb : fa, lane ? hb : ha);
+        } else {
+            if (on && lane == 0) move_class(sa, fa, ha);
+        }
+        __syncwarp();
+    }
+    // slot s := term v, every class anew
+    __device__ __forceinline__ void put(bool on, int s, const DF &v) {
+        dput(on, s, v);
+#pragma unroll 1
+        for (int f = 0; f < 3; ++f) relink<false>(on, s, f, v, s, f, v);
+    }
+    __device__ __forceinline__ void unlink(bool on, int s) const {
+        if (on && lane < 3) move_class(s, lane, -1);
         __syncwarp();
     }
 
@@ -348,400 +354,454 @@ struct WideWalker {
         q0 = n0; q1 = n1;
         qlen = (int)k0 + (int)k1 + (int)k2;
     }
-    __device__ __forceinline__ void q_rename(int from, int to) {
-        q0 = (qlen > 0 && q0 == from) ? to : q0;
-        q1 = (qlen > 1 && q1 == from) ? to : q1;
-        q2 = (qlen > 2 && q2 == from) ? to : q2;
+    __device__ __forceinline__ void q_rename(int from_, int to) {
+        q0 = (qlen > 0 && q0 == from_) ? to : q0;
+        q1 = (qlen > 1 && q1 == from_) ? to : q1;
+        q2 = (qlen > 2 && q2 == from_) ? to : q2;
     }
 
     // Remove slot h: the last live term moves into the hole.
-    __device__ __forceinline__ void drop(int h) {
+    __device__ __forceinline__ void drop(bool on, int h) {
         const int last = r - 1;
-        q_remove(h);
-        if (h != last) {
-            move(last, h);
-            q_rename(last, h);
+        const bool mv = on && h != last;
+        if (on) q_remove(h);
+        unlink(on, h);
+        unlink(mv, last);
+        if (on) r -= 1;
+        if (any(mv)) {
+            put(mv, mv ? h : 0, dget(mv ? last : 0));
+            if (mv) q_rename(last, h);
         }
-        r -= 1;
     }
 
-    // Does any other live slot share two factors (signatures) with the terms
-    // in slots sa or sb?  A superset of the reduction test: the cascade that
-    // follows a positive answer checks exactly.
-    __device__ __forceinline__ bool pair_filter(int sa, int sb) const {
-        const uint4 A = SG[sa], B = SG[sb];
-        bool hit = false;
-#pragma unroll 4
-        for (int k = 0; k < KM; ++k) {
-            const int s = (k << 5) + lane;
-            const uint4 g = SG[s];
-            const int ma = (int)(g.x == A.x) + (int)(g.y == A.y) + (int)(g.z == A.z);
-            const int mb = (int)(g.x == B.x) + (int)(g.y == B.y) + (int)(g.z == B.z);
-            hit |= s < r && ((s != sa && ma >= 2) || (s != sb && mb >= 2));
-        }
-        return __any_sync(kFull, hit);
+    // Slot k against the term v (held one word per lane): which factors are equal, negated,
+    // and where the sum / difference leaves the coefficient set (bit f).
+    struct Against { unsigned eq, ne, cp, cn; };
+    __device__ __forceinline__ static unsigned by_factor_all(unsigned b) {
+        if constexpr (FW == 1) return b & 7u;
+        else return ((b & (b >> 1)) & 1u) | (((b & (b >> 1)) >> 1) & 2u) | (((b & (b >> 1)) >> 2) & 4u);
+    }
+    __device__ __forceinline__ static unsigned by_factor_any(unsigned b) {
+        if constexpr (FW == 1) return b & 7u;
+        else return ((b | (b >> 1)) & 1u) | (((b | (b >> 1)) >> 1) & 2u) | (((b | (b >> 1)) >> 2) & 4u);
+    }
+    __device__ __forceinline__ Against against(int k, const DF &v) const {
+        const DF c = dget(k);
+        Against a;
+        a.eq = by_factor_all(vote(c.p == v.p && c.n == v.n));
+        a.ne = ZT ? by_factor_all(vote(c.p == v.n && c.n == v.p)) : 0u;
+        a.cp = ZT ? by_factor_any(vote(((v.p & c.p) | (v.n & c.n)) != 0ull)) : 0u;
+        a.cn = ZT ? by_factor_any(vote(((v.p & c.n) | (v.n & c.p)) != 0ull)) : 0u;
+        return a;
     }
 
     // Reduction of the term in slot s with the lowest slot sharing (u,v), else
-    // (u,w), else (v,w), whose merged third factor stays ternary; the merged
-    // term keeps s's pair factors and goes to the lower slot.
-    __device__ __forceinline__ void reduce_one(int s) {
-        const T v = get(s);
-        const uint4 vs = SG[s];
-        uint32_t c0 = 0, c1 = 0, c2 = 0;   // bit k: slot k*32 + lane shares the pair by signature
-#pragma unroll 4
-        for (int k = 0; k < KM; ++k) {
-            const int slot = (k << 5) + lane;
-            const uint4 g = SG[slot];
-            const bool live = slot < r && slot != s;
-            const bool eu = g.x == vs.x, ev = g.y == vs.y, ew = g.z == vs.z;
-            c0 |= (uint32_t)(live && eu && ev) << k;
-            c1 |= (uint32_t)(live && eu && ew) << k;
-            c2 |= (uint32_t)(live && ev && ew) << k;
-        }
-        uint32_t m0 = 0, m1 = 0, m2 = 0;   // verified, with a ternary merged third factor
-        uint32_t any = c0 | c1 | c2;
+    // (u,w), else (v,w), whose merged third factor stays in the coefficient set; the
+    // merged term keeps s's pair factors and goes to the lower slot.
+    __device__ __forceinline__ void reduce_one(bool on, int s) {   // s valid in every lane
+        const DF dv = dget(s);
+        int k0 = kNone, k1 = kNone, k2 = kNone;
+        bool n1 = false, n2 = false;
+        int k = next(s, 0);
+        bool act = on && k != s;
 #pragma unroll 1
-        while (any) {
-            const int k = __ffs(any) - 1;
-            any &= any - 1u;
-            const uint32_t bit = 1u << k;
-            const T u = get((k << 5) + lane);
-            const bool xu = eq(u, v, 0), xv = eq(u, v, 1), xwp = eq(u, v, 2), xwn = eqneg(u, v, 2);
-            if ((c0 & bit) && xu && xv && sum_ok(v, u, 2, false)) m0 |= bit;
-            if ((c1 & bit) && xu && (xwp || xwn) && sum_ok(v, u, 1, xwn)) m1 |= bit;
-            if ((c2 & bit) && xv && (xwp || xwn) && sum_ok(v, u, 0, xwn)) m2 |= bit;
+        for (int n = 0; n < R && any(act); ++n) {
+            const Against a = against(k, dv);
+            const bool ev = a.eq & 2u, ewp = a.eq & 4u, ewn = !ewp && (a.ne & 4u);
+            if (act && ev && k < k0 && !(a.cp & 4u)) k0 = k;
+            if (act && (ewp || ewn) && k < k1 && !((ewn ? a.cn : a.cp) & 2u)) { k1 = k; n1 = ewn; }
+            k = act ? (int)next(k, 0) : k;
+            act = act && k != s;
         }
-        const unsigned b0 = __ballot_sync(kFull, m0 != 0u), b1 = __ballot_sync(kFull, m1 != 0u),
-                       b2 = __ballot_sync(kFull, m2 != 0u);
-        if ((b0 | b1 | b2) == 0u) return;
-        const int P = b0 ? 0 : (b1 ? 1 : 2);
-        const uint32_t mp = P == 0 ? m0 : (P == 1 ? m1 : m2);
-        // lowest slot (k*32 + lane) with a partner of pair type P
-        const unsigned mine = mp ? (unsigned)(((__ffs(mp) - 1) << 5) + lane) : 0xffffffffu;
-        const int k = (int)__reduce_min_sync(kFull, mine);
-        const DF dv = dof(v), dk = dget(k);
-        const bool kneg = (P != 0) && dwneg(dk, dv);
+        k = next(s, 1);
+        act = on && k0 == kNone && k1 == kNone && k != s;
+#pragma unroll 1
+        for (int n = 0; n < R && any(act); ++n) {
+            const Against a = against(k, dv);
+            const bool ewp = a.eq & 4u, ewn = !ewp && (a.ne & 4u);
+            if (act && (ewp || ewn) && k < k2 && !((ewn ? a.cn : a.cp) & 1u)) { k2 = k; n2 = ewn; }
+            k = act ? (int)next(k, 1) : k;
+            act = act && k != s;
+        }
+        const bool has = k0 != kNone || k1 != kNone || k2 != kNone;
+        if (!any(has)) return;
+        const int P = k0 != kNone ? 0 : (k1 != kNone ? 1 : 2);
+        k = !has ? s : (P == 0 ? k0 : (P == 1 ? k1 : k2));
+        const bool kneg = P == 1 ? n1 : (P == 2 ? n2 : false);
         const int F = 2 - P;   // third factor: w, v, u
         DF mv;
-        dadd(dv, dk, F, kneg, mv);
+        dadd(dv, dget(k), F, kneg, mv);
         const bool z = dzero(mv, F);
         dcanon(mv);
         const int lo = s < k ? s : k;
         const int hi = s < k ? k : s;
-        q_remove(k);
-        dput(lo, mv);
-        c_mrg += 1;
-        drop(hi);
-        if (z) {
-            drop(lo);
-            c_drp += 1;
-        } else {
-            q_push(lo);
-        }
+        if (has) q_remove(k);
+        dput(has, lo, mv);
+        relink<false>(has, lo, F, mv, lo, F, mv);   // s and k share the other two factors
+        c_mrg += has;
+        drop(has, hi);
+        if (any(has && z)) drop(has && z, lo);
+        c_drp += has && z;
+        if (has && !z) q_push(lo);
     }
 
     __device__ __forceinline__ void cascade() {
 #pragma unroll 1
-        while (qlen > 0) reduce_one(q_pop());
+        while (any(qlen > 0)) {
+            const bool on = qlen > 0;
+            int s = 0;
+            if (on) s = q_pop();
+            reduce_one(on, s);
+        }
     }
 
-    __device__ __forceinline__ void snapshot(uint64_t *bestp) const {
+    // Live slots to the best slots of the walkers that want it, one after another by the
+    // whole warp (8 lanes alone wait for memory 66 times at 351 terms).
+    __device__ __forceinline__ void snapshots(bool want, uint64_t *bestp) const {
+        unsigned pend = __ballot_sync(kFull, want && lane == 0);
+        using V = typename std::conditional<NWG % 2 == 0, ulonglong2, unsigned long long>::type;
+        constexpr int PV = NWG * 8 / (int)sizeof(V);   // vectors per slot
 #pragma unroll 1
-        for (int e = lane; e < r * NWG; e += 32) {
-            if constexpr (GW) {
-                bestp[e] = W[e];
-            } else {
-                const int s = e / NWG, g = e - s * NWG;
-                bestp[e] = W[(size_t)s * NWS + smem_word(g)];
-            }
+        while (pend) {
+            const int a = __ffs(pend) - 1;
+            pend &= pend - 1u;
+            const int ra = __shfl_sync(kFull, r, a);
+            const V *src = reinterpret_cast<const V *>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(W), a));
+            V *dst = reinterpret_cast<V *>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(bestp), a));
+#pragma unroll 8
+            for (int e = threadIdx.x & 31; e < ra * PV; e += 32) dst[e] = src[e];
         }
     }
 
     // Expansion (Section 3.3.1): plus (three new terms), or split under walk policy 1
     // when y3 >= 2^31; the changed terms are queued for the cascade;
     // returns the digest record (0 when no attempt passed).
-    __device__ __forceinline__ uint64_t plus_setup(const SegDesc &d) {
+    __device__ __forceinline__ uint64_t plus_setup(const SegDesc &d, bool on) {
+        uint64_t rec = 0;
+        bool pend = on;
 #pragma unroll 1
-        for (int a = 1; a <= d.plus_attempts; ++a) {
+        for (int a = 1; a <= d.plus_attempts && any(pend); ++a) {
             const U4 y = philox10((uint32_t)t, (uint32_t)(t >> 32), wid, (uint32_t)a, key0, key1);
-            const int pi = (int)__umulhi(y.x, (uint32_t)r);
-            const int pj = (pi + 1 + (int)__umulhi(y.y, (uint32_t)(r - 1))) % r;
+            const int pi = pend ? (int)__umulhi(y.x, (uint32_t)r) : 0;
+            const int pj = pend ? (pi + 1 + (int)__umulhi(y.y, (uint32_t)(r - 1))) % r : 0;
             const int perm = (int)__umulhi(y.z, 6u);
             int A, B, C;
             plus_roles(perm, A, B, C);
             const DF ti = dget(pi), tj = dget(pj);
-            if (policy_of(d) == 1 && y.w >= 0x80000000u) {
-                // split: term i = (A_j, B_i, C_i), new term (A_i - A_j, B_i, C_i)
-                DF ns;
-                const bool ok = dadd(ti, tj, A, true, ns);
-                const bool z = dzero(ns, A);
-                if (!ok || z) continue;
-                dcanon(ns);
-                dput(r, ns);
-                DF ti2 = ti;
-                dtake(ti2, tj, A);
-                dcanon(ti2);
-                dput(pi, ti2);
-                r += 1;
+            const bool split = policy_of(d) == 1 && y.w >= 0x80000000u;
+            DF nw, ti2, tj2;   // the new term, terms i and j afterwards
+            bool ok = dadd(ti, tj, B, false, ti2);   // (A_i, B_i + B_j, C_i)
+            ok &= dadd(tj, ti, C, true, tj2);        // (A_i, B_j, C_j - C_i)
+            ok &= dadd(tj, ti, A, true, nw);         // (A_j - A_i, B_j, C_j)
+            const bool zb = dzero(ti2, B), zc = dzero(tj2, C), za = dzero(nw, A);
+            ok = ok && !(zb || zc || za);
+            dtake(tj2, ti, A);
+            if constexpr (PG) {
+                // split: term i = (A_j, B_i, C_i), new term (A_i - A_j, B_i, C_i), term j unchanged
+                DF sw;
+                const bool sok = dadd(ti, tj, A, true, sw);
+                const bool sz = dzero(sw, A);
+                if (split) {
+                    ok = sok && !sz;
+                    nw = sw;
+                    ti2 = ti;
+                    dtake(ti2, tj, A);
+                    tj2 = tj;
+                }
+            }
+            const bool go = pend && ok;
+            pend = pend && !ok;
+            if (!any(go)) continue;
+            dcanon(nw);
+            dcanon(ti2);
+            dcanon(tj2);
+            r += go;
+            put(go, go ? r - 1 : 0, nw);
+            put(go && !split, pj, tj2);
+            put(go, pi, ti2);
+            c_pls += go;
+            if (go) {
                 plateau = 0;
-                c_pls += 1;
                 qlen = 0;
                 q_push(pi);
+                if (!split) q_push(pj);
                 q_push(r - 1);
-                return plus_record(a, perm, pi, pj, 1);
+                rec = plus_record(a, perm, pi, pj, split ? 1 : 0);
             }
-            DF nb, nc, na;
-            bool ok = dadd(ti, tj, B, false, nb);   // B_i + B_j
-            ok &= dadd(tj, ti, C, true, nc);        // C_j - C_i
-            ok &= dadd(tj, ti, A, true, na);        // A_j - A_i
-            const bool z = dzero(nb, B) || dzero(nc, C) || dzero(na, A);
-            if (!ok || z) continue;
-            dcanon(na);                // (A_j - A_i, B_j, C_j)
-            dput(r, na);
-            dtake(nc, ti, A);          // (A_i, B_j, C_j - C_i)
-            dcanon(nc);
-            dput(pj, nc);
-            dcanon(nb);                // (A_i, B_i + B_j, C_i)
-            dput(pi, nb);
-            r += 1;
-            plateau = 0;
-            c_pls += 1;
-            qlen = 0;
-            q_push(pi);
-            q_push(pj);
-            q_push(r - 1);
-            return plus_record(a, perm, pi, pj);
         }
-        return 0;
+        return rec;
     }
 
-    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, int32_t steps, unsigned char *sm) {
-        lane = threadIdx.x & 31;
-        fq = lane < 3 * FW ? lane : 0;
-        R = d.R;
-        KM = (R + 31) >> 5;
-        if constexpr (GW) {
-            W = reinterpret_cast<uint64_t *>(d.slots) + (size_t)w * R * NWG;
-            SG = reinterpret_cast<uint4 *>(sm);
-        } else {
-            W = reinterpret_cast<uint64_t *>(sm);
-            SG = reinterpret_cast<uint4 *>(W + (size_t)R * NWS);
+    // Classes and hash slices of one walker's live slots from scratch, by the whole warp: a
+    // lane per slot, 32 slots at a time (once per launch).  Per factor, chained hash
+    // buckets first (heads in the slices' space, chains in the factor's next array,
+    // entries slot | 6 more hash bits << 10); every slot walks its bucket for the next
+    // member above it, or the lowest one, by hash, checks that one on the words, and
+    // only after a mismatch checks every entry.  (Comparing every slot with all slots by
+    // the slices took 3.6 ms of a launch of 32768 walkers at 351 terms, this 0.9.)
+    __device__ __forceinline__ static void build(const uint64_t *w, int rr, int R, uint16_t *nx, uint32_t *hs) {
+        const int l = threadIdx.x & 31, KW = (R + 31) >> 5;
+        const int heads = 3 * kHashBits * KW;
+        constexpr uint32_t kEnd = 0xffffu;
+        auto factor = [&](int s, int f, uint64_t (&p)[FW], uint64_t (&n)[FW]) -> uint32_t {
+            uint32_t x = 0u;
+#pragma unroll
+            for (int h = 0; h < FW; ++h) {
+                p[h] = s < rr ? w[(size_t)s * NWG + f * FW + h] : 0ull;
+                n[h] = ZT && s < rr ? w[(size_t)s * NWG + TW + f * FW + h] : 0ull;
+                x += word_hash(p[h], n[h], h);
+            }
+            return x;
+        };
+        uint64_t p[FW], n[FW];
+#pragma unroll 1
+        for (int f = 0; f < 3; ++f) {
+            uint16_t *chain = nx + f * R;
+            for (int e = l; e < heads; e += 32) hs[e] = kEnd;
+            __syncwarp();
+#pragma unroll 4
+            for (int s = l; s < rr; s += 32) {
+                const uint32_t x = factor(s, f, p, n) * 0x9E3779B1u;
+                chain[s] = (uint16_t)atomicExch(&hs[__umulhi(x, (uint32_t)heads)], (uint32_t)s | ((x & 63u) << 10));
+            }
+            __syncwarp();
+            uint16_t found[32];   // by chunk
+#pragma unroll 1
+            for (int q = 0; 32 * q < rr; ++q) {
+                const int s = 32 * q + l;
+                int nxt = s;
+                if (s < rr) {
+                    const uint32_t x = factor(s, f, p, n) * 0x9E3779B1u, tag = x & 63u;
+                    const uint32_t head = hs[__umulhi(x, (uint32_t)heads)];
+                    int above = kNone, below = kNone;
+                    for (uint32_t e = head; e != kEnd; e = chain[e & 1023u]) {
+                        const int k = (int)(e & 1023u);
+                        const bool hit = (e >> 10) == tag;
+                        above = hit && k > s ? min(above, k) : above;
+                        below = hit && k < s ? min(below, k) : below;
+                    }
+                    nxt = above != kNone ? above : (below != kNone ? below : s);
+                    if (nxt != s && !fsame(w, nxt, f, p, n)) {
+                        above = below = kNone;
+                        for (uint32_t e = head; e != kEnd; e = chain[e & 1023u]) {
+                            const int k = (int)(e & 1023u);
+                            if (k == s || (e >> 10) != tag || !fsame(w, k, f, p, n)) continue;
+                            if (k > s) above = min(above, k);
+                            else below = min(below, k);
+                        }
+                        nxt = above != kNone ? above : (below != kNone ? below : s);
+                    }
+                }
+                found[q] = (uint16_t)nxt;
+            }
+            __syncwarp();
+            for (int q = 0; 32 * q < R; ++q)
+                if (32 * q + l < R) chain[32 * q + l] = 32 * q + l < rr ? found[q] : (uint16_t)(32 * q + l);
+            __syncwarp();
         }
+#pragma unroll 2
+        for (int q = 0; q < KW; ++q)
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                const uint32_t x = factor(32 * q + l, f, p, n);
+                uint32_t word = 0u;
+#pragma unroll
+                for (int b = 0; b < kHashBits; ++b) {
+                    // slice order of spreads(): top bits of bytes 0 .. 3, then the next bits
+                    const unsigned m = __ballot_sync(kFull, (x >> (8 * (b & 3) + 7 - (b >> 2))) & 1u);
+                    word = l == b ? m : word;
+                }
+                if (l < kHashBits) hs[(f * kHashBits + l) * KW + q] = word;
+            }
+        __syncwarp();
+    }
+
+    // the sampled term's class sizes and members below it, one factor per lane 0 .. 2
+    __device__ __forceinline__ void classes(int i, int &n0, int &n1, int &n2, int &mine_below) const {
+        int n = 0, b = 0;
+        if (lane < 3) {
+            int p = next(i, lane);
+#pragma unroll 1
+            for (; n < R && p != i; ++n) {
+                b += p < i;
+                p = next(p, lane);
+            }
+        }
+        __syncwarp();
+        n0 = from(n, 0); n1 = from(n, 1); n2 = from(n, 2);
+        mine_below = b;
+    }
+
+    // live: the lanes have a walker (w); the others read the first walker's rows and take part
+    // in the warp's votes only
+    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, bool live, int32_t steps) {
+        fq = lane < 3 * FW ? lane : 0;
         tfg_walker_info *H = d.hdr + w;
-        r = H->r; best_r = H->best_r;
+        r = live ? min(max(H->r, 0), R) : 0;   // in range whatever a restored state holds
+        best_r = live ? H->best_r : -1;        // without a walker: no candidate, no best, no expansion
         t = H->t; plateau = H->plateau; best_t = H->best_t;
         dig = H->digest; wid = H->walker_id;
         key0 = d.key0; key1 = d.key1;
         best_nnz = H->best_nnz;
         c_acc = c_rej = c_noc = c_drp = c_mrg = c_pls = c_red = 0;
         qlen = 0; q0 = q1 = q2 = 0;
-        const uint64_t *src = reinterpret_cast<const uint64_t *>(d.slots) + (size_t)w * R * NWG;
         uint64_t *bestp = reinterpret_cast<uint64_t *>(d.best) + (size_t)w * R * NWG;
-        if constexpr (!GW) {
-            // HBM rows (p0 p1 p2 [n0 n1 n2]) -> shared rows grouped by factor
-#pragma unroll 1
-            for (int e = lane; e < R * NWS; e += 32) {
-                const int s = e / NWS, q = e - s * NWS;
-                const int g = ZT ? ((q & 1) ? TW + (q >> 1) : (q >> 1)) : q;   // source word of shared word q
-                W[e] = g < NWG ? src[(size_t)s * NWG + g] : 0ull;
-            }
-            __syncwarp();
-        }
-#pragma unroll 1
-        for (int s = lane; s < 32 * KM; s += 32) SG[s] = s < R ? sig(get(s)) : make_uint4(0u, 0u, 0u, 0u);
-        __syncwarp();
         nnz = 0;
         if (policy_of(d) == 2) {
             uint32_t mine = 0;
 #pragma unroll 1
-            for (int s = lane; s < r; s += 32) {
-                const T v = get(s);
-                for (int x = 0; x < TW; ++x) mine += (uint32_t)__popcll(v.p[x] | v.n[x]);
+            for (int e = lane; e < r * TW; e += G) {
+                const int s = e / TW, q = e - s * TW;
+                mine += (uint32_t)__popcll(W[(size_t)s * NWG + q] | (ZT ? W[(size_t)s * NWG + TW + q] : 0ull));
             }
-            nnz = __reduce_add_sync(kFull, mine);
+            __syncwarp();
+            nnz = sum(mine);
         }
 
         uint32_t xr0 = 0, xr1 = 0, xr2 = 0, xr3 = 0;
-        int kb = 32;
+        int kb = G;
 #pragma unroll 1
         for (int32_t step = 0; step < steps; ++step) {
             // ---- draw: lane l holds the Philox output of step (batch start + l)
-            if (kb == 32) {
+            if (kb == G) {
                 const uint64_t tl = (uint64_t)t + (uint64_t)lane;
                 const U4 x = philox10((uint32_t)tl, (uint32_t)(tl >> 32), wid, 0u, key0, key1);
                 xr0 = x.x; xr1 = x.y; xr2 = x.z; xr3 = x.w;
                 kb = 0;
             }
-            const uint32_t x0 = __shfl_sync(kFull, xr0, kb), x1 = __shfl_sync(kFull, xr1, kb),
-                           x2 = __shfl_sync(kFull, xr2, kb), x3 = PG ? __shfl_sync(kFull, xr3, kb) : 0u;
+            const uint32_t x0 = from(xr0, kb), x1 = from(xr1, kb), x2 = from(xr2, kb), x3 = PG ? from(xr3, kb) : 0u;
             kb += 1;
 
             const int r_before = r;
             const int i = (int)__umulhi(x0, (uint32_t)r);
+            const DF di = dget(i);   // on its way during the walk over the lists
+            // ---- try_flip: candidates (X, j) with X_j = +-X_i, ordered (X, slot)
+            int nU, nV, nW, below;
+            classes(i, nU, nV, nW, below);
+            const int K = live ? 2 * (nU + nV + nW) : 0;
+            const int c = (int)__umulhi(x1, (uint32_t)K);
+            const int mi = c >> 1;
             int action = kNoCand, X = 0, j = 0, rho = 0, sneg = 0;
-            {
-                const T ti = get(i);
-                const uint4 si = SG[i];
-                // ---- try_flip: candidates (X, j) with X_j = +-X_i, ordered (X, slot)
-                uint32_t bu = 0, bv = 0, bw = 0;   // bit k: slot k*32 + lane is a candidate
-#pragma unroll 4
-                for (int k = 0; k < KM; ++k) {
-                    const int s = (k << 5) + lane;
-                    const uint4 g = SG[s];
-                    const bool live = s < r && s != i;
-                    bu |= (uint32_t)(live && g.x == si.x) << k;
-                    bv |= (uint32_t)(live && g.y == si.y) << k;
-                    bw |= (uint32_t)(live && g.z == si.z) << k;
+            if (K > 0) {
+                rho = c & 1;
+                X = (int)(mi >= nU) + (int)(mi >= nU + nV);
+            }
+            const int idx = mi - (X == 0 ? 0 : (X == 1 ? nU : nU + nV));
+            const int bX = from(below, X);
+            if (K > 0) {
+                // the idx-th candidate of factor X in slot order: the cycle after i has the
+                // members above i, then those below
+                const int n = X == 0 ? nU : (X == 1 ? nV : nW);
+                int go = idx < bX ? n - bX + idx : idx - bX;
+                j = next(i, X);
+#pragma unroll 1
+                for (; go > 0; --go) j = next(j, X);
+            }
+            __syncwarp();
+            const DF dj = dget(j);
+            const bool wneg = dwneg(dj, di);
+            sneg = (X == 2 && wneg && K > 0) ? 1 : 0;
+            // flip: (Y, Z) cyclic after X, rho swaps; Y_i += Y_j, Z_j -= s Z_i
+            const int X1 = X == 2 ? 0 : X + 1, X2 = X == 0 ? 2 : X - 1;
+            const int Y = rho ? X2 : X1, Z = rho ? X1 : X2;
+            DF ti2, tj2;
+            bool ok = dadd(di, dj, Y, false, ti2);
+            ok &= dadd(dj, di, Z, sneg == 0, tj2);
+            const bool acc = K > 0 && ok;
+            if (K > 0) action = ok ? kAccept : kReject;
+            c_noc += K == 0;
+            c_rej += action == kReject;
+            c_acc += acc;
+            qlen = 0;
+            if (any(acc)) {
+                const bool zi = dzero(ti2, Y);
+                const bool zj = dzero(tj2, Z);
+                if (policy_of(d) == 2) {
+                    const uint32_t ci = dnnz(ti2), cj = dnnz(tj2), bi = dnnz(di), bj = dnnz(dj);
+                    if (acc) nnz += (zi ? 0u : ci) + (zj ? 0u : cj) - bi - bj;
                 }
-                uint32_t any = bu | bv | bw;   // signature hits: verify on the full words
+                dcanon(ti2);
+                dcanon(tj2);
+                dput(acc, i, ti2);
+                dput(acc, j, tj2);
+                // of the other factors the normalisation changes the sign of w at most
+                relink<true>(acc, i, Y, ti2, j, Z, tj2);
+                const bool zz = acc && (zi || zj);
+                if (policy_of(d) != 2) {
+                    // A third slot shares a pair with the new term i iff it is in two of its
+                    // classes x, e1, z, with the new term j iff in two of x, e2, e3: the five
+                    // classes' members (j aside in x) modulo 32, a lane each, as a superset
+                    // test (the cascade checks exactly).
+                    uint32_t mask = 0u;
+                    if (acc && !zz && lane < 5) {
+                        const int s = lane < 3 ? i : j;
+                        const int f = lane == 0 ? X : ((lane == 1 || lane == 4) ? Z : Y);
+                        int p = next(s, f);
 #pragma unroll 1
-                while (any) {
-                    const int k = __ffs(any) - 1;
-                    any &= any - 1u;
-                    const uint32_t bit = 1u << k;
-                    const int s = (k << 5) + lane;
-                    if ((bu & bit) && !fmatch(s, 0, ti, false)) bu &= ~bit;
-                    if ((bv & bit) && !fmatch(s, 1, ti, false)) bv &= ~bit;
-                    if ((bw & bit) && !fmatch(s, 2, ti, true)) bw &= ~bit;
-                }
-                const uint32_t tot = __reduce_add_sync(kFull, (uint32_t)__popc(bu) | ((uint32_t)__popc(bv) << 10) |
-                                                                  ((uint32_t)__popc(bw) << 20));
-                const int nU = (int)(tot & 1023u), nV = (int)((tot >> 10) & 1023u), nW = (int)(tot >> 20);
-                const int K = 2 * (nU + nV + nW);
-
-                if (K > 0) {
-                    const int c = (int)__umulhi(x1, (uint32_t)K);
-                    rho = c & 1;
-                    const int mi = c >> 1;
-                    int idx;
-                    if (mi < nU) { X = 0; idx = mi; }
-                    else if (mi < nU + nV) { X = 1; idx = mi - nU; }
-                    else { X = 2; idx = mi - nU - nV; }
-                    // the idx-th candidate of factor X in slot order (k, then lane)
-                    const uint32_t mk = X == 0 ? bu : (X == 1 ? bv : bw);
-                    int k = 0;
-                    unsigned b = __ballot_sync(kFull, mk & 1u);
-#pragma unroll 1
-                    for (; k + 1 < KM; ) {
-                        const int cnt = __popc(b);
-                        if (idx < cnt) break;
-                        idx -= cnt;
-                        ++k;
-                        b = __ballot_sync(kFull, (mk >> k) & 1u);
-                    }
-#pragma unroll 1
-                    for (int q = 0; q < idx && b; ++q) b &= b - 1u;
-                    j = (k << 5) + __ffs(b) - 1;
-                    const DF di = dof(ti), dj = dget(j);
-                    sneg = (X == 2 && dwneg(dj, di)) ? 1 : 0;
-
-                    // flip: (Y, Z) cyclic after X, rho swaps; Y_i += Y_j, Z_j -= s Z_i
-                    int Y = X == 0 ? 1 : (X == 1 ? 2 : 0);
-                    int Z = X == 0 ? 2 : (X == 1 ? 0 : 1);
-                    if (rho) { const int tmp = Y; Y = Z; Z = tmp; }
-                    DF ti2, tj2;
-                    bool ok = dadd(di, dj, Y, false, ti2);
-                    ok &= dadd(dj, di, Z, sneg == 0, tj2);
-                    if (!ok) {
-                        action = kReject;
-                        c_rej += 1;
-                    } else {
-                        action = kAccept;
-                        c_acc += 1;
-                        const bool zi = dzero(ti2, Y);
-                        const bool zj = dzero(tj2, Z);
-                        if (policy_of(d) == 2)
-                            nnz += (zi ? 0u : dnnz(ti2)) + (zj ? 0u : dnnz(tj2)) - dnnz(di) - dnnz(dj);
-                        dcanon(ti2);
-                        dcanon(tj2);
-                        dput(i, ti2);
-                        dput(j, tj2);
-                        qlen = 0;
-                        if (zi || zj) {
-                            q_push(i);
-                            q_push(j);
-                            const int hi = i > j ? i : j, lo = i > j ? j : i;
-                            const bool zhi = (hi == i) ? zi : zj, zlo = (lo == i) ? zi : zj;
-                            if (zhi) { drop(hi); c_drp += 1; }
-                            if (zlo) { drop(lo); c_drp += 1; }
-                            if (policy_of(d) == 2) qlen = 0;   // no reduction edges
-                        } else if (policy_of(d) != 2 && pair_filter(i, j)) {
-                            q_push(i);
-                            q_push(j);
+                        for (int q = 0; q < R && p != s; ++q) {
+                            mask |= lane == 0 && p == j ? 0u : 1u << (p & 31);
+                            p = next(p, f);
                         }
                     }
-                } else {
-                    c_noc += 1;
+                    __syncwarp();
+                    const uint32_t cx = from(mask, 0), cz = from(mask, 1), e1 = from(mask, 2), e2 = from(mask, 3),
+                                   e3 = from(mask, 4);
+                    if ((cx & cz) | (e1 & (cx | cz)) | (e2 & (cx | e3)) | (cx & e3)) {
+                        q_push(i);
+                        q_push(j);
+                    }
+                }
+                if (any(zz)) {
+                    if (zz) {
+                        q_push(i);
+                        q_push(j);
+                    }
+                    const int hi = i > j ? i : j, lo = i > j ? j : i;
+                    const bool zhi = zz && ((hi == i) ? zi : zj), zlo = zz && ((lo == i) ? zi : zj);
+                    if (any(zhi)) drop(zhi, hi);
+                    if (any(zlo)) drop(zlo, lo);
+                    c_drp += (uint32_t)zhi + (uint32_t)zlo;
+                    if (policy_of(d) == 2) qlen = 0;   // no reduction edges
                 }
             }
-
-            // ---- reduction cascade (flip), then bookkeeping, then plus + cascade
-            bool plus_phase = false;
-            uint64_t rec2 = 0;
-#pragma unroll 1
-            for (;;) {
+            cascade();
+            // ---- digest, best scheme, plateau
+            c_red += r < r_before;
+            dig = digest_mix(dig, flip_record(action, X, rho, sneg, i, j, r));
+            // walk policy 1: a failed try_flip expands and ends the step (no best update)
+            const bool failed = policy_of(d) == 1 && action != kAccept;
+            // best scheme: always when better, with probability 0.01 when equal
+            // (policy 2: better = least (rank, non-zero coefficients))
+            const bool better = !failed && (r < best_r || (policy_of(d) == 2 && r == best_r && nnz < best_nnz));
+            const bool again = !failed && r == best_r && (policy_of(d) != 2 || nnz == best_nnz) && x2 < d.refresh_thresh;
+            plateau += 1;
+            if (better) {
+                best_r = r;
+                if (policy_of(d) == 2) best_nnz = nnz;
+                best_t = t;
+                plateau = 0;
+            }
+            if (any(better || again)) snapshots(better || again, bestp);
+            // expansion: plus on a plateau near the best rank (policy 0), or Algorithm 1's
+            // expand after a failed try_flip / with probability p_expand (policy 1)
+            bool expand;
+            if (policy_of(d) == 2)
+                expand = false;
+            else if (policy_of(d) == 1)
+                expand = failed ? (r < R && r >= 2) : (x3 < d.expand_thresh && r <= best_r + 2 && r < R && r >= 2);
+            else
+                expand = d.plus_enabled && plateau >= d.plateau_len && r <= best_r + 2 && r < R && r >= 2;
+            __syncwarp();
+            if (any(expand)) {
+                const uint64_t rec = plus_setup(d, expand);
                 cascade();
-                if (plus_phase) {
-                    dig = digest_mix(dig, rec2 | ((uint64_t)(uint32_t)r << 44));
-                    break;
-                }
-                if (r < r_before) c_red += 1;
-                dig = digest_mix(dig, flip_record(action, X, rho, sneg, i, j, r));
-                // walk policy 1: a failed try_flip expands and ends the step (no best update)
-                const bool failed = policy_of(d) == 1 && action != kAccept;
-                // best scheme: always when better, with probability 0.01 when equal
-                // (policy 2: better = least (rank, non-zero coefficients))
-                if (policy_of(d) == 2) {
-                    if (r < best_r || (r == best_r && nnz < best_nnz)) {
-                        snapshot(bestp);
-                        best_r = r;
-                        best_nnz = nnz;
-                        best_t = t;
-                        plateau = 0;
-                    } else {
-                        if (r == best_r && nnz == best_nnz && x2 < d.refresh_thresh) snapshot(bestp);
-                        plateau += 1;
-                    }
-                } else if (failed) {
-                    plateau += 1;
-                } else if (r < best_r) {
-                    snapshot(bestp);
-                    best_r = r;
-                    best_t = t;
-                    plateau = 0;
-                } else {
-                    if (r == best_r && x2 < d.refresh_thresh) snapshot(bestp);
-                    plateau += 1;
-                }
-                // expansion: plus on a plateau near the best rank (policy 0), or Algorithm 1's
-                // expand after a failed try_flip / with probability p_expand (policy 1)
-                bool expand;
-                if (policy_of(d) == 2)
-                    expand = false;
-                else if (policy_of(d) == 1)
-                    expand = failed ? (r < R && r >= 2) : (x3 < d.expand_thresh && r <= best_r + 2 && r < R && r >= 2);
-                else
-                    expand = d.plus_enabled && plateau >= d.plateau_len && r <= best_r + 2 && r < R && r >= 2;
-                if (expand) {
-                    rec2 = plus_setup(d);
-                    if (rec2) { plus_phase = true; continue; }
-                }
-                break;
+                if (rec) dig = digest_mix(dig, rec | ((uint64_t)(uint32_t)r << 44));
             }
             t += 1;
         }
 
-        // ---- write back
-        uint64_t *dst = reinterpret_cast<uint64_t *>(d.slots) + (size_t)w * R * NWG;
-        if constexpr (!GW) {
-#pragma unroll 1
-            for (int e = lane; e < R * NWG; e += 32) {
-                const int s = e / NWG, g = e - s * NWG;
-                dst[e] = W[(size_t)s * NWS + smem_word(g)];
-            }
-        }
-        if (lane == 0) {
+        // ---- write back (the slots were written in place)
+        if (live && lane == 0) {
             H->r = r; H->best_r = best_r;
             H->t = t; H->plateau = plateau; H->best_t = best_t;
             H->digest = dig;
@@ -752,90 +812,116 @@ struct WideWalker {
     }
 };
 
-template <int MODE, bool GW, int FW>
-__host__ __device__ constexpr size_t wide_walker_bytes(int R) {
-    return (GW ? (size_t)0 : (size_t)R * WideWalker<MODE, GW, false, FW>::NWS * 8) + (size_t)((R + 31) / 32) * 32 * 16;
-}
+constexpr int kWideBlock = 64;
 
-constexpr int kWideWarps = 2;   // walkers (warps) per block
-
-// With the term words in HBM, registers bound residency: capped for 16
-// two-warp blocks per SM with one word per factor (measured +4-8% on ranks 285
-// and 351), 8 with two.
-template <int MODE, bool GW, bool PG, int FW>
-__global__ void __launch_bounds__(32 * kWideWarps, GW ? 16 / FW : 1) walk_wide_kernel(const SegDesc d, const int32_t steps) {
+// per: walkers per warp (1 .. 4), the first of its four groups of lanes
+template <int MODE, bool PG, int FW, bool GM>
+__global__ void __launch_bounds__(kWideBlock, 10) walk_wide_kernel(const SegDesc d, const int32_t steps, const int per) {
     extern __shared__ __align__(16) unsigned char wide_sm[];
-    const int warp = threadIdx.x >> 5;
-    const int64_t w = (int64_t)blockIdx.x * kWideWarps + warp;
-    if (w >= d.n_walkers) return;   // whole warps exit together
-    WideWalker<MODE, GW, PG, FW> wk;
-    wk.run(d, w, steps, wide_sm + wide_walker_bytes<MODE, GW, FW>(d.R) * warp);
+    using WW = WideWalker<MODE, PG, FW, GM>;
+    const int wl = threadIdx.x & 31, group = wl / WW::G;
+    const size_t bytes = WW::walker_bytes(d.R);
+    unsigned char *at = wide_sm + bytes * per * (threadIdx.x >> 5);
+    const int64_t first = ((int64_t)blockIdx.x * (kWideBlock / 32) + (threadIdx.x >> 5)) * per;
+    if (first >= d.n_walkers) return;   // no block-wide barrier is used
+    const int here = (int)min((int64_t)per, d.n_walkers - first);   // the warp's walkers
+    WW wk;
+    wk.R = d.R;
+    wk.KW = (d.R + 31) >> 5;
+    const int words = d.R * WW::NWG;
+    uint64_t *slots = reinterpret_cast<uint64_t *>(d.slots) + (size_t)first * words;
+    // the whole warp stages its walkers and builds their classes, one after another
+#pragma unroll 1
+    for (int a = 0; a < here; ++a) {
+        wk.attach(at + bytes * a, slots + (size_t)a * words);
+        if constexpr (!GM) {
+#pragma unroll 4
+            for (int e = wl; e < words; e += 32) wk.W[e] = slots[(size_t)a * words + e];
+            __syncwarp();
+        }
+        WW::build(wk.W, min(max(d.hdr[first + a].r, 0), d.R), d.R, wk.nx, wk.hs);
+    }
+    wk.lane = wl % WW::G;
+    wk.gb = wl - wk.lane;
+    const bool live = group < here;
+    const int a = live ? group : 0;
+    wk.attach(at + bytes * a, slots + (size_t)a * words);
+    wk.run(d, first + a, live, steps);
+    if constexpr (!GM) {
+        __syncwarp();
+#pragma unroll 1
+        for (int b = 0; b < here; ++b) {
+            wk.attach(at + bytes * b, slots);
+#pragma unroll 4
+            for (int e = wl; e < words; e += 32) slots[(size_t)b * words + e] = wk.W[e];
+        }
+    }
 }
 
 }  // namespace dev
 
 namespace {
 
-constexpr int kWideMaxSmem = 227 * 1024;
-
-// Term words stay in HBM from this capacity on: shared-memory residency (22.8 KB
-// per walker at 354 slots) limits the larger ranks.  Measured on 16384 walkers:
-// rank 202 (capacity 205) 1.00e9 shared vs 0.98e9 HBM steps/s; rank 285: 0.69e9 vs
-// 0.85e9; rank 351: 0.46e9 vs 0.73e9.  Two words per factor double the bytes per
-// slot, so the switch comes at half the capacity.
-template <int FW>
-constexpr int wide_hbm_words_min_r() { return 256 / FW; }
-
 template <int MODE, int FW>
 void prepare_walk_wide() {
     static bool attr = [] {
-        cudaFuncSetAttribute(dev::walk_wide_kernel<MODE, false, false, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideMaxSmem);
-        cudaFuncSetAttribute(dev::walk_wide_kernel<MODE, true, false, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideMaxSmem);
-        cudaFuncSetAttribute(dev::walk_wide_kernel<MODE, false, true, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideMaxSmem);
-        cudaFuncSetAttribute(dev::walk_wide_kernel<MODE, true, true, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideMaxSmem);
+        auto set = [](auto kernel) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinkSmem);
+        };
+        set(dev::walk_wide_kernel<MODE, false, FW, false>);
+        set(dev::walk_wide_kernel<MODE, false, FW, true>);
+        set(dev::walk_wide_kernel<MODE, true, FW, false>);
+        set(dev::walk_wide_kernel<MODE, true, FW, true>);
         return true;
     }();
     (void)attr;
 }
 
-template <int MODE, bool GW, int FW>
-void launch_wide_as(const SegDesc &d, int32_t steps, cudaStream_t st) {
-    const size_t smem = dev::wide_walker_bytes<MODE, GW, FW>(d.R) * dev::kWideWarps;
-    if (d.n_walkers <= 0 || smem > (size_t)kWideMaxSmem) return;
-    const int64_t grid = (d.n_walkers + dev::kWideWarps - 1) / dev::kWideWarps;
-    if (d.walk_policy == 0)
-        dev::walk_wide_kernel<MODE, GW, false, FW><<<(unsigned)grid, 32 * dev::kWideWarps, smem, st>>>(d, steps);
-    else
-        dev::walk_wide_kernel<MODE, GW, true, FW><<<(unsigned)grid, 32 * dev::kWideWarps, smem, st>>>(d, steps);
-}
-
+// Walkers per warp: four, unless that leaves an SM's schedulers without two warps each; a
+// warp takes the changing part of a step when any of its walkers does, so a lone
+// walker's step is shorter.  The terms go to shared memory when the whole population
+// resides at once that way.  Measured, (4,5,5), 300 walkers, 400 steps: four a warp in
+// device memory 0.91 ms, in shared memory 0.82, one a warp 0.49 (the kernel before: 0.45).
 template <int MODE, int FW>
 void launch_walk_wide(const SegDesc &d, int32_t steps, int /*grid*/, int /*block*/, cudaStream_t st) {
     prepare_walk_wide<MODE, FW>();
-    if (d.R >= wide_hbm_words_min_r<FW>()) launch_wide_as<MODE, true, FW>(d, steps, st);
-    else launch_wide_as<MODE, false, FW>(d, steps, st);
+    using Shared = dev::WideWalker<MODE, false, FW, false>;
+    using Device = dev::WideWalker<MODE, false, FW, true>;
+    if (d.n_walkers <= 0) return;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per = 32 / Shared::G;
+    while (per > 1 && (d.n_walkers + per - 1) / per < (int64_t)sms * 8) per /= 2;
+    const int walkers = dev::kWideBlock / 32 * per;   // of a block
+    const unsigned grid = (unsigned)((d.n_walkers + walkers - 1) / walkers);
+    const bool shared = link_terms_shared(Shared::walker_bytes(d.R) * walkers, grid);
+    const size_t smem = (shared ? Shared::walker_bytes(d.R) : Device::walker_bytes(d.R)) * walkers;
+    if (shared) {
+        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, false><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+        else dev::walk_wide_kernel<MODE, true, FW, false><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+    } else {
+        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, true><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+        else dev::walk_wide_kernel<MODE, true, FW, true><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+    }
+}
+
+// G = 32 is the mapping's name in tfg_params and tfg_mapping; the kernel sets its own launch shape.
+template <int MODE, int FW>
+WalkVariant wide_variant() {
+    return WalkVariant{MODE, 64, 3 * FW, 32, 0, 0, &launch_walk_wide<MODE, FW>,
+                       reinterpret_cast<const void *>(&dev::walk_wide_kernel<MODE, false, FW, true>),
+                       &prepare_walk_wide<MODE, FW>, 1023};
 }
 
 }  // namespace
 
 // Factor-aligned terms: 3 (factors of at most 64 coefficients) or 6 (at most
-// 128) words of 64 bits per sign; capacity 1023 slots (the shared-memory need
-// of two walkers per block stays under 227 KB).
+// 128) words of 64 bits per sign; capacity 1023 slots (74 KB of shared memory for a
+// block's eight walkers).
 const WalkVariant *walk_variants_wide(int *n) {
-    static const WalkVariant v[] = {
-        WalkVariant{TFG_MODE_ZT, 64, 3, 32, 0, 0, &launch_walk_wide<TFG_MODE_ZT, 1>,
-                    reinterpret_cast<const void *>(&dev::walk_wide_kernel<TFG_MODE_ZT, true, false, 1>),
-                    &prepare_walk_wide<TFG_MODE_ZT, 1>, 1023},
-        WalkVariant{TFG_MODE_Z2, 64, 3, 32, 0, 0, &launch_walk_wide<TFG_MODE_Z2, 1>,
-                    reinterpret_cast<const void *>(&dev::walk_wide_kernel<TFG_MODE_Z2, true, false, 1>),
-                    &prepare_walk_wide<TFG_MODE_Z2, 1>, 1023},
-        WalkVariant{TFG_MODE_ZT, 64, 6, 32, 0, 0, &launch_walk_wide<TFG_MODE_ZT, 2>,
-                    reinterpret_cast<const void *>(&dev::walk_wide_kernel<TFG_MODE_ZT, true, false, 2>),
-                    &prepare_walk_wide<TFG_MODE_ZT, 2>, 1023},
-        WalkVariant{TFG_MODE_Z2, 64, 6, 32, 0, 0, &launch_walk_wide<TFG_MODE_Z2, 2>,
-                    reinterpret_cast<const void *>(&dev::walk_wide_kernel<TFG_MODE_Z2, true, false, 2>),
-                    &prepare_walk_wide<TFG_MODE_Z2, 2>, 1023},
-    };
+    static const WalkVariant v[] = {wide_variant<TFG_MODE_ZT, 1>(), wide_variant<TFG_MODE_Z2, 1>(),
+                                    wide_variant<TFG_MODE_ZT, 2>(), wide_variant<TFG_MODE_Z2, 2>()};
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;
 }
