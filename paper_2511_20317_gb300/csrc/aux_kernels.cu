@@ -375,7 +375,8 @@ void verify_teams(const SegDesc &d, int64_t first, int64_t count, unsigned long 
     // slab up to kSlabWords, else in even ones.  A slab of one u-index has at most 128 x
     // 128 entries.
     constexpr int64_t kWarpWords = 3072, kSlabWords = 40960;
-    if (words <= kWarpWords && !wide) {
+    // Few walkers (a collected best scheme): a block each, whose warps share the terms.
+    if (words <= kWarpWords && !wide && count > 2 * sms) {
         verify_variant<Wd, false, FB, false>(d, first, count, lu, (int)words, sms, fail, st);
         return;
     }

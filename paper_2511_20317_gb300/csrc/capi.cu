@@ -92,7 +92,9 @@ int min_factor_len(const tfg_format &f) { return std::min(f.m * f.n, std::min(f.
 // The variant of the smallest capacity >= R for a mapping (G lanes per walker);
 // at equal capacity a bit-sliced variant (fl >= the longest factor) wins, and a
 // square one (every factor exactly fl) over that.
-const tfg::WalkVariant *pick_variant(int mode, int bits, int tw, int G, int R, const tfg_format &fmt) {
+// by_mapping: without the variants that tfg_params.mapping does not name
+const tfg::WalkVariant *pick_variant(int mode, int bits, int tw, int G, int R, const tfg_format &fmt,
+                                     bool by_mapping = false) {
     const int maxlen = max_factor_len(fmt), minlen = min_factor_len(fmt);
     auto score = [](const tfg::WalkVariant &x) { return (x.fl ? 1 : 0) + (x.sq ? 1 : 0); };
     int cnt = 0;
@@ -100,7 +102,7 @@ const tfg::WalkVariant *pick_variant(int mode, int bits, int tw, int G, int R, c
     const tfg::WalkVariant *best = nullptr;
     for (int a = 0; a < cnt; ++a) {
         if (v[a].mode != mode || v[a].word_bits != bits || v[a].tw != tw || v[a].G != G) continue;
-        if (v[a].capacity() < R) continue;
+        if (v[a].capacity() < R || (by_mapping && v[a].auto_only)) continue;
         if (v[a].fl && v[a].fl < maxlen) continue;
         if (v[a].sq && (minlen != v[a].fl || maxlen != v[a].fl)) continue;
         if (!best || v[a].S < best->S || (v[a].S == best->S && score(v[a]) > score(*best))) best = &v[a];
@@ -124,11 +126,15 @@ const tfg::WalkVariant *with_block(const tfg::WalkVariant *v, int block) {
     return v;
 }
 
-// Default mapping: one thread per walker (shared-memory slots) when such a
-// variant exists for the rank; otherwise the fewest lanes per walker that keep
+// Default mapping: one thread per walker when such a variant exists for the rank (32-bit
+// terms of 33 to 64 slots: for populations that fill the GPU that way; (2,4,4), 300 steps,
+// lane groups / thread per walker: 1000 walkers 0.38 / 0.58 ms, 30000 walkers 3.0 /
+// 0.68; Algorithm 1 policy 0.47 / 1.4 and 3.4 / 2.1); otherwise the fewest lanes per walker that keep
 // at most 4 slots per lane; otherwise 32 lanes.
-const tfg::WalkVariant *default_variant(int mode, int bits, int tw, int R, const tfg_format &fmt) {
-    if (const tfg::WalkVariant *v = pick_variant(mode, bits, tw, 1, R, fmt)) return v;
+const tfg::WalkVariant *default_variant(int mode, int bits, int tw, int R, const tfg_format &fmt, int64_t walkers,
+                                        int policy) {
+    const bool many = walkers >= (policy == 1 ? 16384 : 8192);
+    if (const tfg::WalkVariant *v = pick_variant(mode, bits, tw, 1, R, fmt, !many)) return v;
     static const int order[4] = {4, 8, 16, 32};
     for (int G : order) {
         const tfg::WalkVariant *v = pick_variant(mode, bits, tw, G, R, fmt);
@@ -397,8 +403,8 @@ static int plan_segments(int32_t n_formats, const tfg_format *fmts, const int32_
         first += s.n;
         if (first > (int64_t)UINT32_MAX) { set_error("more than 2^32 walkers"); return TFG_EINVAL; }
         off = layout_segment(s, off);
-        s.var = prm.mapping ? pick_variant(s.fmt.mode, s.word_bits, s.tw, prm.mapping, s.R, s.fmt)
-                            : default_variant(s.fmt.mode, s.word_bits, s.tw, s.R, s.fmt);
+        s.var = prm.mapping ? pick_variant(s.fmt.mode, s.word_bits, s.tw, prm.mapping, s.R, s.fmt, true)
+                            : default_variant(s.fmt.mode, s.word_bits, s.tw, s.R, s.fmt, s.n, prm.walk_policy);
         s.var = with_block(s.var, prm.block_threads);
         if (!s.var) { set_error("no compiled kernel variant for this format/rank/mapping"); return TFG_EINVAL; }
     }

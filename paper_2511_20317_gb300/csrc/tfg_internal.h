@@ -54,6 +54,7 @@ struct WalkVariant {
     int cap = 0;         // slot capacity when not given by G and S
     int fl = 0;          // > 0: formats whose factors have at most fl coefficients only (bit-sliced)
     int sq = 0;          // 1: formats whose three factors have exactly fl coefficients only
+    bool auto_only = false;   // not selectable by tfg_params.mapping
     int capacity() const { return cap ? cap : (G == 1 ? S : G * S); }
 };
 

@@ -358,6 +358,24 @@ struct LinkWalker {
         uint32_t ea, eb;
         relink_pair<false>(s, f, v, s, f, v, ea, eb);
     }
+    // Lists: slot s (a class of its own) into the class of slot m
+    __device__ __forceinline__ void link(int s, int f, int m) {
+        int p = m, n = next(p, f);
+#pragma unroll 1
+        while (!(p < n ? (p < s && s < n) : (s > p || s < n))) {
+            p = n;
+            n = next(p, f);
+        }
+        next(p, f) = (uint8_t)s;
+        next(s, f) = (uint8_t)n;
+        if constexpr (CNT) {
+#pragma unroll 1
+            for (; n != s; n = next(n, f)) {
+                count(n, 1);
+                count(s, 1);
+            }
+        }
+    }
     // take slot s out of its class of factor f (it becomes a class of its own)
     __device__ __forceinline__ void unlink(int s, int f) {
         if constexpr (ROWS) {
@@ -385,13 +403,6 @@ struct LinkWalker {
             }
         }
     }
-    // slot s := term v, every class anew
-    __device__ __forceinline__ void put(int s, const T &v) {
-        st(s, v);
-#pragma unroll 1
-        for (int f = 0; f < 3; ++f) relink(s, f, v);
-    }
-
     // ---- reduction queue (slot indices)
     __device__ __forceinline__ void q_push(int s) {
         q0 = (qlen == 0) ? s : q0;
@@ -418,18 +429,44 @@ struct LinkWalker {
         q2 = (qlen > 2 && q2 == from) ? to : q2;
     }
 
+    // Slot h (in no class) takes slot last's term and place in its classes; last leaves them.
+    __device__ __forceinline__ void move_slot(int last, int h) {
+        st(h, ld(last));
+        // hash bits
+#pragma unroll 1
+        for (int f = 0; f < 3; ++f) {
+            uint32_t *from = hs + (f * kHashBits * NW + (last >> 5)) * kLane, *to = hs + (f * kHashBits * NW + (h >> 5)) * kLane;
+#pragma unroll
+            for (int b = 0; b < kHashBits; ++b) {
+                const uint32_t v = (from[b * NW * kLane] >> (last & 31)) & 1u, w = to[b * NW * kLane];
+                to[b * NW * kLane] = (w & ~(1u << (h & 31))) | (v << (h & 31));
+            }
+            if constexpr (ROWS) {
+                uint32_t e = row(last, f);
+                row(last, f) = 0u;
+                row(h, f) = e;
+                const uint32_t both = (1u << last) | (1u << h);
+#pragma unroll 1
+                while (e) {
+                    row(__ffs(e) - 1, f) ^= both;
+                    e &= e - 1u;
+                }
+            } else {
+                const int m = next(last, f);
+                unlink(last, f);
+                if (m != last) link(h, f, m);
+            }
+        }
+    }
     // Remove slot h: the last live term moves into the hole.
     __device__ __forceinline__ void drop(int h) {
         const int last = r - 1;
         q_remove(h);
 #pragma unroll 1
-        for (int f = 0; f < 3; ++f) {
-            unlink(h, f);
-            if (h != last) unlink(last, f);
-        }
+        for (int f = 0; f < 3; ++f) unlink(h, f);
         r -= 1;
         if (h != last) {
-            put(h, ld(last));
+            move_slot(last, h);
             q_rename(last, h);
         }
     }
@@ -561,10 +598,26 @@ struct LinkWalker {
             }
             O::canon(nx, mk);
             O::canon(ti2, mk);
+            // Slots i and j and the new one are stored, then enter their classes factor by
+            // factor (a split leaves term j, and of term i only A changes): of each factor
+            // the slot that had a class before comes first, the new slot, still alone, last.
+            const int n = r;
             r += 1;
-            put(r - 1, nx);
-            if (!split) put(pj, tj2);
-            put(pi, ti2);
+            st(pi, ti2);
+            st(n, nx);
+            uint32_t e0, e1;
+            if (split) {
+                relink_pair<true>(pi, A, ti2, n, B, nx, e0, e1);
+                relink_pair<true>(n, A, nx, n, C, nx, e0, e1);
+            } else {
+                st(pj, tj2);
+#pragma unroll 1
+                for (int h = 0; h < 3; ++h) {
+                    const bool h0 = h == 0, h1 = h == 1;
+                    relink_pair<true>(h0 ? pi : (h1 ? pj : n), h0 ? B : (h1 ? C : B), h0 ? ti2 : (h1 ? tj2 : nx),
+                                      h0 ? pj : n, h0 ? A : (h1 ? A : C), h0 ? tj2 : nx, e0, e1);
+                }
+            }
             restart(d);
             c_pls += 1;
             qlen = 0;
@@ -947,11 +1000,5 @@ void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cuda
         else dev::walk_link_kernel<MODE, Wd, NW, true, true><<<grid, block, smem, st>>>(d, steps);
     }
 }
-
-// capacity CAP, BLOCK walkers per block
-#define TFG_LINK_VARIANT(MODE, WD, BITS, CAP, BLOCK) \
-    WalkVariant{MODE, BITS, 1, 1, CAP, BLOCK, &launch_walk_link<MODE, WD, (CAP + 31) / 32>, \
-                reinterpret_cast<const void *>(&dev::walk_link_kernel<MODE, WD, (CAP + 31) / 32, BITS == 64, false>), \
-                &prepare_walk_link<MODE, WD, (CAP + 31) / 32>}
 
 }  // namespace tfg

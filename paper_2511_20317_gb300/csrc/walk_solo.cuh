@@ -1097,11 +1097,6 @@ void launch_walk_solo(const SegDesc &d, int32_t steps, int grid, int /*block*/, 
     dev::solo_kernel<MODE, Wd, RMAX, BT, FL, SQ>()<<<grid, BT, solo_smem_bytes<MODE, Wd, RMAX, BT, FL>(), st>>>(d, steps);
 }
 
-#define TFG_SOLO_VARIANT(MODE, WD, BITS, RMAX, BT) \
-    WalkVariant{MODE, BITS, 1, 1, RMAX, BT, &launch_walk_solo<MODE, WD, RMAX, BT>, \
-                reinterpret_cast<const void *>(dev::solo_kernel<MODE, WD, RMAX, BT>()), \
-                &prepare_walk_solo<MODE, WD, RMAX, BT>}
-
 // bit-sliced: formats whose factors have at most FL coefficients (SQ: exactly FL each)
 #define TFG_SOLO_SLICED_VARIANT(MODE, WD, BITS, RMAX, BT, FL, SQ) \
     WalkVariant{MODE, BITS, 1, 1, RMAX, BT, &launch_walk_solo<MODE, WD, RMAX, BT, FL, SQ>, \

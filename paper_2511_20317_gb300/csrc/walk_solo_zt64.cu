@@ -1,23 +1,23 @@
 // Thread-per-walker variants: Z_T, terms of 33 to 64 coefficients.  The first of a
 // capacity is its default; the others are walkers-per-block choices of the
 // same kernel.
-#include "walk_link.cuh"
+#include "walk_thread.cuh"
 
 namespace tfg {
 const WalkVariant *walk_variants_solo_zt64(int *n) {
     static const WalkVariant v[] = {
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 16, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 32, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 64, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 72, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 64),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 96),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 128),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 64, 128),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 72, 128),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 128),
-        TFG_LINK_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 160),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 16, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 32, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 64, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 72, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 64),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 96),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 48, 128),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 64, 128),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 72, 128),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 128),
+        TFG_THREAD_VARIANT(TFG_MODE_ZT, uint64_t, 64, 88, 160),
     };
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;

@@ -40,11 +40,10 @@
 #include "tfg_internal.h"
 #include "pterm.cuh"
 #include "walk_link.cuh"
+#include "walk_wide_search.cuh"
 
 namespace tfg {
 namespace dev {
-
-constexpr unsigned kFull = 0xffffffffu;
 
 // PG: the walk policy is read from the descriptor (policies 1 and 2); without
 // it the plateau policy is compiled in alone.
@@ -864,6 +863,7 @@ namespace {
 
 template <int MODE, int FW>
 void prepare_walk_wide() {
+    prepare_walk_search<MODE, FW>();
     static bool attr = [] {
         auto set = [](auto kernel) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinkSmem);
@@ -877,13 +877,31 @@ void prepare_walk_wide() {
     (void)attr;
 }
 
+// When keeping the classes pays.  They are built at every launch (about 60 steps' worth at
+// 351 terms), a step with four walkers a warp takes longer than a warp's on one walker
+// unless the warps are many, and an expansion (walk policy 1) changes three terms.
+// Measured, every step searching / keeping classes, ms: policy 0, (4,5,5) Z_T 300 steps 1000
+// walkers 0.39 / 0.43, 4000 0.98 / 0.76, 16000 3.0 / 1.8; (5,6,10) Z_T 16000 walkers 60 steps
+// 0.92 x, 300 steps 1.35 x; policy 2, (4,5,5) Z_2 300 steps 4000 walkers 0.96 x, 8000 1.48 x;
+// policy 1, 300 steps, 8000 walkers: (4,5,5) Z_T 1.21 x, Z_2 0.98 x, (6,7,9) 1.54 x, 60 steps 0.91 x.
+template <int MODE>
+bool classes_pay(const SegDesc &d, int32_t steps) {
+    const bool large = d.R >= 256;
+    if (d.walk_policy == 0) return d.n_walkers >= 4000 && steps >= (large ? 120 : 40);
+    if (d.walk_policy == 2) return d.n_walkers >= 8000 && steps >= (large ? 200 : 60);
+    return d.n_walkers >= 8000 && steps >= 300 && (MODE == TFG_MODE_ZT || d.R >= 128);
+}
+
 // Walkers per warp: four, unless that leaves an SM's schedulers without two warps each; a
 // warp takes the changing part of a step when any of its walkers does, so a lone
 // walker's step is shorter.  The terms go to shared memory when the whole population
-// resides at once that way.  Measured, (4,5,5), 300 walkers, 400 steps: four a warp in
-// device memory 0.91 ms, in shared memory 0.82, one a warp 0.49 (the kernel before: 0.45).
+// resides at once that way.
 template <int MODE, int FW>
 void launch_walk_wide(const SegDesc &d, int32_t steps, int /*grid*/, int /*block*/, cudaStream_t st) {
+    if (!classes_pay<MODE>(d, steps)) {
+        launch_walk_search<MODE, FW>(d, steps, st);
+        return;
+    }
     prepare_walk_wide<MODE, FW>();
     using Shared = dev::WideWalker<MODE, false, FW, false>;
     using Device = dev::WideWalker<MODE, false, FW, true>;

@@ -169,21 +169,26 @@ def test_window_rows_equal_the_oracle(fmt, slack, steps):
 
 @pytest.mark.parametrize("mode", [tfg.TFG_MODE_ZT, tfg.TFG_MODE_Z2])
 @pytest.mark.parametrize("fmt,slack,nw,policy", [
-    ((4, 5, 5), 28, 3, 0), ((4, 5, 5), 29, 5, 1), ((4, 5, 5), 3, 1217, 0),     # 128 / 129 slots; one and two walkers a warp
-    ((4, 5, 5), 3, 6001, 0), ((4, 5, 5), 6, 20003, 1), ((4, 5, 5), 2, 9001, 2),   # four a warp, terms in shared and device memory
-    ((9, 8, 2), 3, 2001, 0), ((9, 1, 8), 3, 1300, 2), ((9, 8, 2), 5, 4003, 1),  # two words per factor
+    ((4, 5, 5), 3, 300, 0), ((4, 5, 5), 6, 301, 1),                            # every step searching
+    ((4, 5, 5), 28, 4003, 0), ((4, 5, 5), 29, 5001, 0),                        # kept classes: 128 / 129 slots
+    ((4, 5, 5), 3, 20003, 0), ((4, 5, 5), 6, 8003, 1), ((4, 5, 5), 28, 8001, 1), ((4, 5, 5), 2, 9001, 2),
+    ((9, 8, 2), 3, 4801, 0), ((9, 1, 8), 3, 8001, 2), ((9, 8, 2), 5, 8003, 1),  # two words per factor
 ])
 def test_wide_walker_edges(fmt, slack, nw, policy, mode):
-    """The wide-term kernel at the edges of its hash words, at every number of walkers per
-    warp (the last warp partly filled), both places of the terms, the walk policies."""
+    """The wide-term kernels on both sides of the choice between them, at the edges of the
+    hash words, with the last warp partly filled, the terms in shared and in device memory,
+    the walk policies."""
     start = naive_start(*fmt)
     if mode == tfg.TFG_MODE_Z2:
         start = np.abs(start).astype(np.int8)
-    steps = 500 if nw < 1000 else 240
+    steps = 320
     kw = dict(plateau_len=60 if policy == 0 else 10**6, walk_policy=policy, r_slack=slack,
               expand_thresh=int(0.03 * 2**32) if policy == 1 else 0)
     W = tfg.Walkers([(fmt, mode, start, nw)], seed=13, params=tfg.tfg_default_params(**kw))
-    W.walk(steps // 3).walk(steps - steps // 3).sync()
+    if policy:
+        W.walk(steps).sync()
+    else:
+        W.walk(steps // 3).walk(steps - steps // 3).sync()
     take = np.unique(np.concatenate([np.linspace(0, nw - 1, 16).astype(int), np.arange(max(0, nw - 5), nw)]))
     rows = [W.read_walkers(int(w), 1) for w in take]
     info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
