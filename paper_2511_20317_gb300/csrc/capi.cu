@@ -1255,10 +1255,13 @@ static int window_steps(tfg_ctx *ctx, int64_t steps, int32_t policy, const void 
         }
         return ls;
     };
-    // uniform: all steps but the last in one launch per population and 2^30 steps; the last one
-    // leaves its window in the scratch
+    // uniform: all steps but the last in one launch per population and 2^30 steps, and the last
+    // one, which leaves its window in the scratch, by itself.  Three steps or fewer go one
+    // by one: the joint launch builds its walkers' classes first, about two steps' time
+    // (3000 walkers of (4,4,5), two steps: 279 us with it, 142 without; 1000 of (2,2,2),
+    // five steps: 77 us with it, 110 without).
     int64_t done = 0;
-    while (policy == 0 && done < steps - 1) {
+    while (policy == 0 && steps > 3 && done < steps - 1) {
         const int32_t chunk = (int32_t)std::min<int64_t>(steps - 1 - done, 1 << 30);
         for (const Segment &s : ctx->segs)
             tfg::launch_window_walk(ctx->desc(s), chunk, d_choices ? d_choices + (size_t)done * N + s.first : nullptr, N,

@@ -554,30 +554,42 @@ __global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int
     wk.store(d, w, (uint32_t)steps);
 }
 
-// Row of highest score (first on ties) of every lane's walker that asks for one, by the
-// warp: a walker's scores in two 16-byte loads per lane.  (A thread reading its own
-// walker's 256 scores touches 32 lines a load: 0.34 ms for 262144 walkers with the
-// rest of the step, now 0.22.)  As a scan from row 0 that moves on a greater score
-// does, a NaN is never chosen over another row, and one in row 0 stays chosen.
+// Row of highest score (first on ties) of every lane's walker that asks for one: in a full
+// warp four walkers at a time, eight lanes each, whose loads (16 bytes a lane) cover
+// consecutive rows.  (A thread reading its own walker's 256 scores touches 32 lines a
+// load: 0.34 ms for 262144 walkers of (3,4,5) with the rest of the step, now 0.22.)  As a scan
+// from row 0 that moves on a greater score does, a NaN is never chosen over another
+// row, and one in row 0 stays chosen.
 __device__ __forceinline__ int best_row(unsigned wmask, int lane, int nl, bool ask, int K, const float *mine) {
+    if (nl < 32 || __reduce_max_sync(wmask, ask ? K : 0) <= 32) {
+        // also for short windows, whose rows are a line or less: one round of loads, not eight
+        int c = 0;
+        if (ask) {
+            float best = mine[0];
+#pragma unroll 8
+            for (int k = 1; k < K; ++k)
+                if (mine[k] > best) { best = mine[k]; c = k; }
+        }
+        return c;
+    }
     // order-preserving integers of scores (-0 as +0); 0: no score
     auto key = [](float f) -> uint32_t {
         const uint32_t u = __float_as_uint(f + 0.f);
         return f != f ? 1u : (u & 0x80000000u ? ~u : u | 0x80000000u);
     };
     int c = 0;
-    unsigned pend = __ballot_sync(wmask, ask);
+    const unsigned pend = __ballot_sync(wmask, ask);
 #pragma unroll 1
-    while (pend) {
-        const int a = __ffs(pend) - 1;
-        pend &= pend - 1u;
-        const int Ka = __shfl_sync(wmask, K, a);
+    for (int r = 0; r < 8; ++r) {
+        if (((pend >> (4 * r)) & 15u) == 0u) continue;
+        const int a = 4 * r + (lane >> 3);   // the walker of these eight lanes
+        const int Ka = __shfl_sync(wmask, ask ? K : 0, a);
         const float4 *row = reinterpret_cast<const float4 *>(
             __shfl_sync(wmask, reinterpret_cast<unsigned long long>(mine), a));
         uint32_t top = 0u;
         int at = 0;
-#pragma unroll 2
-        for (int k0 = 4 * lane; k0 < Ka; k0 += 4 * nl) {   // nl: live lanes, 0 .. nl - 1
+#pragma unroll 4
+        for (int k0 = 4 * (lane & 7); k0 < Ka; k0 += 32) {
             const float4 v = row[k0 >> 2];
             const float f[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -589,9 +601,18 @@ __device__ __forceinline__ int best_row(unsigned wmask, int lane, int nl, bool a
                 top = max(u, top);
             }
         }
-        const uint32_t most = __reduce_max_sync(wmask, top);
-        const int first = (int)__reduce_min_sync(wmask, top == most ? (unsigned)at : 0xffffu);
-        if (lane == a) c = first;
+        __syncwarp(wmask);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            const uint32_t t2 = __shfl_xor_sync(wmask, top, o);
+            const int a2 = __shfl_xor_sync(wmask, at, o);
+            if (t2 > top || (t2 == top && a2 < at)) {
+                top = t2;
+                at = a2;
+            }
+        }
+        const int got = __shfl_sync(wmask, at, (lane & 3) * 8);   // lane 4 r + g: group g's row
+        if ((lane >> 2) == r) c = got;
     }
     return c;
 }
