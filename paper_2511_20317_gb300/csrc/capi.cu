@@ -1183,13 +1183,10 @@ int tfg_mlp_train_step(void *d_state, void *d_params, const uint16_t *d_x, const
     if (n < 0 || !d_err || (n > 0 && (!d_x || !d_label || !d_weight))) { set_error("bad arguments"); return TFG_EINVAL; }
     if (((uintptr_t)d_x % 16) != 0) { set_error("features must be 16-byte aligned"); return TFG_EINVAL; }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-    if (n == 0) {
-        cudaError_t e = cudaMemsetAsync(s + 3 * P, 0, sizeof(float) * (P + 1), st);
-        if (e != cudaSuccess) return cuda_fail(e, "memset");
-    }
-    // the gradient from per-CTA rows added in CTA order: the same bits on every run
-    tfg::launch_mlp_grad(d_params, d_x, d_label, d_weight, n, s + 3 * P, d_err, st, s + train_partial_offset());
-    tfg::launch_adam(s, s + P, s + 2 * P, s + 3 * P, d_params, lr, step, st);
+    // the gradient from per-CTA rows added in a fixed order: the same bits on every run
+    float *rows = s + train_partial_offset();
+    const int parts = tfg::launch_mlp_grad(d_params, d_x, d_label, d_weight, n, s + 3 * P, d_err, st, rows);
+    tfg::launch_adam(s, s + P, s + 2 * P, s + 3 * P, rows, parts, d_params, lr, step, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "adam launch");
     return TFG_OK;

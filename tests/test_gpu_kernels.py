@@ -198,3 +198,41 @@ def test_wide_walker_edges(fmt, slack, nw, policy, mode):
     assert_parity(info, slots, best, ref, range(take.size), f"{fmt} slack {slack} policy {policy} mode {mode}")
     assert W.verify_all() == 0
     W.close()
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (127, 1), (129, 0), (128 * 152 + 1, 0), (128 * 152 * 2 + 77, 1),
+                                     (128 * 152 * 3 + 5, 0)])
+def test_gradient_tiles_and_warpgroups(n, shift):
+    """Gradient sums at the edges of the tiles and of the two warpgroups' shares, the
+    parameters at a 16-byte or (shift) only 4-byte boundary, single launch and training
+    step, against the float64 reference.  Bound per entry: one bf16 ulp (2^-8) on each
+    operand of every product term, plus FP32 sum error."""
+    import torch
+    from oracle import mlp
+    rng = np.random.default_rng(n)
+    p = mlp.Params.random(rng)
+    x = rng.integers(0, 9, size=(n, mlp.IN)).astype(np.float32)
+    x[:, 24:] = mlp.bf16_round(rng.normal(0, 1, size=(n, mlp.IN - 24)))
+    label = (rng.random(n) < 0.3).astype(np.float32)
+    weight = (rng.random(n) / n).astype(np.float32)
+    y, cache = mlp.forward(p, x)
+    loss, dy = mlp.logistic_loss(y, label, weight)
+    ref = mlp.backward(p, cache, dy, bf16_operands=True)
+    blob = np.frombuffer(p.blob(), dtype=np.uint8)
+    room = torch.zeros(blob.size + 16, dtype=torch.uint8, device="cuda")
+    params = room[4 * shift:4 * shift + blob.size]
+    params.copy_(torch.from_numpy(blob.copy()))
+    xs = torch.from_numpy(mlp.bf16_bits(mlp.bf16_round(x)).view(np.int16).copy()).cuda().view(torch.bfloat16)
+    ls, ws = torch.from_numpy(label).cuda(), torch.from_numpy(weight).cuda()
+    P = tfg.MLP_NUM_PARAMS
+    g, gloss = tfg.tfg_mlp_grad(params, xs, ls, ws)
+    tr = tfg.MlpTrainer(params)
+    tr.step(xs, ls, ws, 0.0)
+    state = tr.state[3 * P:4 * P + 1].cpu().numpy()
+    for vec, total in ((g.cpu().numpy(), gloss), (state[:P], state[P])):
+        assert abs(total - loss) <= 1e-4 * (1 + abs(loss))
+        got = mlp.split_vector(vec.astype(np.float64))
+        for name in ["W1", "W2", "b1", "b2", "w3", "b3"]:
+            bound = 2.0 ** -7 * np.asarray(ref["_abs"][name]) + 1e-6 * (1 + np.abs(ref[name]))
+            diff = np.abs(np.asarray(got[name]) - np.asarray(ref[name]))
+            assert (diff <= bound).all(), (name, float(np.max(diff - bound)))
