@@ -2,7 +2,7 @@
 // tensor cores, shared by the row-scoring kernel (features read from device
 // memory) and the fused window-scoring kernel (features computed in place).
 //
-// A CTA holds the weights once (W1^T and W2^T as K-major BF16 operands, the
+// A CTA holds the weights once (W1 and W2 as MN-major BF16 operands, the
 // vectors in FP32) and runs NWG independent warpgroups.  Warpgroup g owns
 // TMEM columns [128 g, 128 g + 128) (its accumulator), an A tile X (128 rows
 // x 32 features) and an A tile H1 (128 rows x KH hidden inputs) in shared
@@ -22,9 +22,9 @@
 //
 // Bias folding (Prod::kFold, used where the producer controls the feature
 // rows): the constant-one input f31 is joined by f29 = f30 = 1 on every
-// real row, and W1^T's rows 29, 30, 31 hold s = W1[31] + b1 as three BF16
+// real row, and W1's rows 29, 30, 31 hold s = W1[31] + b1 as three BF16
 // pieces (s = hi + mid + lo to FP32 precision), so MMA1 adds the bias; H1
-// gets 16 more columns (KH = 144): three of value one whose W2^T rows hold b2
+// gets 16 more columns (KH = 144): three of value one whose W2 rows hold b2
 // as three BF16 pieces, the rest zero, so MMA2 adds b2.  The epilogues then
 // only apply ReLU (and the w3 dot product).  Features f29 and f30 are zero by
 // definition, so their W1 rows never contribute otherwise; rows past a window
@@ -51,15 +51,16 @@ constexpr uint32_t kParamB2 = kParamB1 + kHid * 4;
 constexpr uint32_t kParamW3 = kParamB2 + kHid * 4;
 constexpr uint32_t kParamB3 = kParamW3 + kHid * 4;
 constexpr uint32_t kParamBytes = kParamB3 + 16;
+constexpr uint32_t kWRow = (kHid / 8) * 128;   // shared bytes of eight rows of a weight matrix
 
-// Shared-memory layout (dynamic part): W1^T, W2^T, the vectors, then per
+// Shared-memory layout (dynamic part): W1, W2, the vectors, then per
 // warpgroup X and H1.  KH = 128, or 144 with the folded b2.
 template <bool FOLD>
 struct Layout {
     static constexpr int KH = FOLD ? kHid + 16 : kHid;
-    static constexpr uint32_t W1T = 0;                            // B of MMA1: 128 (hidden) x 32 (input)
-    static constexpr uint32_t W2T = W1T + kHid * kIn * 2;         // B of MMA2: 128 (out) x KH
-    static constexpr uint32_t Vec = W2T + kHid * KH * 2;          // b1, b2, w3 (w3 only when folded)
+    static constexpr uint32_t W1 = 0;                             // B of MMA1: 32 (input) x 128 (hidden)
+    static constexpr uint32_t W2 = W1 + kHid * kIn * 2;           // B of MMA2: KH x 128 (out)
+    static constexpr uint32_t Vec = W2 + kHid * KH * 2;           // b1, b2, w3 (w3 only when folded)
     static constexpr uint32_t VecBytes = (FOLD ? 1 : 3) * kHid * 4;
     static constexpr uint32_t WG = Vec + VecBytes;                // first warpgroup area
     static constexpr uint32_t X = 0;                              // per warpgroup: X 128 x 32
@@ -122,40 +123,39 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
 
 __device__ __forceinline__ __nv_bfloat16 bf(float v) { return __float2bfloat16_rn(v); }
 
-// Weights and vectors of the parameter blob into the CTA's shared memory.
+// Weights and vectors of the parameter blob into the CTA's shared memory.  W1 and W2 stay
+// row-major (row = input unit), 16 bytes at a time into 8 x 16-byte core matrices: the
+// products read them as MN-major B operands.
 template <bool FOLD>
 __device__ __forceinline__ void load_weights(const uint8_t *__restrict__ params, uint8_t *smem, int tid, int nthr) {
     using LY = Layout<FOLD>;
-    constexpr int KH = LY::KH;
-    const __nv_bfloat16 *W1 = reinterpret_cast<const __nv_bfloat16 *>(params + kParamW1);
-    const __nv_bfloat16 *W2 = reinterpret_cast<const __nv_bfloat16 *>(params + kParamW2);
     const float *b1 = reinterpret_cast<const float *>(params + kParamB1);
     const float *b2 = reinterpret_cast<const float *>(params + kParamB2);
-    uint8_t *sW1T = smem + LY::W1T, *sW2T = smem + LY::W2T;
-    // B operands are K-major: row = output unit, K = input unit
-    for (int e = tid; e < kIn * kHid; e += nthr) {
-        const int i = e / kHid, h = e % kHid;
-        __nv_bfloat16 v = W1[e];
-        if (FOLD && i >= 29) {
-            // rows 29..31: W1[31] + b1 in three bf16 pieces (inputs 29..31 are one)
-            const float s = __bfloat162float(W1[31 * kHid + h]) + b1[h];
-            const float hi = __bfloat162float(bf(s)), mid = __bfloat162float(bf(s - hi));
-            v = i == 31 ? bf(hi) : (i == 30 ? bf(mid) : bf(s - hi - mid));
-        }
-        *reinterpret_cast<__nv_bfloat16 *>(sW1T + tc::kmajor_offset(h, i, kIn)) = v;
-    }
-    for (int e = tid; e < kHid * KH; e += nthr) {
-        const int o = e / KH, h = e % KH;
-        __nv_bfloat16 v;
-        if (h < kHid) {
-            v = W2[h * kHid + o];
+    // consecutive lanes take the eight rows of a core matrix
+    for (int e = tid; e < (kIn + LY::KH) * (kHid / 8); e += nthr) {
+        const int row = ((e >> 7) << 3) | (e & 7), kg = (e >> 3) & 15;   // rows of W1, then of W2
+        uint4 v;
+        if (FOLD && row >= 29 && (row < kIn || row >= kIn + kHid)) {
+            // W1's rows 29..31: W1[31] + b1 in three bf16 pieces (inputs 29..31 are one);
+            // W2's rows 128..130: b2 likewise (H1 columns 128..130 are one), then zeros
+            const int piece = row < kIn ? 31 - row : row - (kIn + kHid);
+            uint32_t h[4];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int c = 8 * kg + k;
+                float f = row < kIn
+                              ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(params)[31 * kHid + c]) + b1[c]
+                              : b2[c];
+                const float hi = __bfloat162float(bf(f)), mid = __bfloat162float(bf(f - hi));
+                f = piece == 0 ? hi : (piece == 1 ? mid : (piece == 2 ? f - hi - mid : 0.f));
+                const uint32_t bits = __bfloat16_as_ushort(bf(f));
+                h[k >> 1] = (k & 1) ? (h[k >> 1] | bits << 16) : bits;
+            }
+            v = make_uint4(h[0], h[1], h[2], h[3]);
         } else {
-            // K rows 128..130: b2 in three bf16 pieces (H1 columns 128..130 are one), then zeros
-            const float s = b2[o];
-            const float hi = __bfloat162float(bf(s)), mid = __bfloat162float(bf(s - hi));
-            v = h == kHid ? bf(hi) : (h == kHid + 1 ? bf(mid) : (h == kHid + 2 ? bf(s - hi - mid) : bf(0.f)));
+            v = *reinterpret_cast<const uint4 *>(params + ((size_t)row * kHid + kg * 8) * 2);
         }
-        *reinterpret_cast<__nv_bfloat16 *>(sW2T + tc::kmajor_offset(o, h, KH)) = v;
+        *reinterpret_cast<uint4 *>(smem + LY::W1 + (row >> 3) * kWRow + kg * 128 + (row & 7) * 16) = v;
     }
     float *vec = reinterpret_cast<float *>(smem + LY::Vec);
     if (FOLD) {
@@ -171,18 +171,16 @@ __device__ __forceinline__ void st_row8(uint8_t *tile, int q, int col0, int K, u
 }
 
 // The pipeline.  Prod (one object per thread; static bool kFold) provides
-//   void begin(int64_t tile, int q)   start loading tile `tile`'s input for row q
+//   bool begin(int q)                 start loading the warpgroup's next tile's input for row q;
+//                                     false: no tile is left (the same answer for the 128 rows)
 //   void mid(int q)                   second load phase of the tile begun last (may be empty)
-//   bool live()                       false: the tile begun last is skipped (the same answer for
-//                                     the 128 rows; asked only when the tile is due, so that its
-//                                     loads have landed)
 //   int64_t fill(uint8_t *sX, int q)  write row q of the tile loaded last into X (kFold:
 //                                     features 29 and 30 one on every real row); returns
 //                                     the row's output index (-1: no output)
 //   void emit(float y, int64_t o)     the score y of the row whose fill returned o
 template <int NWG, class Prod>
-__device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Prod &prod, int64_t ntiles,
-                                          int *__restrict__ err, uint32_t first_limit, uint8_t *smem,
+__device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Prod &prod, int *__restrict__ err,
+                                          uint32_t first_limit, uint8_t *smem,
                                           uint64_t *mbar, uint32_t *tslot, int *timeout_flag) {
     constexpr bool FOLD = Prod::kFold;
     using LY = Layout<FOLD>;
@@ -209,32 +207,21 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
     const uint32_t tlane = tacc + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t mb = tc::smem_u32(&mbar[g]);
     const uint32_t aX = tc::smem_u32(sX), aH1 = tc::smem_u32(sH1);
-    const uint32_t aW1 = tc::smem_u32(smem + LY::W1T), aW2 = tc::smem_u32(smem + LY::W2T);
+    const uint32_t aW1 = tc::smem_u32(smem + LY::W1), aW2 = tc::smem_u32(smem + LY::W2);
     const float *vec = reinterpret_cast<const float *>(smem + LY::Vec);
-    const float *sB1 = vec, *sB2 = vec + kHid, *sW3 = FOLD ? vec : vec + 2 * kHid;
+    const int lane = tid & 31;
+    const float2 *sB1 = reinterpret_cast<const float2 *>(vec) + (lane & 3);   // b1, b2, w3, not folded: this lane's columns
     const float b3 = *reinterpret_cast<const float *>(params + kParamB3);
-    constexpr uint32_t idesc = tc::idesc_bf16_f32(kTile, kHid);
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(kTile, kHid) | tc::kMnMajorB;
     uint32_t phase = 0;
     bool timed_out = false, first_wait = true;
 
-    const int64_t stride = (int64_t)gridDim.x * NWG;
-    int64_t t = (int64_t)blockIdx.x * NWG + g;
-    // the first live tile, its features in X
-    if (t < ntiles) {
-        prod.begin(t, q);
-        prod.mid(q);
-    }
-    while (t < ntiles && !prod.live()) {   // skipped tile (uniform over the warpgroup)
-        t += stride;
-        if (t < ntiles) {
-            prod.begin(t, q);
-            prod.mid(q);
-        }
-    }
-    int64_t out_cur = t < ntiles ? prod.fill(sX, q) : -1;
-    while (t < ntiles) {
-        int64_t tn = t + stride;
-        if (tn < ntiles) prod.begin(tn, q);   // first load phase of the next tile
+    // the first tile, its features in X
+    bool has = prod.begin(q);
+    if (has) prod.mid(q);
+    int64_t out_cur = has ? prod.fill(sX, q) : -1;
+    while (has) {
+        const bool more = prod.begin(q);   // first load phase of the next tile
         tc::fence_async_smem();
         tc::fence_before_sync();
         wg_sync(g);
@@ -243,7 +230,7 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
 #pragma unroll
             for (int kc = 0; kc < kIn / 16; ++kc)
                 tc::mma_bf16(tacc, tc::make_desc(aX + kc * 256, 128, (kIn / 8) * 128),
-                             tc::make_desc(aW1 + kc * 256, 128, (kIn / 8) * 128), idesc, kc > 0);
+                             tc::make_desc(aW1 + kc * 2 * kWRow, kWRow, 128), idesc, kc > 0);
             tc::mma_commit(mb);
         }
         bool ok = tc::mbar_wait(mb, phase, first_wait ? first_limit : tc::kWaitLimit);
@@ -251,8 +238,8 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
         if (wg_any(g, !ok)) { timed_out = true; break; }
         phase ^= 1;
         tc::fence_after_sync();
-        // ---- epi1: h1 = bf16(relu(z1 + b1)) -> H1 (row q), TMEM chunks of 16 one ahead
-        {
+        // ---- epi1: h1 = bf16(relu(z1 + b1)) -> H1
+        if constexpr (FOLD) {   // row q, TMEM chunks of 16 columns one ahead
             uint32_t ra[16], rb[16];
             tmem_ld16_nowait(tlane, ra);
             tmem_wait(ra);
@@ -265,18 +252,26 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
                 for (int u = 0; u < 16; u += 8) {
                     float f[8];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        f[k] = __uint_as_float(cur[u + k]);
-                        if (!FOLD) f[k] += sB1[16 * c + u + k];
-                    }
+                    for (int k = 0; k < 8; ++k) f[k] = __uint_as_float(cur[u + k]);
                     st_row8(sH1, q, 16 * c + u, KH,
                             make_uint4(pack_relu_bf16x2(f[0], f[1]), pack_relu_bf16x2(f[2], f[3]),
                                        pack_relu_bf16x2(f[4], f[5]), pack_relu_bf16x2(f[6], f[7])));
                 }
                 if (c + 1 < kHid / 16) tmem_wait(nxt);
             }
+        } else {   // blocks of 16 rows x 32 columns: a lane's bias serves four rows
+            tc::for_blocks(tlane, [&](int c, int h, uint32_t(&r)[16]) {
+                float v[16];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 b = sB1[16 * c + 4 * j];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) v[4 * j + e] = __uint_as_float(r[4 * j + e]) + ((e & 1) ? b.y : b.x);
+                }
+                tc::st_block<true>(aH1, lane, (q & 96) + 16 * h, c, v);
+            });
         }
-        if (tn < ntiles) prod.mid(q);   // second load phase of the next tile
+        if (more) prod.mid(q);   // second load phase of the next tile
         tc::fence_async_smem();
         tc::fence_before_sync();
         wg_sync(g);
@@ -285,25 +280,18 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
 #pragma unroll
             for (int kc = 0; kc < KH / 16; ++kc)
                 tc::mma_bf16(tacc, tc::make_desc(aH1 + kc * 256, 128, (KH / 8) * 128),
-                             tc::make_desc(aW2 + kc * 256, 128, (KH / 8) * 128), idesc, kc > 0);
+                             tc::make_desc(aW2 + kc * 2 * kWRow, kWRow, 128), idesc, kc > 0);
             tc::mma_commit(mb);
         }
-        // while MMA2 runs: the next live tile's features into X (MMA1, its only reader, is done)
-        while (tn < ntiles && !prod.live()) {
-            tn += stride;
-            if (tn < ntiles) {
-                prod.begin(tn, q);
-                prod.mid(q);
-            }
-        }
-        const int64_t out_next = tn < ntiles ? prod.fill(sX, q) : -1;
+        // while MMA2 runs: the next tile's features into X (MMA1, its only reader, is done)
+        const int64_t out_next = more ? prod.fill(sX, q) : -1;
         ok = tc::mbar_wait(mb, phase);
         if (wg_any(g, !ok)) { timed_out = true; break; }
         phase ^= 1;
         tc::fence_after_sync();
         // ---- epi2: y = b3 + w3 . relu(z2 + b2)
-        float2 y2 = make_float2(b3, 0.f);
-        {
+        if constexpr (FOLD) {
+            float2 y2 = make_float2(b3, 0.f);
             uint32_t ra[16], rb[16];
             tmem_ld16_nowait(tlane, ra);
             tmem_wait(ra);
@@ -314,26 +302,45 @@ __device__ __forceinline__ void run_tiles(const uint8_t *__restrict__ params, Pr
                 if (c + 1 < kHid / 16) tmem_ld16_nowait(tlane + 16 * (c + 1), nxt);
 #pragma unroll
                 for (int u = 0; u < 16; u += 4) {
-                    const float4 w = *reinterpret_cast<const float4 *>(sW3 + 16 * c + u);
-                    float z0 = __uint_as_float(cur[u]), z1 = __uint_as_float(cur[u + 1]);
-                    float z2 = __uint_as_float(cur[u + 2]), z3 = __uint_as_float(cur[u + 3]);
-                    if (!FOLD) {
-                        const float4 b = *reinterpret_cast<const float4 *>(sB2 + 16 * c + u);
-                        const float2 s01 = __fadd2_rn(make_float2(z0, z1), make_float2(b.x, b.y));
-                        const float2 s23 = __fadd2_rn(make_float2(z2, z3), make_float2(b.z, b.w));
-                        z0 = s01.x; z1 = s01.y; z2 = s23.x; z3 = s23.y;
-                    }
+                    const float4 w = *reinterpret_cast<const float4 *>(vec + 16 * c + u);
+                    const float z0 = __uint_as_float(cur[u]), z1 = __uint_as_float(cur[u + 1]);
+                    const float z2 = __uint_as_float(cur[u + 2]), z3 = __uint_as_float(cur[u + 3]);
                     y2 = __ffma2_rn(make_float2(fmaxf(z0, 0.f), fmaxf(z1, 0.f)), make_float2(w.x, w.y), y2);
                     y2 = __ffma2_rn(make_float2(fmaxf(z2, 0.f), fmaxf(z3, 0.f)), make_float2(w.z, w.w), y2);
                 }
                 if (c + 1 < kHid / 16) tmem_wait(nxt);
             }
+            prod.emit(y2.x + y2.y, out_cur);
+        } else {
+            float2 ys[4];   // rows lane / 4 + 8 k of the warp's 32, this lane's 32 columns
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ys[k] = make_float2(0.f, 0.f);
+            tc::for_blocks(tlane, [&](int c, int h, uint32_t(&r)[16]) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 b = sB1[kHid / 2 + 16 * c + 4 * j], w = sB1[kHid + 16 * c + 4 * j];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const float2 z = __fadd2_rn(
+                            make_float2(__uint_as_float(r[4 * j + 2 * k]), __uint_as_float(r[4 * j + 2 * k + 1])), b);
+                        ys[2 * h + k] = __ffma2_rn(make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)), w, ys[2 * h + k]);
+                    }
+                }
+            });
+            float y = 0.f;   // lane l sums row l / 4 + 8 (l % 4) over its four lanes
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float t = ys[k].x + ys[k].y;
+                t += __shfl_xor_sync(0xffffffffu, t, 1);
+                t += __shfl_xor_sync(0xffffffffu, t, 2);
+                y = (lane & 3) == k ? t : y;
+            }
+            prod.emit(b3 + y, __shfl_sync(0xffffffffu, out_cur, (lane >> 2) + 8 * (lane & 3)));
         }
-        prod.emit(y2.x + y2.y, out_cur);
         // the next MMA1 overwrites the accumulator: order this thread's loads before it
         tc::fence_before_sync();
         out_cur = out_next;
-        t = tn;
+        has = more;
     }
     if (timed_out) {
         // the awaited products may still be in flight: one more bounded wait before release

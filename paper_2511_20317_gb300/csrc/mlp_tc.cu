@@ -23,11 +23,13 @@ struct RowsProducer {
     const __nv_bfloat16 *x;
     int64_t n;
     float *out;
+    int64_t tile, tiles;   // the next one, their number
     uint4 v[4];
     int64_t row_loaded;
-    __device__ __forceinline__ bool live() const { return true; }
-    __device__ __forceinline__ void begin(int64_t tile, int q) {
+    __device__ __forceinline__ bool begin(int q) {
+        if (tile >= tiles) return false;
         row_loaded = tile * mlp::kTile + q;
+        tile += (int64_t)gridDim.x * kWG;
 #pragma unroll
         for (int c = 0; c < 4; ++c) v[c] = make_uint4(0, 0, 0, 0);
         if (row_loaded < n) {
@@ -35,6 +37,7 @@ struct RowsProducer {
 #pragma unroll
             for (int c = 0; c < 4; ++c) v[c] = src[c];
         }
+        return true;
     }
     __device__ __forceinline__ void mid(int) {}
     __device__ __forceinline__ int64_t fill(uint8_t *sX, int q) {
@@ -59,8 +62,9 @@ __global__ void __launch_bounds__(kWG * 128, 1) mlp_score_kernel(const uint8_t *
     p.x = x;
     p.n = n;
     p.out = out;
-    mlp::run_tiles<kWG>(params, p, (n + mlp::kTile - 1) / mlp::kTile, err, first_limit, smem, mbar, &tslot,
-                        &tflag);
+    p.tile = (int64_t)blockIdx.x * kWG + (threadIdx.x >> 7);
+    p.tiles = (n + mlp::kTile - 1) / mlp::kTile;
+    mlp::run_tiles<kWG>(params, p, err, first_limit, smem, mbar, &tslot, &tflag);
 }
 
 uint32_t g_first_wait_limit = tc::kWaitLimit;

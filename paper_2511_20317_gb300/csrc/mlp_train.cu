@@ -56,64 +56,11 @@ constexpr uint32_t kSH = kSD + kWGs * kTile * kHid * 2; // per warpgroup (s, h) 
 constexpr uint32_t kSX = kSH + kWGs * kTile * kHid * 2; // per warpgroup two of (s, i) = X
 constexpr uint32_t kSVec = kSX + kWGs * 2 * kTile * kIn * 2;   // 0 - b1, b2, w3
 constexpr uint32_t kTrainSmem = kSVec + 3 * kHid * 4;
-constexpr uint32_t kHidRow = (kHid / 8) * 128;   // bytes of eight rows of a tile 128 columns wide
+constexpr uint32_t kHidRow = tc::kBlockRow;      // bytes of eight rows of a tile 128 columns wide
 constexpr uint32_t kInRow = (kIn / 8) * 128;     // of one 32 columns wide
 
 // tensor memory: the warpgroups' accumulators at 0 and 128, dW2^T, dW1^T
 constexpr uint32_t kTmemCols = 512, kTmemDW2 = kWGs * 128, kTmemDW1 = kTmemDW2 + 128;
-
-// 32 columns x 16 rows of an accumulator: registers 4 j + {0, 1} hold columns 8 j + 2 (lane % 4)
-// + {0, 1} of row lane / 4, registers 4 j + {2, 3} those of row lane / 4 + 8.
-__device__ __forceinline__ void tmem_ld_block(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    asm volatile(""
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
-                   "+r"(r[14]), "+r"(r[15]));
-}
-
-// f(c, h, r) for the eight blocks of a warp's 32 rows (half h) x 128 columns (32 c), each block's
-// load issued before the work on the one before it.
-template <class F>
-__device__ __forceinline__ void for_blocks(uint32_t tacc, F &&f) {
-    uint32_t ra[16], rb[16];
-    tmem_ld_block(tacc, ra);
-    tmem_ld_wait(ra);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        uint32_t(&cur)[16] = (b & 1) ? rb : ra;
-        uint32_t(&nxt)[16] = (b & 1) ? ra : rb;
-        if (b < 7) tmem_ld_block(tacc + ((uint32_t)(((b + 1) & 1) * 16) << 16) + 32 * ((b + 1) >> 1), nxt);
-        f(b >> 1, b & 1, cur);
-        if (b < 7) tmem_ld_wait(nxt);
-    }
-}
-
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-// A block (as tmem_ld_block's, values v) as BF16 into rows row0 .. row0 + 15 (a multiple of 8),
-// columns 32 c .. 32 c + 31 of a 128-column tile: eight core matrices.
-__device__ __forceinline__ void st_block(uint32_t tile, int lane, int row0, int c, const float (&v)[16]) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const uint32_t at = tile + (uint32_t)(row0 / 8 + k) * kHidRow + (uint32_t)c * 512 + (uint32_t)lane * 16;
-        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at),
-                     "r"(pack2(v[2 * k], v[2 * k + 1])), "r"(pack2(v[4 + 2 * k], v[5 + 2 * k])),
-                     "r"(pack2(v[8 + 2 * k], v[9 + 2 * k])), "r"(pack2(v[12 + 2 * k], v[13 + 2 * k]))
-                     : "memory");
-    }
-}
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool full) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
@@ -185,10 +132,9 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
 
     if (warp == kWGs * 4) {
         if (lane == 0) {
-            constexpr uint32_t kTransA = 1u << 15, kTransB = 1u << 16;   // MN-major operands
-            constexpr uint32_t id_z = tc::idesc_bf16_f32(128, 128) | kTransB, id_h = tc::idesc_bf16_f32(128, 128),
-                               id_w2 = tc::idesc_bf16_f32(128, 128) | kTransA | kTransB,
-                               id_w1 = tc::idesc_bf16_f32(128, 32) | kTransA | kTransB;
+            constexpr uint32_t id_z = tc::idesc_bf16_f32(128, 128) | tc::kMnMajorB, id_h = tc::idesc_bf16_f32(128, 128),
+                               id_w2 = tc::idesc_bf16_f32(128, 128) | tc::kMnMajorA | tc::kMnMajorB,
+                               id_w1 = tc::idesc_bf16_f32(128, 32) | tc::kMnMajorA | tc::kMnMajorB;
             uint32_t phase = 0;   // bit g: parity of the next readiness of warpgroup g
             bool ok = true, first_w2 = true, first_w1 = true;
             auto ready = [&](int g) {
@@ -300,7 +246,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
             // ---- layer 1: h1 = relu(z1 + b1) as BF16; bits of z1 > 0.  As -z: its minimum with +0
             // has the sign bit exactly where z > 0.
             uint32_t mask[4] = {0u, 0u, 0u, 0u};
-            for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
+            tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
                 float v[16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -312,7 +258,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                         v[4 * j + e] = -t;
                     }
                 }
-                st_block(H, lane, wq * 32 + h * 16, c, v);
+                tc::st_block<false>(H, lane, wq * 32 + h * 16, c, v);
             });
             publish();
             if (!(ok = wait())) break;
@@ -320,7 +266,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
             float2 ys[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) ys[q] = make_float2(0.f, 0.f);
-            for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
+            tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float2 b = B2[16 * c + 4 * j], w = W3[16 * c + 4 * j];
@@ -349,7 +295,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
 #pragma unroll
             for (int q = 0; q < 4; ++q) dy[q] = __shfl_sync(0xffffffffu, dy1, (lane & 28) | q);
             // dz2 = dy w3 relu'(z2); sums for w3 and b2
-            for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
+            tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
                 float v[16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -370,12 +316,12 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                         v[4 * j + 2 * q + 1] = on.y * w.y;
                     }
                 }
-                st_block(D, lane, wq * 32 + h * 16, c, v);
+                tc::st_block<false>(D, lane, wq * 32 + h * 16, c, v);
             });
             publish();
             if (!(ok = wait())) break;
             // ---- dz1 = dH1 relu'(z1) over dZ2; sums for b1
-            for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
+            tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
                 float v[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {   // bit 31 - (16 h + e) of mask[c]
@@ -383,7 +329,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                     const int a = 8 * c + 2 * (e >> 2) + (e & 1);
                     gb1[a] += v[e];
                 }
-                st_block(D, lane, wq * 32 + h * 16, c, v);
+                tc::st_block<false>(D, lane, wq * 32 + h * 16, c, v);
             });
             cp_async_wait();   // the next tile's rows
             publish();

@@ -38,6 +38,10 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint
     return d;
 }
 
+// An operand read MN-major takes the same core matrices of a row-major tile whose rows run
+// along K: its leading byte offset is the distance between 8-row groups, its stride byte
+// offset that between 8-column groups (128 B).
+constexpr uint32_t kMnMajorA = 1u << 15, kMnMajorB = 1u << 16;   // bits of the instruction descriptor
 // Instruction descriptor of kind::f16: D = F32, A = B = BF16, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -107,6 +111,63 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(r[c]);
+}
+
+// 32 columns x 16 rows of an accumulator: registers 4 j + {0, 1} hold columns 8 j + 2 (lane % 4)
+// + {0, 1} of row lane / 4, registers 4 j + {2, 3} those of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_block(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    asm volatile(""
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                   "+r"(r[14]), "+r"(r[15]));
+}
+
+// f(c, h, r) for the eight blocks of a warp's 32 rows (half h) x 128 columns (32 c), each block's
+// load issued before the work on the one before it.
+template <class F>
+__device__ __forceinline__ void for_blocks(uint32_t tacc, F &&f) {
+    uint32_t ra[16], rb[16];
+    tmem_ld_block(tacc, ra);
+    tmem_ld_wait(ra);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        uint32_t(&cur)[16] = (b & 1) ? rb : ra;
+        uint32_t(&nxt)[16] = (b & 1) ? ra : rb;
+        if (b < 7) tmem_ld_block(tacc + ((uint32_t)(((b + 1) & 1) * 16) << 16) + 32 * ((b + 1) >> 1), nxt);
+        f(b >> 1, b & 1, cur);
+        if (b < 7) tmem_ld_wait(nxt);
+    }
+}
+
+template <bool RELU>
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    uint32_t r;
+    if (RELU) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// A block (as tmem_ld_block's, values v; RELU: negative ones as zero) as BF16 into rows row0 .. row0 + 15 (a multiple of 8),
+// columns 32 c .. 32 c + 31 of a 128-column tile: eight core matrices.
+constexpr uint32_t kBlockRow = 16 * 128;   // bytes of eight rows of the tile
+template <bool RELU>
+__device__ __forceinline__ void st_block(uint32_t tile, int lane, int row0, int c, const float (&v)[16]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t at = tile + (uint32_t)(row0 / 8 + k) * kBlockRow + (uint32_t)c * 512 + (uint32_t)lane * 16;
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at),
+                     "r"(pack2<RELU>(v[2 * k], v[2 * k + 1])), "r"(pack2<RELU>(v[4 + 2 * k], v[5 + 2 * k])),
+                     "r"(pack2<RELU>(v[8 + 2 * k], v[9 + 2 * k])), "r"(pack2<RELU>(v[12 + 2 * k], v[13 + 2 * k]))
+                     : "memory");
+    }
 }
 
 }  // namespace tc

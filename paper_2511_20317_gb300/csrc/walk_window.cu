@@ -313,16 +313,19 @@ __global__ void __launch_bounds__(128) window_kernel(const SegDesc d, __nv_bfloa
     else window_of<Wd, 1>(d, w, lane, st[warp], srow[warp], feat, desc, kwin);
 }
 
-// Producer of the fused scoring kernel: tile t is half t & 1 (rows 0-127 or
-// 128-255) of walker t >> 1's window; thread q computes the features of row
-// 128 (t & 1) + q from its descriptor and the walker's two slots, straight
-// into the A tile.  A second half with no candidate is skipped; rows past the
-// window get zero features and no score.  Loads in two phases, so that no
-// load waits on another while the previous tile runs: begin() the window size,
-// the row's descriptor and the walker's rank (every row's descriptor word is
-// read; a row past the window holds a stale or undefined one, so its slot
-// indices are clamped), mid() the two slots the descriptor names; the skip
-// decision (live) is taken when the tile is due.
+// Producer of the fused scoring kernel.  A warpgroup takes a contiguous share of the half
+// windows (unit 2 w + half: rows 0-127 or 128-255 of walker w) and lays their rows end to
+// end in groups of 32, the last group of a window ragged: warp j of its tile k takes
+// group 4 k + j.  (A tile for every half left a fifth to a quarter of the rows empty:
+// 262144 walkers of (3,4,5), windows of about 180 rows, @SCORE@.)
+// A lane holds the window size of one unit of 32 and the running count of their
+// groups; the next 32 sizes are loaded a chunk ahead.  A thread computes the features of
+// its row from the row's descriptor and the walker's two slots, straight into the A
+// tile; rows past the window get zero features and no score.  Loads in two
+// phases, so that none waits on another while the previous tile runs: begin() the row's
+// descriptor and the walker's rank (every row's descriptor word is read; a row past
+// the window holds a stale or undefined one, so its slot indices are clamped), mid()
+// the two slots the descriptor names.
 template <class Wd>
 struct WindowProducer {
     static constexpr bool kFold = true;   // the producer writes features 29, 30 = 1: biases in the MMAs
@@ -333,21 +336,64 @@ struct WindowProducer {
     const int *kwin;
     float *score;
     Masks<Wd, 1> mk;
+    // the warpgroup's units: those of this chunk of 32 start at base, the next one's at next
+    int64_t base, next, end;
+    int size, size_next, upto, total;   // this lane's unit: window size, groups up to and with it; all groups
+    int first;                          // the next tile's first group, counted from the chunk's
     // loaded by begin() / mid()
     int64_t w;
-    int row, half, K, r, best_r;
+    int row, K, r, best_r;
     uint2 dci;
     PTerm<Wd, 1, true> ti, tj;
-    __device__ __forceinline__ void begin(int64_t tile, int q) {
-        w = tile >> 1;
-        half = (int)(tile & 1);
-        row = half * kWin / 2 + q;
-        K = kwin[w];
+    __device__ __forceinline__ int groups(int64_t u, int k) const {   // of unit u, window size k
+        const int left = k - (int)(u & 1) * (kWin / 2);
+        return left <= 0 ? 0 : min((left + 31) / 32, kWin / 64);
+    }
+    __device__ __forceinline__ int size_at(int64_t u) const { return u < end ? kwin[u >> 1] : 0; }
+    __device__ __forceinline__ void share(int64_t units, int64_t part, int64_t parts) {
+        base = next = units * part / parts;
+        end = units * (part + 1) / parts;
+        size_next = size_at(next + (threadIdx.x & 31));
+        total = first = 0;
+    }
+    // the next chunk of units
+    __device__ __forceinline__ void advance(int lane) {
+        first -= total;
+        base = next;
+        next += 32;
+        size = size_next;
+        size_next = size_at(next + lane);
+        upto = groups(base + lane, size);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int below = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += below;
+        }
+        total = __shfl_sync(0xffffffffu, upto, 31);
+    }
+    __device__ __forceinline__ bool begin(int q) {
+        const int lane = q & 31;
+        while (first >= total && next < end) advance(lane);
+        if (first >= total) return false;
+        while (first + (q >> 5) >= total && next < end) advance(lane);   // this warp's group
+        const int mine = first + (q >> 5);
+        first += 4;
+        // the unit that holds it (none: past the last one)
+        const int src = min(__popc(__ballot_sync(0xffffffffu, upto <= mine)), 31);
+        const int64_t u = base + src;
+        K = mine < total ? __shfl_sync(0xffffffffu, size, src) : 0;
+        row = (int)(u & 1) * (kWin / 2) + 32 * (mine - __shfl_sync(0xffffffffu, upto, src) + groups(u, K)) + lane;
+        if (mine >= total) {
+            row = 0;
+            w = base >> 1;
+        } else {
+            w = u >> 1;
+        }
         dci = desc[(size_t)w * kWin + row];
         r = hdr[w].r;
         best_r = hdr[w].best_r;
+        return true;
     }
-    __device__ __forceinline__ bool live() const { return !(half && K <= kWin / 2); }
     __device__ __forceinline__ void mid(int) {
         const int i = min((int)(dci.x & 1023u), R - 1), j = min((int)((dci.x >> 12) & 1023u), R - 1);
         const Wd *src = slots + (size_t)w * R * 2;
@@ -398,7 +444,8 @@ __global__ void __launch_bounds__(kScoreWG * 128, 1)
     pr.kwin = kwin;
     pr.score = score;
     pr.mk.load(d);
-    mlp::run_tiles<kScoreWG>(params, pr, d.n_walkers * 2, err, first_limit, smem, mbar, &tslot, &tflag);
+    pr.share(d.n_walkers * 2, (int64_t)blockIdx.x * kScoreWG + (threadIdx.x >> 7), (int64_t)gridDim.x * kScoreWG);
+    mlp::run_tiles<kScoreWG>(params, pr, err, first_limit, smem, mbar, &tslot, &tflag);
 }
 
 // Log entry `slot` := (features, label, walker id, step).
