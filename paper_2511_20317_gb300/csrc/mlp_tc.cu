@@ -1,7 +1,7 @@
 // Learned flip proposal: the scoring MLP 32 -> 128 -> 128 -> 1 (ReLU) on the
 // 5th-generation tensor cores for rows of features in device memory
 // (tfg_mlp_score).  The tile pipeline (mlp_pipe.cuh) runs four warpgroups per
-// CTA, one CTA per SM; each thread loads its row of the next tile while the
+// CTA, one CTA per SM; each thread loads its part of the next tile while the
 // current tile's products run.
 //
 // Parameter blob (device, see include/tfg.h): W1 bf16 [32][128], W2 bf16
@@ -17,33 +17,35 @@ namespace {
 
 constexpr int kWG = 4;
 
-// Rows of features from device memory (bf16 [n][32]); rows past n are zero.
+// Rows of features from device memory (bf16 [n][32]); rows past n are zero.  Eight lanes
+// load the eight rows of a core matrix (a warp reads 512 bytes in a row), a tile ahead.
 struct RowsProducer {
-    static constexpr bool kFold = false;   // arbitrary rows: the biases are added in the epilogues
+    static constexpr bool kFold = false;   // arbitrary rows
     const __nv_bfloat16 *x;
     int64_t n;
     float *out;
     int64_t tile, tiles;   // the next one, their number
+    int64_t row0;          // of the tile begun last
     uint4 v[4];
-    int64_t row_loaded;
     __device__ __forceinline__ bool begin(int q) {
         if (tile >= tiles) return false;
-        row_loaded = tile * mlp::kTile + q;
+        row0 = tile * mlp::kTile;
         tile += (int64_t)gridDim.x * kWG;
+        const int lane = q & 31;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = make_uint4(0, 0, 0, 0);
-        if (row_loaded < n) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(x + row_loaded * mlp::kIn);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = src[c];
+        for (int k = 0; k < 4; ++k) {
+            const int64_t row = row0 + ((q >> 5) * 4 + k) * 8 + (lane & 7);
+            v[k] = make_uint4(0, 0, 0, 0);
+            if (row < n) v[k] = *reinterpret_cast<const uint4 *>(x + row * mlp::kIn + (lane >> 3) * 8);
         }
         return true;
     }
     __device__ __forceinline__ void mid(int) {}
     __device__ __forceinline__ int64_t fill(uint8_t *sX, int q) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) mlp::st_row8(sX, q, 8 * c, mlp::kIn, v[c]);
-        return row_loaded < n ? row_loaded : -1;
+        for (int k = 0; k < 4; ++k)
+            *reinterpret_cast<uint4 *>(sX + ((q >> 5) * 4 + k) * ((mlp::kIn / 8) * 128) + (q & 31) * 16) = v[k];
+        return row0 + q < n ? row0 + q : -1;
     }
     __device__ __forceinline__ void emit(float y, int64_t o) {
         if (o >= 0) out[o] = y;

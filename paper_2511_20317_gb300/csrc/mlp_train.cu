@@ -62,10 +62,6 @@ constexpr uint32_t kInRow = (kIn / 8) * 128;     // of one 32 columns wide
 // tensor memory: the warpgroups' accumulators at 0 and 128, dW2^T, dW1^T
 constexpr uint32_t kTmemCols = 512, kTmemDW2 = kWGs * 128, kTmemDW1 = kTmemDW2 + 128;
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool full) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar_saddr) {
     asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(mbar_saddr) : "memory");
 }
@@ -226,13 +222,13 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                 const int rg = wq * 4 + i;
                 const int64_t row = row0 + rg * 8 + (lane & 7);
                 const bool in = row < n;
-                cp_async16(X + rg * kInRow + lane * 16, x + (in ? row * kIn + (lane >> 3) * 8 : 0), in);
+                tc::cp_async16(X + rg * kInRow + lane * 16, x + (in ? row * kIn + (lane >> 3) * 8 : 0), in);
             }
         };
         bool ok = true;
         if (own > 0) {
             load_x(0);
-            cp_async_wait();
+            tc::cp_async_wait();
             publish();
         }
         for (int64_t k = 0; k < own; ++k) {
@@ -246,14 +242,15 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
             // ---- layer 1: h1 = relu(z1 + b1) as BF16; bits of z1 > 0.  As -z: its minimum with +0
             // has the sign bit exactly where z > 0.
             uint32_t mask[4] = {0u, 0u, 0u, 0u};
+            float2 b[4], w[4];   // a chunk's biases and weights, kept for the lower rows
             tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
                 float v[16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 nb = nB1[16 * c + 4 * j];
+                    if (h == 0) b[j] = nB1[16 * c + 4 * j];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const float t = fminf(((e & 1) ? nb.y : nb.x) - __uint_as_float(r[4 * j + e]), 0.f);
+                        const float t = fminf(((e & 1) ? b[j].y : b[j].x) - __uint_as_float(r[4 * j + e]), 0.f);
                         mask[c] = __funnelshift_l(__float_as_uint(t), mask[c], 1);
                         v[4 * j + e] = -t;
                     }
@@ -269,12 +266,12 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
             tc::for_blocks(tacc, [&](int c, int h, uint32_t(&r)[16]) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 b = B2[16 * c + 4 * j], w = W3[16 * c + 4 * j];
+                    if (h == 0) b[j] = B2[16 * c + 4 * j], w[j] = W3[16 * c + 4 * j];
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const float2 z = __fadd2_rn(
-                            make_float2(__uint_as_float(r[4 * j + 2 * q]), __uint_as_float(r[4 * j + 2 * q + 1])), b);
-                        ys[2 * h + q] = __ffma2_rn(make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)), w, ys[2 * h + q]);
+                            make_float2(__uint_as_float(r[4 * j + 2 * q]), __uint_as_float(r[4 * j + 2 * q + 1])), b[j]);
+                        ys[2 * h + q] = __ffma2_rn(make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)), w[j], ys[2 * h + q]);
                     }
                 }
             });
@@ -299,12 +296,12 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                 float v[16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 b = B2[16 * c + 4 * j], w = W3[16 * c + 4 * j];
+                    if (h == 0) b[j] = B2[16 * c + 4 * j], w[j] = W3[16 * c + 4 * j];
                     const int a = 8 * c + 2 * j;
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const float2 z = __fadd2_rn(
-                            make_float2(__uint_as_float(r[4 * j + 2 * q]), __uint_as_float(r[4 * j + 2 * q + 1])), b);
+                            make_float2(__uint_as_float(r[4 * j + 2 * q]), __uint_as_float(r[4 * j + 2 * q + 1])), b[j]);
                         const float d = dy[2 * h + q];
                         const float2 on = make_float2(z.x > 0.f ? d : 0.f, z.y > 0.f ? d : 0.f);
                         const float2 gw = __ffma2_rn(make_float2(d, d), make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)),
@@ -312,8 +309,8 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                         const float2 gm = __fadd2_rn(make_float2(gm2[a], gm2[a + 1]), on);
                         gw3[a] = gw.x; gw3[a + 1] = gw.y;
                         gm2[a] = gm.x; gm2[a + 1] = gm.y;
-                        v[4 * j + 2 * q] = on.x * w.x;
-                        v[4 * j + 2 * q + 1] = on.y * w.y;
+                        v[4 * j + 2 * q] = on.x * w[j].x;
+                        v[4 * j + 2 * q + 1] = on.y * w[j].y;
                     }
                 }
                 tc::st_block<false>(D, lane, wq * 32 + h * 16, c, v);
@@ -331,10 +328,10 @@ __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_kernel(
                 }
                 tc::st_block<false>(D, lane, wq * 32 + h * 16, c, v);
             });
-            cp_async_wait();   // the next tile's rows
+            tc::cp_async_wait();   // the next tile's rows
             publish();
         }
-        cp_async_wait();
+        tc::cp_async_wait();
         if (!ok) timeout = 1;
     }
     tc::fence_before_sync();

@@ -113,8 +113,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(r[c]);
 }
 
+// 16 bytes from global to shared memory (zeros unless full), and the wait for all of a thread's.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool full) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // 32 columns x 16 rows of an accumulator: registers 4 j + {0, 1} hold columns 8 j + 2 (lane % 4)
-// + {0, 1} of row lane / 4, registers 4 j + {2, 3} those of row lane / 4 + 8.
+// + {0, 1} of row lane / 4, registers 4 j + {2, 3} those of row lane / 4 + 8.  (Measured, 16
+// warps an SM: such a load every 32 cycles and scheduler; one of 16 columns of a lane's own
+// row, the 32x32b shape, every 9.)
 __device__ __forceinline__ void tmem_ld_block(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.16x256b.x4.b32 "

@@ -41,60 +41,74 @@ __device__ __forceinline__ int popc_w(Wd v) {
     else return __popcll(v);
 }
 
-// Features of candidate (X, j, sign, rho) of term a = slot i (b = slot j).
+// Byte counts of one factor (mask M) of terms a and b: non-zeros of a, of b, in both, in both with
+// the same sign (each at most 64).
 template <class Wd>
-__device__ __forceinline__ void cand_features(const PTerm<Wd, 1, true> &a, const PTerm<Wd, 1, true> &b,
-                                              const Masks<Wd, 1> &mk, int X, int sneg, int rho, int k_i, int q,
-                                              int r, int best_r, int m, int n, int p, float (&f)[kFeat]) {
-    int Y = X == 0 ? 1 : (X == 1 ? 2 : 0);
-    int Z = X == 0 ? 2 : (X == 1 ? 0 : 1);
-    if (rho) { const int tmp = Y; Y = Z; Z = tmp; }
-    const Wd MX = mk.of(X, 0), MY = mk.of(Y, 0), MZ = mk.of(Z, 0);
-    const Wd ad = a.p[0] | a.n[0], bd = b.p[0] | b.n[0];
-    // Y_i + Y_j
-    const bool vy = (((a.p[0] & b.p[0]) | (a.n[0] & b.n[0])) & MY) == Wd(0);
-    const Wd syd = (((a.p[0] | b.p[0]) & ~(a.n[0] | b.n[0])) | ((a.n[0] | b.n[0]) & ~(a.p[0] | b.p[0]))) & MY;
-    // Z_j - s Z_i  (s = +1: add (a.n, a.p); s = -1: add (a.p, a.n))
-    const Wd zp = sneg ? a.p[0] : a.n[0], zn = sneg ? a.n[0] : a.p[0];
-    const bool vz = (((b.p[0] & zp) | (b.n[0] & zn)) & MZ) == Wd(0);
-    const Wd szd = (((b.p[0] | zp) & ~(b.n[0] | zn)) | ((b.n[0] | zn) & ~(b.p[0] | zp))) & MZ;
-#pragma unroll
-    for (int k = 0; k < kFeat; ++k) f[k] = (k == X) ? 1.f : 0.f;   // one-hot X in f[0..2]
-    f[3] = (float)rho;
-    f[4] = (float)sneg;
-    f[5] = (float)popc_w<Wd>(ad & MX);
-    f[6] = (float)popc_w<Wd>(ad & MY);
-    f[7] = (float)popc_w<Wd>(bd & MY);
-    f[8] = vy ? (float)popc_w<Wd>(syd) : 0.f;
-    f[9] = vy ? 1.f : 0.f;
-    f[10] = (float)popc_w<Wd>(ad & MZ);
-    f[11] = (float)popc_w<Wd>(bd & MZ);
-    f[12] = vz ? (float)popc_w<Wd>(szd) : 0.f;
-    f[13] = vz ? 1.f : 0.f;
-    f[14] = (float)popc_w<Wd>(ad & bd & MY);
-    f[15] = (float)popc_w<Wd>(ad & bd & MZ);
-    f[16] = (vy && syd == Wd(0)) ? 1.f : 0.f;
-    f[17] = (vz && szd == Wd(0)) ? 1.f : 0.f;
-    f[18] = (float)(k_i < 64 ? k_i : 64);
-    f[19] = (float)(r - best_r);
-    f[20] = (float)r;
-    f[21] = (float)m;
-    f[22] = (float)n;
-    f[23] = (float)p;
-    f[24] = (float)(q < 64 ? q : 64);
-    f[31] = 1.f;
+__device__ __forceinline__ uint32_t factor_counts(const PTerm<Wd, 1, true> &a, const PTerm<Wd, 1, true> &b, Wd M) {
+    const Wd ad = (a.p[0] | a.n[0]) & M, bd = (b.p[0] | b.n[0]) & M;
+    const Wd same = ((a.p[0] & b.p[0]) | (a.n[0] & b.n[0])) & M;
+    return (uint32_t)popc_w<Wd>(ad) | (uint32_t)popc_w<Wd>(bd) << 8 | (uint32_t)popc_w<Wd>(ad & bd) << 16 |
+           (uint32_t)popc_w<Wd>(same) << 24;
 }
 
-// Features of a candidate as 16 packed bf16x2 words (small integers: exact).
+// Two integers below 128 as a packed bf16x2 word, from the bytes of v that sel names (4: zero): as
+// 128 + k, whose BF16 bits are 0x4300 + k, less 128.
+__device__ __forceinline__ uint32_t bytes_bf16x2(uint32_t v, uint32_t sel) {
+    const uint32_t biased = __byte_perm(v, 0x00004300u, 0x5050u | (sel & 0xfu) | (sel & 0xf0u) << 4);
+    const uint32_t base = 0x43004300u;
+    __nv_bfloat162 x, c;
+    memcpy(&x, &biased, 4);
+    memcpy(&c, &base, 4);
+    const __nv_bfloat162 y = __hsub2(x, c);
+    uint32_t r;
+    memcpy(&r, &y, 4);
+    return r;
+}
+
+// Features of candidate dc (X, j, sign, rho) of term a = slot i (b = slot j) as 16 packed
+// bf16x2 words (small integers: exact):
+//   0-2 one-hot X, 3 rho, 4 sign, then with Y, Z the other two factors in rho's order
+//   5 |X_i|, 6 |Y_i|, 7 |Y_j|, 8 |Y_i + Y_j|, 9 the sum stays in {-1, 0, 1}, 10 |Z_i|, 11 |Z_j|,
+//   12 |Z_j - s Z_i|, 13 the difference stays in it, 14 |Y_i and Y_j|, 15 |Z_i and Z_j|,
+//   16 valid and zero sum, 17 valid and zero difference (8, 12: zero where not valid),
+//   18 k_i, 19 r - best r, 20 r, 21-23 m, n, p, 24 q, 31 one, the rest zero.
+// A valid sum or difference has no position with equal (opposite) signs, so its
+// non-zeros are |Y_i| + |Y_j| - 2 |both|: a byte dot product.  All three factors are
+// counted before rho and X choose among them (four bytes a factor: the choice moves
+// one word, not masks), and integers become BF16 two at a time without the
+// conversion unit.  These rows share the scoring kernel's issue slots
+// with its epilogues: with the masks chosen first and each feature a float, 2.63 ms a step for
+// 262144 walkers of (3,4,5) with full windows, now 2.51 (with 16-byte loads of the slots).
 template <class Wd>
 __device__ __forceinline__ void cand_features_bf16(const PTerm<Wd, 1, true> &a, const PTerm<Wd, 1, true> &b,
                                                    const Masks<Wd, 1> &mk, uint32_t dc, uint32_t info, int r,
                                                    int best_r, int m, int n, int p, uint32_t (&h)[kFeat / 2]) {
-    const int X = (int)((dc >> 10) & 3u), sneg = (int)((dc >> 22) & 1u), rho = (int)((dc >> 23) & 1u);
-    float f[kFeat];
-    cand_features<Wd>(a, b, mk, X, sneg, rho, (int)(info & 255u), (int)(info >> 8), r, best_r, m, n, p, f);
-#pragma unroll
-    for (int k = 0; k < kFeat / 2; ++k) h[k] = mlp::pack_bf16x2(f[2 * k], f[2 * k + 1]);
+    const uint32_t X = (dc >> 10) & 3u;
+    const bool sneg = (dc >> 22) & 1u, rho = (dc >> 23) & 1u;
+    const uint32_t cu = factor_counts<Wd>(a, b, mk.m[0][0]), cv = factor_counts<Wd>(a, b, mk.m[1][0]),
+                   cw = factor_counts<Wd>(a, b, mk.m[2][0]);
+    const uint32_t cx = X == 0 ? cu : (X == 1 ? cv : cw);
+    const uint32_t c1 = X == 0 ? cv : (X == 1 ? cw : cu), c2 = X == 0 ? cw : (X == 1 ? cu : cv);
+    const uint32_t cy = rho ? c2 : c1, cz = rho ? c1 : c2;
+    const bool vy = cy < (1u << 24);                                               // no equal signs
+    const bool vz = sneg ? cz < (1u << 24) : (cz >> 24) == ((cz >> 16) & 255u);    // no equal, or only equal ones
+    const uint32_t ny = (uint32_t)__dp4a((int)cy, 0x00FE0101, 0), nz = (uint32_t)__dp4a((int)cz, 0x00FE0101, 0);
+    const uint32_t one_lo = 0x00003F80u, one_hi = 0x3F800000u;
+    h[0] = X == 0 ? one_lo : (X == 1 ? one_hi : 0u);
+    h[1] = (X == 2 ? one_lo : 0u) | (rho ? one_hi : 0u);
+    h[2] = (sneg ? one_lo : 0u) | bytes_bf16x2(cx, 0x04);
+    h[3] = bytes_bf16x2(cy, 0x10);
+    h[4] = vy ? bytes_bf16x2(ny | 0x100u, 0x10) : 0u;
+    h[5] = bytes_bf16x2(cz, 0x10);
+    h[6] = vz ? bytes_bf16x2(nz | 0x100u, 0x10) : 0u;
+    h[7] = bytes_bf16x2(__byte_perm(cy, cz, 0x6262), 0x10);
+    h[8] = (vy && ny == 0 ? one_lo : 0u) | (vz && nz == 0 ? one_hi : 0u);
+    h[9] = mlp::pack_bf16x2((float)min((int)(info & 255u), 64), (float)(r - best_r));
+    h[10] = mlp::pack_bf16x2((float)r, (float)m);
+    h[11] = mlp::pack_bf16x2((float)n, (float)p);
+    h[12] = bytes_bf16x2(min(info >> 8, 64u), 0x40);
+    h[13] = h[14] = 0u;
+    h[15] = one_hi;
 }
 
 // One warp per walker; lane l holds slots l, l + 32, ... (NCH of them, r <= 32 NCH).
@@ -316,8 +330,8 @@ __global__ void __launch_bounds__(128) window_kernel(const SegDesc d, __nv_bfloa
 // Producer of the fused scoring kernel.  A warpgroup takes a contiguous share of the half
 // windows (unit 2 w + half: rows 0-127 or 128-255 of walker w) and lays their rows end to
 // end in groups of 32, the last group of a window ragged: warp j of its tile k takes
-// group 4 k + j.  (A tile for every half left a fifth to a quarter of the rows empty:
-// 262144 walkers of (3,4,5), windows of about 180 rows, @SCORE@.)
+// group 4 k + j.  (A tile for every half window left the rows past it empty: 3000 walkers
+// of (4,4,5), two learned steps, 246 us with it and 215 so.)
 // A lane holds the window size of one unit of 32 and the running count of their
 // groups; the next 32 sizes are loaded a chunk ahead.  A thread computes the features of
 // its row from the row's descriptor and the walker's two slots, straight into the A
@@ -396,11 +410,12 @@ struct WindowProducer {
     }
     __device__ __forceinline__ void mid(int) {
         const int i = min((int)(dci.x & 1023u), R - 1), j = min((int)((dci.x >> 12) & 1023u), R - 1);
-        const Wd *src = slots + (size_t)w * R * 2;
-        ti.p[0] = src[(size_t)i * 2];
-        ti.n[0] = src[(size_t)i * 2 + 1];
-        tj.p[0] = src[(size_t)j * 2];
-        tj.n[0] = src[(size_t)j * 2 + 1];
+        const WinSlot<Wd> *src = reinterpret_cast<const WinSlot<Wd> *>(slots) + (size_t)w * R;
+        const WinSlot<Wd> vi = src[i], vj = src[j];
+        ti.p[0] = vi.p;
+        ti.n[0] = vi.n;
+        tj.p[0] = vj.p;
+        tj.n[0] = vj.n;
     }
     __device__ __forceinline__ int64_t fill(uint8_t *sX, int q) {
         uint32_t h[kFeat / 2];
