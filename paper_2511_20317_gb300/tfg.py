@@ -335,15 +335,24 @@ def tfg_mlp_score(params, x, out=None, err=None, stream=None):
         out = torch.empty(n, dtype=torch.float32, device=x.device)
     own_err = err is None
     if own_err:
-        err = torch.zeros(1, dtype=torch.int32, device=x.device)
+        err = _host_error_word()
     st = stream if stream is not None else torch.cuda.current_stream()
     _check(lib().tfg_mlp_score(ctypes.c_void_p(params.data_ptr()), ctypes.c_void_p(x.data_ptr()), n,
                                ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(err.data_ptr()),
                                ctypes.c_void_p(st.cuda_stream)))
     if own_err:
-        if int(err.item()) != 0:
+        st.synchronize()
+        if int(err) != 0:
             raise TfgError(TFG_ETIMEOUT, "tensor-core completion wait gave up")
     return out
+
+
+def _host_error_word():
+    """An error word of a launch's own, in pinned host memory: the kernel writes it only when
+    a wait gives up, so that a call needs neither a launch to clear it nor a copy to
+    read it (20000 rows scored: 53 us with a word on the device, 39 so)."""
+    import torch
+    return torch.zeros(1, dtype=torch.int32, pin_memory=True)
 
 
 def _vp(t):
@@ -355,11 +364,12 @@ def tfg_mlp_grad(params, x, label, weight, stream=None):
     import torch
     P = MLP_NUM_PARAMS
     grad = torch.empty(P + 1, dtype=torch.float32, device=x.device)
-    err = torch.zeros(1, dtype=torch.int32, device=x.device)
+    err = _host_error_word()
     st = stream if stream is not None else torch.cuda.current_stream()
     _check(lib().tfg_mlp_grad(_vp(params), _vp(x), _vp(label), _vp(weight), x.shape[0], _vp(grad), _vp(err),
                               ctypes.c_void_p(st.cuda_stream)))
-    if int(err.item()) != 0:
+    st.synchronize()
+    if int(err) != 0:
         raise TfgError(TFG_ETIMEOUT, "tensor-core completion wait gave up")
     return grad[:P], float(grad[P].item())
 

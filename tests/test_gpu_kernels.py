@@ -236,3 +236,33 @@ def test_gradient_tiles_and_warpgroups(n, shift):
             bound = 2.0 ** -7 * np.asarray(ref["_abs"][name]) + 1e-6 * (1 + np.abs(ref[name]))
             diff = np.abs(np.asarray(got[name]) - np.asarray(ref[name]))
             assert (diff <= bound).all(), (name, float(np.max(diff - bound)))
+
+
+@pytest.mark.parametrize("fmt,nw", [((2, 2, 2), 5), ((2, 2, 3), 40009), ((3, 3, 3), 20011)])
+def test_window_scores_of_ragged_windows(fmt, nw):
+    """Scores of every window row, windows of all sizes laid end to end in groups of 32 rows and
+    many windows to a warpgroup, against the network on the dumped features (float32
+    products of the same bf16 operands).  Bound as for row scoring: two bf16 flips of a
+    hidden unit a row, 2 * 2^-8 * max_h |h1_h| sum_o |W2[h,o] w3[o]|, plus FP32 sums."""
+    import torch
+    from oracle import mlp
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=3, params=tfg.tfg_default_params(plateau_len=100))
+    W.walk_window(200, policy=0)
+    feat, _, kwin = W.window_dump()
+    feat, kwin = feat.clone(), kwin.clone()
+    p = mlp.Params.random(np.random.default_rng(6))
+    blob = torch.from_numpy(np.frombuffer(p.blob(), dtype=np.uint8).copy()).cuda()
+    W.walk_window(1, policy=1, mlp_params=blob)
+    W.sync()
+    _, score, kwin2 = W.window_buffers()
+    assert torch.equal(kwin, kwin2) and (nw < 100 or kwin.unique().numel() > 1)
+    W1, W2, b1, b2, w3 = (torch.from_numpy(np.asarray(a, np.float32)).cuda() for a in (p.W1, p.W2, p.b1, p.b2, p.w3))
+    path = W2.abs() @ w3.abs()
+    for lo in range(0, nw, 4096):
+        rows = torch.arange(256, device="cuda")[None] < kwin[lo:lo + 4096, None]
+        x = feat[lo:lo + 4096][rows].float()
+        h1 = torch.relu(x.double() @ W1.double() + b1.double()).float().bfloat16().float()
+        y = torch.relu(h1.double() @ W2.double() + b2.double()) @ w3.double() + float(p.b3)
+        bound = 2 * ((h1.abs() * 2.0 ** -8) * path).amax(1) + 1e-5 * (1 + y.abs())
+        assert ((score[lo:lo + 4096][rows].double() - y).abs() <= bound).all()
+    W.close()
