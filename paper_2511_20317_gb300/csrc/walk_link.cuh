@@ -8,9 +8,9 @@
 // only an accepted flip moves two slots to other classes.
 //   NW = 1 (at most 32 slots): one 32-bit row per slot and factor, bit k = slot
 //     k holds an equal factor (ROWS);
-//   NW > 1: the slots of a class form a cyclic list in ascending order, one byte
+//   NW > 1, or LIST: the slots of a class form a cyclic list in ascending order, one byte
 //     per slot and factor (the next member), so that a walker needs 4 bytes
-//     per slot instead of 3 * 4 * NW.
+//     per slot instead of 3 * 4 * NW (link_lists_pay says when at most 32 slots take lists).
 // Where a changed factor goes is found by its 8-bit hash: the hashes of all
 // slots are held bit-sliced (word q of slice b: bit b of the hashes of slots
 // 32 q .. 32 q + 31), so that one pass over the 8 NW words of the factor compares
@@ -39,6 +39,7 @@
 //   -> flip + ternary validity -> zero-term removal -> sign normalisation ->
 //   reduction cascade -> best/plateau -> plus transition (+ cascade).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 #include "pterm.cuh"
@@ -57,11 +58,11 @@ __device__ __forceinline__ uint32_t sign_spread(uint32_t x) {
     return r;
 }
 
-template <int MODE, class Wd, int NW, bool GM, bool PG, bool CNT = false>
+template <int MODE, class Wd, int NW, bool GM, bool PG, bool CNT = false, bool LIST = false>
 struct LinkWalker {
     static constexpr bool ZT = (MODE == TFG_MODE_ZT);
     static constexpr int NWS = ZT ? 2 : 1;   // words per slot
-    static constexpr bool ROWS = NW == 1 && !CNT;
+    static constexpr bool ROWS = NW == 1 && !CNT && !LIST;
     static constexpr bool kCounts = CNT;
     using T = PTerm<Wd, 1, ZT>;
     using O = Ops<Wd, 1, ZT>;
@@ -935,12 +936,12 @@ __device__ __forceinline__ void link_rows(LW &wk, const SegDesc &d, int64_t w, b
 // Blocks of any whole number of warps (kLinkMaxBlock threads at most): a warp's
 // rows are its own.
 constexpr int kLinkMaxBlock = 160;
-template <int MODE, class Wd, int NW, bool GM, bool PG>
+template <int MODE, class Wd, int NW, bool GM, bool PG, bool LIST = false>
 __global__ void __launch_bounds__(kLinkMaxBlock, 3) walk_link_kernel(const SegDesc d, const int32_t steps) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= d.n_walkers) return;   // no block-wide barrier is used
-    using LW = LinkWalker<MODE, Wd, NW, GM, PG>;
+    using LW = LinkWalker<MODE, Wd, NW, GM, PG, false, LIST>;
     LW wk;
     link_rows<LW, Wd>(wk, d, w, GM, smem_raw);
     wk.run(d, w, steps);
@@ -958,6 +959,10 @@ void prepare_walk_link() {
         };
         set(dev::walk_link_kernel<MODE, Wd, NW, false, false>);
         set(dev::walk_link_kernel<MODE, Wd, NW, false, true>);
+        if constexpr (NW == 1 && sizeof(Wd) == 4) {
+            set(dev::walk_link_kernel<MODE, Wd, NW, false, false, true>);
+            set(dev::walk_link_kernel<MODE, Wd, NW, false, true, true>);
+        }
         if constexpr (sizeof(Wd) == 8) {
             set(dev::walk_link_kernel<MODE, Wd, NW, true, false>);
             set(dev::walk_link_kernel<MODE, Wd, NW, true, true>);
@@ -976,12 +981,37 @@ void prepare_walk_link() {
 // resident) 9.2e9 / 7.0e9; (3,3,4) 40330 walkers (1.1 times what fits) 1.02e10 /
 // 1.24e10; (4,4,5) 80660 walkers (4.5 times) 5.3e9 / 9.5e9.  32-bit terms (at
 // most 32 slots of 8 bytes) always go to shared memory.
-inline bool link_terms_shared(size_t block_bytes, int64_t grid) {
-    if (block_bytes > (size_t)kLinkSmem) return false;
+// Blocks an SM's shared memory holds (1 KB a block is the system's), over all SMs
+inline int64_t link_resident(size_t block_bytes) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return grid <= (int64_t)sms * (int64_t)(kLinkSmem / (block_bytes + 1024));   // 1 KB a block is the system's
+    return (int64_t)sms * (int64_t)(kLinkSmem / (block_bytes + 1024));
+}
+inline bool link_terms_shared(size_t block_bytes, int64_t grid) {
+    return block_bytes <= (size_t)kLinkSmem && grid <= link_resident(block_bytes);
+}
+
+// At most 32 slots: classes as rows (12 bytes a slot) or as lists (4).  A row is read at
+// once, a list member by member, so rows are the faster where as many walkers reside;
+// lists let up to twice as many (16 warps an SM, by their registers), and pay when rows
+// need half as many waves of blocks again, under policy 1 twice as many.  Not
+// where a factor is so short that many slots share it (lists grow long): at least
+// six coefficients.  Measured, rows / lists, ms per 1000 steps: (2,3,4) 20000 walkers (one
+// wave) Z_T 1.55 / 1.81, 65536 (two / one) Z_T 3.03 / 2.52, Z_2 3.82 / 2.81, 131072 (three /
+// two) Z_T 4.79 / 4.46, Z_2 5.84 / 5.07, policy 1 Z_T 100000 (three / two) 7.0 / 7.9, 65536
+// Z_2 (two / one) 12.0 / 10.1, policy 2 Z_T 65536 3.13 / 2.20; (2,3,3) 65536 Z_T (two /
+// one) 2.79 / 2.32, 262144 (five / four) 7.3 / 7.8; (2,2,6) Z_T 65536 (two / one) 3.16 /
+// 3.17, 131072 (three / two) 5.02 / 5.62.
+inline bool link_lists_pay(const SegDesc &d, size_t rows_bytes, size_t lists_bytes, int64_t grid, int block) {
+    const int shortest = std::min(d.m * d.n, std::min(d.n * d.p, d.p * d.m));
+    if (shortest < 6) return false;
+    auto waves = [&](size_t bytes) {   // of at most 16 warps an SM
+        const size_t room = std::max(bytes, (size_t)kLinkSmem / (512 / block) - 1024);
+        return (grid + link_resident(room) - 1) / std::max<int64_t>(link_resident(room), 1);
+    };
+    const int64_t rows = waves(rows_bytes), lists = waves(lists_bytes);
+    return d.walk_policy == 1 ? rows >= 2 * lists : 2 * rows >= 3 * lists;
 }
 
 template <int MODE, class Wd, int NW>
@@ -990,6 +1020,16 @@ void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cuda
     using Shared = dev::LinkWalker<MODE, Wd, NW, false, false>;
     using Device = dev::LinkWalker<MODE, Wd, NW, true, false>;
     const size_t block_bytes = Shared::thread_bytes(d.R) * block;
+    if constexpr (NW == 1 && sizeof(Wd) == 4) {
+        const size_t lists = dev::LinkWalker<MODE, Wd, NW, false, false, false, true>::thread_bytes(d.R) * block;
+        if (link_lists_pay(d, block_bytes, lists, grid, block)) {
+            if (d.walk_policy == 0)
+                dev::walk_link_kernel<MODE, Wd, NW, false, false, true><<<grid, block, lists, st>>>(d, steps);
+            else
+                dev::walk_link_kernel<MODE, Wd, NW, false, true, true><<<grid, block, lists, st>>>(d, steps);
+            return;
+        }
+    }
     const bool shared = sizeof(Wd) == 4 || link_terms_shared(block_bytes, grid);
     const size_t smem = shared ? block_bytes : Device::thread_bytes(d.R) * block;
     if (shared) {

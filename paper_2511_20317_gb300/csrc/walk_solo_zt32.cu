@@ -13,8 +13,8 @@ const WalkVariant *walk_variants_solo_zt32(int *n) {
         TFG_THREAD_VARIANT(TFG_MODE_ZT, uint32_t, 32, 24, 32),
         TFG_THREAD_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, 32),
         TFG_THREAD_VARIANT_AUTO(TFG_MODE_ZT, uint32_t, 32, 64, 32),
-        TFG_SOLO_SLICED_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, TFG_SLICED_ZT_BLOCK, 9, false),
-        TFG_SOLO_SLICED_VARIANT(TFG_MODE_ZT, uint32_t, 32, 32, TFG_SLICED_ZT_BLOCK, 9, true),
+        TFG_SLICED_ZT_VARIANT(uint32_t, 32, TFG_SLICED_ZT_BLOCK, 9, false),
+        TFG_SLICED_ZT_VARIANT(uint32_t, 32, TFG_SLICED_ZT_BLOCK, 9, true),
     };
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;

@@ -50,6 +50,28 @@ void launch_walk_thread(const SegDesc &d, int32_t steps, int grid, int block, cu
     launch_walk_link<MODE, Wd, (CAP + 31) / 32>(d, steps, grid, block, st);
 }
 
+// Bit-sliced kernels of Z_T (walk_solo.cuh): 971 instructions a warp-step at 64% of the issue
+// rate, against about 600 with kept classes.  The plateau policy keeps classes from more
+// than a warp a scheduler on; below, a step's latency counts, and there the slices are the
+// faster.  Measured, (3,3,3), ms per 1000 steps, slices / classes: 1024 walkers 1.36 / 1.44,
+// 14000 1.39 / 1.46, 20000 1.77 / 1.57, 40000 2.29 / 1.74, 65536 2.88 / 2.43, 131072 5.2 /
+// 4.66; policy 1, 20000 walkers 2.35 / 2.71, 65536 4.11 / 4.01.  Over Z_2 (643
+// instructions, half the slices, in registers) slices are always the faster: 65536 walkers
+// 2.05 / 2.50.
+constexpr int64_t kSlicedMax = 152 * 128;
+template <class Wd, int BT, int FL, bool SQ>
+void prepare_walk_sliced_zt() {
+    prepare_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>();
+    prepare_walk_link<TFG_MODE_ZT, Wd, 1>();
+}
+template <class Wd, int BT, int FL, bool SQ>
+void launch_walk_sliced_zt(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
+    if (d.walk_policy == 0 && d.n_walkers > kSlicedMax)
+        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, (int)((d.n_walkers + 31) / 32), 32, st);
+    else
+        launch_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>(d, steps, grid, block, st);
+}
+
 }  // namespace tfg
 
 // capacity CAP, BLOCK walkers per block
@@ -63,3 +85,8 @@ void launch_walk_thread(const SegDesc &d, int32_t steps, int grid, int block, cu
     WalkVariant{MODE, BITS, 1, 1, CAP, BLOCK, &launch_walk_link<MODE, WD, (CAP + 31) / 32>, \
                 reinterpret_cast<const void *>(&dev::walk_link_kernel<MODE, WD, (CAP + 31) / 32, BITS == 64, false>), \
                 &prepare_walk_link<MODE, WD, (CAP + 31) / 32>, 0, 0, 0, true}
+// Z_T bit-sliced, 32 slots: factors of at most FL coefficients (SQ: exactly FL each)
+#define TFG_SLICED_ZT_VARIANT(WD, BITS, BT, FL, SQ) \
+    WalkVariant{TFG_MODE_ZT, BITS, 1, 1, 32, BT, &launch_walk_sliced_zt<WD, BT, FL, SQ>, \
+                reinterpret_cast<const void *>(dev::solo_kernel<TFG_MODE_ZT, WD, 32, BT, FL, SQ>()), \
+                &prepare_walk_sliced_zt<WD, BT, FL, SQ>, 0, FL, SQ ? 1 : 0}

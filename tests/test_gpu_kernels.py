@@ -266,3 +266,27 @@ def test_window_scores_of_ragged_windows(fmt, nw):
         bound = 2 * ((h1.abs() * 2.0 ** -8) * path).amax(1) + 1e-5 * (1 + y.abs())
         assert ((score[lo:lo + 4096][rows].double() - y).abs() <= bound).all()
     W.close()
+
+
+@pytest.mark.parametrize("fmt,nw,policy", [((2, 3, 4), 60001, 0), ((2, 3, 4), 60001, 1), ((2, 3, 4), 60001, 2),
+                                           ((2, 3, 3), 70001, 0), ((3, 3, 3), 70001, 0), ((3, 3, 3), 19456, 0),
+                                           ((3, 3, 3), 19457, 0), ((3, 3, 3), 20033, 2), ((2, 2, 6), 60001, 0)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_populations_at_which_the_class_walker_changes(fmt, nw, policy, mode):
+    """Populations on either side of the choice between factor classes as rows and as lists (two
+    waves of rows against one of lists; short factors keep rows) and between bit
+    slices and classes, walkers spread over the population against the oracle."""
+    L, steps = 40, 400
+    start = naive_start(*fmt)
+    kw = dict(plateau_len=L if policy == 0 else 10**6, walk_policy=policy,
+              expand_thresh=int(0.03 * 2**32) if policy == 1 else 0)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=14, params=tfg.tfg_default_params(**kw))
+    W.walk(steps).sync()
+    take = np.linspace(0, nw - 1, 48).astype(int)
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=14, mode=mode, plateau_len=kw["plateau_len"], policy=policy,
+                         expand_thresh=kw["expand_thresh"])
+    ref.walk(steps, threads=THREADS)
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} policy {policy} mode {mode}")
+    W.close()
