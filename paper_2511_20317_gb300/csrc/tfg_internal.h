@@ -38,7 +38,20 @@ struct SegDesc {
     int32_t walk_policy;  // 0: plateau plus transitions; 1: Algorithm 1 expansions
     uint32_t expand_thresh;
     int32_t pad3;
+    int64_t all_walkers;  // of all populations, whose kernels share the GPU
 };
+
+// Lanes of a warp that hold walkers, for the kernels of one walker per thread: the fewest (a
+// power of two) at which all populations together make at most `warps` warps, 32 when
+// no fewer do.  A warp's step takes the path of every lane and its loops the turns of the
+// longest, so a population too small to fill the GPU is spread over more warps.  Up to
+// eight warps an SM their steps hardly slow one another.  Measured, 500 steps, ms, 32
+// lanes / 16 / 8 / 4 / 2 / 1: (2,2,2) 1024 walkers 0.60 / 0.52 / 0.45 / 0.40 / 0.35 / 0.35,
+// 4096 0.60 / 0.53 / 0.48 / 0.46 / 0.50 / 0.74; (2,3,4) 1024 0.77 / 0.67 / 0.57 / 0.48 / 0.39 /
+// 0.36, 10000 0.77 / 0.73 / 0.70 / 1.03; (4,4,5) 1024 1.36 / 1.17 / 0.99 / 0.80 / 0.65 / 0.60.
+constexpr int kSpreadWarps = 8;   // an SM
+int walk_lanes(const SegDesc &d, int64_t warps);
+int sm_count();
 
 // One compiled variant of the walk kernel.
 struct WalkVariant {

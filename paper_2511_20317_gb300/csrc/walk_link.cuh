@@ -983,13 +983,36 @@ void prepare_walk_link() {
 // most 32 slots of 8 bytes) always go to shared memory.
 // Blocks an SM's shared memory holds (1 KB a block is the system's), over all SMs
 inline int64_t link_resident(size_t block_bytes) {
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return (int64_t)sms * (int64_t)(kLinkSmem / (block_bytes + 1024));
+    return (int64_t)sm_count() * (int64_t)(kLinkSmem / (block_bytes + 1024));
 }
 inline bool link_terms_shared(size_t block_bytes, int64_t grid) {
     return block_bytes <= (size_t)kLinkSmem && grid <= link_resident(block_bytes);
+}
+
+// Launch shape of a class walker and the place of its terms (thread_bytes with the terms in
+// shared / device memory; device 0: shared only).  A population too small to fill the
+// GPU takes blocks of one warp with walkers in few lanes (walk_lanes), as many warps as
+// reside at once; their columns are a full warp's.  Terms in device memory leave
+// room for more warps, which outweighs the reads from L2 when that means a quarter of
+// the lanes, eight at most: (4,4,5), 500 steps, shared / device, 2048 walkers 0.99 (8 lanes)
+// / 0.82 (2), 4096 1.17 (16) / 1.19 (4), 10000 1.36 (32) / 1.75 (16).
+struct LinkShape {
+    int grid, block;
+    bool shared;
+    size_t smem;
+};
+inline LinkShape link_shape(const SegDesc &d, int grid, int block, size_t shared_bytes, size_t device_bytes) {
+    auto lanes = [&](size_t bytes) {
+        return walk_lanes(d, std::min<int64_t>((int64_t)kSpreadWarps * sm_count(), link_resident(32 * bytes)));
+    };
+    const int ls = lanes(shared_bytes), lg = device_bytes ? lanes(device_bytes) : 32;
+    const bool spread_device = 4 * lg <= ls && ls <= 8;
+    const bool shared = device_bytes == 0 ||
+                        (!spread_device && (ls < 32 || link_terms_shared(shared_bytes * block, grid)));
+    const int l = shared ? ls : lg;
+    const size_t bytes = shared ? shared_bytes : device_bytes;
+    if (l == 32) return {grid, block, shared, bytes * block};
+    return {(int)((d.n_walkers + l - 1) / l), l, shared, bytes * 32};
 }
 
 // At most 32 slots: classes as rows (12 bytes a slot) or as lists (4).  A row is read at
@@ -1019,10 +1042,11 @@ void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cuda
     prepare_walk_link<MODE, Wd, NW>();
     using Shared = dev::LinkWalker<MODE, Wd, NW, false, false>;
     using Device = dev::LinkWalker<MODE, Wd, NW, true, false>;
-    const size_t block_bytes = Shared::thread_bytes(d.R) * block;
+    const LinkShape k = link_shape(d, grid, block, Shared::thread_bytes(d.R),
+                                   sizeof(Wd) == 8 ? Device::thread_bytes(d.R) : (size_t)0);
     if constexpr (NW == 1 && sizeof(Wd) == 4) {
         const size_t lists = dev::LinkWalker<MODE, Wd, NW, false, false, false, true>::thread_bytes(d.R) * block;
-        if (link_lists_pay(d, block_bytes, lists, grid, block)) {
+        if (k.block == block && link_lists_pay(d, k.smem, lists, grid, block)) {
             if (d.walk_policy == 0)
                 dev::walk_link_kernel<MODE, Wd, NW, false, false, true><<<grid, block, lists, st>>>(d, steps);
             else
@@ -1030,14 +1054,12 @@ void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cuda
             return;
         }
     }
-    const bool shared = sizeof(Wd) == 4 || link_terms_shared(block_bytes, grid);
-    const size_t smem = shared ? block_bytes : Device::thread_bytes(d.R) * block;
-    if (shared) {
-        if (d.walk_policy == 0) dev::walk_link_kernel<MODE, Wd, NW, false, false><<<grid, block, smem, st>>>(d, steps);
-        else dev::walk_link_kernel<MODE, Wd, NW, false, true><<<grid, block, smem, st>>>(d, steps);
+    if (k.shared) {
+        if (d.walk_policy == 0) dev::walk_link_kernel<MODE, Wd, NW, false, false><<<k.grid, k.block, k.smem, st>>>(d, steps);
+        else dev::walk_link_kernel<MODE, Wd, NW, false, true><<<k.grid, k.block, k.smem, st>>>(d, steps);
     } else if constexpr (sizeof(Wd) == 8) {
-        if (d.walk_policy == 0) dev::walk_link_kernel<MODE, Wd, NW, true, false><<<grid, block, smem, st>>>(d, steps);
-        else dev::walk_link_kernel<MODE, Wd, NW, true, true><<<grid, block, smem, st>>>(d, steps);
+        if (d.walk_policy == 0) dev::walk_link_kernel<MODE, Wd, NW, true, false><<<k.grid, k.block, k.smem, st>>>(d, steps);
+        else dev::walk_link_kernel<MODE, Wd, NW, true, true><<<k.grid, k.block, k.smem, st>>>(d, steps);
     }
 }
 

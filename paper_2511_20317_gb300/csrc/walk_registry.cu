@@ -1,5 +1,9 @@
-// Registry of the compiled walk-kernel variants.
+// Registry of the compiled walk-kernel variants, and the launch shape of small populations.
+#include <algorithm>
+#include <atomic>
 #include <vector>
+
+#include <cuda_runtime.h>
 
 #include "tfg_internal.h"
 
@@ -35,5 +39,23 @@ const WalkVariant *walk_variants(int *count) {
     }();
     *count = (int)all.size();
     return all.data();
+}
+
+int sm_count() {
+    static std::atomic<int> known[64];   // by device; 0: not asked yet
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    const bool keep = dev >= 0 && dev < 64;
+    if (keep && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
+    if (keep) known[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
+int walk_lanes(const SegDesc &d, int64_t warps) {
+    const int64_t n = std::max(d.all_walkers, d.n_walkers);
+    int lanes = 32;
+    while (lanes > 1 && (n + lanes / 2 - 1) / (lanes / 2) <= warps) lanes /= 2;
+    return lanes;
 }
 }  // namespace tfg

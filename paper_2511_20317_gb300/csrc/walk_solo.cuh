@@ -20,6 +20,7 @@
 //   -> flip + ternary validity -> zero-term removal -> sign normalisation ->
 //   reduction cascade -> best/plateau -> plus transition (+ cascade).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -1026,7 +1027,8 @@ __host__ __device__ constexpr size_t solo_packed_bytes() {
 
 template <int MODE, class Wd, int RMAX, int BT, int FL = 0, bool SQ = false>
 __device__ __forceinline__ void walk_solo_body(const SegDesc &d, int32_t steps, unsigned char *smem_raw) {
-    const int64_t w = (int64_t)blockIdx.x * BT + threadIdx.x;
+    // BT threads, or few lanes of a warp (32 bits: 2^32 walkers' records alone exceed the memory)
+    const int64_t w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= d.n_walkers) return;   // no block-wide barrier is used
     SoloWalker<MODE, Wd, RMAX, BT, FL, SQ> wk;
     constexpr int NWS = (MODE == TFG_MODE_ZT) ? 2 : 1;
@@ -1094,7 +1096,18 @@ void prepare_walk_solo() {
 template <int MODE, class Wd, int RMAX, int BT, int FL = 0, bool SQ = false>
 void launch_walk_solo(const SegDesc &d, int32_t steps, int grid, int /*block*/, cudaStream_t st) {
     prepare_walk_solo<MODE, Wd, RMAX, BT, FL, SQ>();
-    dev::solo_kernel<MODE, Wd, RMAX, BT, FL, SQ>()<<<grid, BT, solo_smem_bytes<MODE, Wd, RMAX, BT, FL>(), st>>>(d, steps);
+    // Small populations: one warp a block, walkers in few of its lanes; the rows are a full block's.
+    // A step here is mostly the search, the same for every lane, so that a second warp on
+    // a scheduler costs more than fewer lanes save: at most a warp a scheduler.  (16000
+    // walkers, 500 warps of 32 lanes / 1000 of 16, 300 steps: (3,3,3) Z_2 0.335 / 0.403 ms, (2,3,4)
+    // Z_2 policy 2 0.366 / 0.463; 300 walkers, 32 lanes / 1: 0.325 / 0.299 and 0.357 / 0.331, (2,2,2)
+    // Z_T policy 1 2.96 / 0.99.)
+    constexpr size_t smem = solo_smem_bytes<MODE, Wd, RMAX, BT, FL>();
+    const int fit = std::min(4, (int)((size_t)227 * 1024 / (smem + 1024)));
+    const int lanes = walk_lanes(d, (int64_t)fit * sm_count());
+    const int block = lanes < 32 ? lanes : BT;
+    if (lanes < 32) grid = (int)((d.n_walkers + lanes - 1) / lanes);
+    dev::solo_kernel<MODE, Wd, RMAX, BT, FL, SQ>()<<<grid, block, smem, st>>>(d, steps);
 }
 
 // bit-sliced: formats whose factors have at most FL coefficients (SQ: exactly FL each)

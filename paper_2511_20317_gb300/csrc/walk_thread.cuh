@@ -7,23 +7,33 @@
 
 namespace tfg {
 
+// Lanes a warp would get if the population kept classes: few for a small one.
+inline int class_lanes(const SegDesc &d) { return walk_lanes(d, (int64_t)kSpreadWarps * sm_count()); }
+// At most a full warp a scheduler: a step's latency counts, not its instructions.
+inline bool one_warp_each(const SegDesc &d) { return d.n_walkers <= (int64_t)128 * sm_count(); }
+
 // Keeping the classes pays when most steps only read them, and when the rank is large.
 // It does not when nearly every step changes the scheme and nothing else in the step
 // needs the search: walk policy 2 (no reduction test after a flip) on few slots or over
 // Z_2 (9 of 10 flips are accepted), and walk policy 1 on the smallest ranks, where
-// expansions and reductions alternate.  A small population is bound by the latency
-// of one step, where the classes' short dependent loops cost most.  Measured, 300 steps,
-// ms testing every slot / keeping classes:
-//   policy 1: (2,2,2) Z_T 1000 walkers 3.25 / 4.18, (2,2,3) Z_T 3.05 / 2.69, 30000 walkers 5.08 / 3.28;
-//     Z_2 (2,3,3) 30000 2.31 / 2.47, (2,3,4) 1000 1.70 / 2.00, 30000 3.00 / 2.20, (2,4,5) 1000 3.35 / 1.71
-//   policy 2: Z_T (2,3,3) 1000 0.40 / 0.48, 30000 0.53 / 0.53, (2,3,4) 30000 0.62 / 0.56, (2,4,5) 1000 0.70 / 0.63;
-//     Z_2 (2,3,4) 30000 0.45 / 0.63, (4,4,5) 30000 1.04 / 1.42
+// expansions and reductions alternate.  Small populations keep classes all the same: their
+// short dependent loops are what few lanes a warp save most on.  Measured, 300 steps, ms
+// testing every slot / keeping classes (both in few lanes where that is faster):
+//   policy 1: Z_T (2,2,2) 1200 walkers 1.26 / 0.87, 10000 3.16 / 3.08, 18000 3.19 / 3.47;
+//     Z_2 (2,2,3) 1200 0.73 / 0.47, 2500 1.05 / 0.85, 5000 1.06 / 1.18; (2,3,3) 5000 1.71 / 1.08,
+//     10000 1.66 / 1.54, 18000 1.58 / 1.64; (2,3,4) 1200 1.05 / 0.46, 10000 1.75 / 1.35
+//   policy 2: Z_T (2,2,3) 1200 0.32 / 0.27, 5000 0.36 / 0.43; (2,3,4) 1200 0.40 / 0.26, 5000 0.45 /
+//     0.43, 18000 0.46 / 0.50, 30000 0.62 / 0.56; Z_2 (2,3,4) 1200 0.34 / 0.35, 18000 0.37 / 0.59;
+//     (4,4,5) 1200 0.68 / 0.51, 5000 0.70 / 0.74, 30000 1.04 / 1.42
 template <int MODE, class Wd>
 inline bool every_slot_faster(const SegDesc &d) {
-    constexpr bool z2 = MODE == TFG_MODE_Z2;
-    constexpr int64_t small = 16384;
-    if (d.walk_policy == 2) return z2 || (sizeof(Wd) == 4 && (d.R <= 20 || d.n_walkers < small));
-    if (d.walk_policy == 1) return sizeof(Wd) == 4 && (z2 ? d.R <= 24 || d.n_walkers < small : d.R <= 12);
+    constexpr bool z2 = MODE == TFG_MODE_Z2, small = sizeof(Wd) == 4;
+    const int lanes = class_lanes(d);
+    if (d.walk_policy == 2) {
+        if (z2) return small || lanes > 1;
+        return small && (d.R <= 20 ? lanes > 2 : lanes > 4 && one_warp_each(d));
+    }
+    if (d.walk_policy == 1) return small && (z2 ? d.R <= 24 && lanes > (d.R <= 16 ? 2 : 8) : d.R <= 12 && lanes > 8);
     return false;
 }
 
@@ -51,14 +61,17 @@ void launch_walk_thread(const SegDesc &d, int32_t steps, int grid, int block, cu
 }
 
 // Bit-sliced kernels of Z_T (walk_solo.cuh): 971 instructions a warp-step at 64% of the issue
-// rate, against about 600 with kept classes.  The plateau policy keeps classes from more
-// than a warp a scheduler on; below, a step's latency counts, and there the slices are the
-// faster.  Measured, (3,3,3), ms per 1000 steps, slices / classes: 1024 walkers 1.36 / 1.44,
-// 14000 1.39 / 1.46, 20000 1.77 / 1.57, 40000 2.29 / 1.74, 65536 2.88 / 2.43, 131072 5.2 /
-// 4.66; policy 1, 20000 walkers 2.35 / 2.71, 65536 4.11 / 4.01.  Over Z_2 (643
-// instructions, half the slices, in registers) slices are always the faster: 65536 walkers
-// 2.05 / 2.50.
-constexpr int64_t kSlicedMax = 152 * 128;
+// rate, against 600 to 800 with kept classes.  The plateau policy keeps classes beyond a warp a
+// scheduler, and so does every policy in a small population.  Measured, (3,3,3), slices /
+// classes, ms: 300 steps, 1200 walkers 0.35 / 0.24, 5000 0.43 / 0.41, 10000 0.44 / 0.47; policy
+// 1, 2500 0.65 / 0.59; policy 2, 2500 0.365 / 0.34, 5000 0.38 / 0.43; 1000 steps, 14000 1.39 / 1.46,
+// 20000 1.77 / 1.57, 40000 2.29 / 1.74, 65536 2.88 / 2.43, 131072 5.2 / 4.66; policy 1, 20000 2.35 /
+// 2.71, 65536 4.11 / 4.01.  Over Z_2 (643 instructions, half the slices, in registers)
+// the slices are the faster or as fast: 300 walkers 0.30 / 0.29, 5000 0.32 / 0.48, 65536 2.05 / 2.50.
+inline bool slices_faster(const SegDesc &d) {
+    const int lanes = class_lanes(d);
+    return d.walk_policy == 0 ? lanes > 4 && one_warp_each(d) : lanes > 2;
+}
 template <class Wd, int BT, int FL, bool SQ>
 void prepare_walk_sliced_zt() {
     prepare_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>();
@@ -66,10 +79,10 @@ void prepare_walk_sliced_zt() {
 }
 template <class Wd, int BT, int FL, bool SQ>
 void launch_walk_sliced_zt(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
-    if (d.walk_policy == 0 && d.n_walkers > kSlicedMax)
-        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, (int)((d.n_walkers + 31) / 32), 32, st);
-    else
+    if (slices_faster(d))
         launch_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>(d, steps, grid, block, st);
+    else
+        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, (int)((d.n_walkers + 31) / 32), 32, st);
 }
 
 }  // namespace tfg

@@ -820,13 +820,12 @@ static void window_walk_variant(const SegDesc &d, int32_t steps, int32_t *choice
         return true;
     }();
     (void)attr;
-    const unsigned grid = (unsigned)((d.n_walkers + kBlock - 1) / kBlock);
-    const size_t bytes = Shared::thread_bytes(d.R) * kBlock;
-    if (sizeof(Wd) == 4 || link_terms_shared(bytes, grid)) {
-        dev::window_walk_kernel<Wd, NW, false><<<grid, kBlock, bytes, st>>>(d, steps, choices, stride, log);
+    const LinkShape k = link_shape(d, (int)((d.n_walkers + kBlock - 1) / kBlock), kBlock, Shared::thread_bytes(d.R),
+                                   sizeof(Wd) == 8 ? Device::thread_bytes(d.R) : (size_t)0);
+    if (k.shared) {
+        dev::window_walk_kernel<Wd, NW, false><<<k.grid, k.block, k.smem, st>>>(d, steps, choices, stride, log);
     } else if constexpr (sizeof(Wd) == 8) {
-        dev::window_walk_kernel<Wd, NW, true><<<grid, kBlock, Device::thread_bytes(d.R) * kBlock, st>>>(d, steps, choices,
-                                                                                                        stride, log);
+        dev::window_walk_kernel<Wd, NW, true><<<k.grid, k.block, k.smem, st>>>(d, steps, choices, stride, log);
     }
 }
 

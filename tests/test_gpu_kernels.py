@@ -290,3 +290,44 @@ def test_populations_at_which_the_class_walker_changes(fmt, nw, policy, mode):
     ref.walk(steps, threads=THREADS)
     assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} policy {policy} mode {mode}")
     W.close()
+
+
+@pytest.mark.parametrize("nw", [1, 1217, 2433, 4865, 9729])
+@pytest.mark.parametrize("fmt,mode,policy", [((2, 2, 2), 0, 0), ((2, 3, 4), 1, 1), ((3, 3, 3), 0, 0), ((3, 3, 3), 1, 0),
+                                             ((2, 3, 3), 0, 2), ((4, 4, 5), 0, 0), ((4, 4, 5), 1, 2)])
+def test_small_populations_in_few_lanes(fmt, mode, policy, nw):
+    """Populations of which a warp takes 1, 2, 4, 8 or 16 walkers (a block's last lanes empty),
+    alone and beside another population, against the oracle: the walkers at both ends and spread between."""
+    L, steps = 60, 300
+    start = naive_start(*fmt)
+    kw = dict(plateau_len=L if policy == 0 else 10**6, walk_policy=policy,
+              expand_thresh=int(0.03 * 2**32) if policy == 1 else 0)
+    other = [((2, 2, 3), 0, naive_start(2, 2, 3), 77)] if nw < 5000 else []
+    W = tfg.Walkers([(fmt, mode, start, nw)] + other, seed=15, params=tfg.tfg_default_params(**kw))
+    W.walk(steps // 2).walk(steps - steps // 2).sync()
+    take = np.unique(np.concatenate([np.arange(min(nw, 8)), np.linspace(0, nw - 1, 24).astype(int),
+                                     np.arange(max(0, nw - 8), nw)]))
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=15, mode=mode, plateau_len=kw["plateau_len"], policy=policy,
+                         expand_thresh=kw["expand_thresh"])
+    ref.walk(steps, threads=THREADS)
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} policy {policy} mode {mode}")
+    assert W.verify_all() == 0
+    W.close()
+
+
+@pytest.mark.parametrize("fmt,nw", [((2, 2, 2), 301), ((3, 4, 5), 1217), ((4, 4, 4), 2433), ((2, 3, 3), 4865)])
+def test_uniform_window_walk_in_few_lanes(fmt, nw):
+    """The joint launch of uniform window steps on small populations equals the same steps
+    one by one, walker records and choices."""
+    steps = 12
+    mk = lambda: tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=16, params=tfg.tfg_default_params(plateau_len=50))
+    A, B = mk(), mk()
+    ca = A.walk_window(steps, policy=0, record_choices=True)
+    cb = [B.walk_window(1, policy=0, record_choices=True) for _ in range(steps)]
+    A.sync(), B.sync()
+    assert np.array_equal(ca.cpu().numpy(), np.concatenate([c.cpu().numpy() for c in cb]))
+    for x, y in zip(A.read_walkers(0, nw), B.read_walkers(0, nw)):
+        assert np.array_equal(x, y)
+    A.close(), B.close()
