@@ -197,7 +197,7 @@ struct tfg_ctx {
         d.best = ws + s.off_best;
         d.hdr = reinterpret_cast<tfg_walker_info *>(ws + s.off_hdr);
         d.n_walkers = s.n;
-        d.all_walkers = total;
+        d.beside = prm.use_graph == 2 ? total : s.n;   // forked: all populations at once
         d.R = s.R;
         d.m = s.fmt.m; d.n = s.fmt.n; d.p = s.fmt.p;
         d.lt = s.lt; d.tw = s.tw; d.nws = s.nws; d.word_bits = s.word_bits;

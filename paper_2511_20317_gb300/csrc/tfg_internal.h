@@ -38,20 +38,21 @@ struct SegDesc {
     int32_t walk_policy;  // 0: plateau plus transitions; 1: Algorithm 1 expansions
     uint32_t expand_thresh;
     int32_t pad3;
-    int64_t all_walkers;  // of all populations, whose kernels share the GPU
+    int64_t beside;       // walkers of the populations whose kernels run at the same time, this one's included
 };
 
 // Lanes of a warp that hold walkers, for the kernels of one walker per thread: the fewest (a
-// power of two) at which all populations together make at most `warps` warps, 32 when
-// no fewer do.  A warp's step takes the path of every lane and its loops the turns of the
+// power of two) at which the populations running together make at most `warps` warps, 32
+// when no fewer do.  A warp's step takes the path of every lane and its loops the turns of the
 // longest, so a population too small to fill the GPU is spread over more warps.  Up to
 // eight warps an SM their steps hardly slow one another.  Measured, 500 steps, ms, 32
 // lanes / 16 / 8 / 4 / 2 / 1: (2,2,2) 1024 walkers 0.60 / 0.52 / 0.45 / 0.40 / 0.35 / 0.35,
 // 4096 0.60 / 0.53 / 0.48 / 0.46 / 0.50 / 0.74; (2,3,4) 1024 0.77 / 0.67 / 0.57 / 0.48 / 0.39 /
-// 0.36, 10000 0.77 / 0.73 / 0.70 / 1.03; (4,4,5) 1024 1.36 / 1.17 / 0.99 / 0.80 / 0.65 / 0.60.
-constexpr int kSpreadWarps = 8;   // an SM
+// 0.36, 10000 0.77 / 0.73 / 0.70 / 1.03; (4,4,5) 1024 1.36 / 1.17 / 0.99 / 0.80 / 0.65 / 0.60;
+// policy 1, (2,4,5) Z_2 10000 2.46 / 1.96 / 1.87 / 2.66, 20000 2.81 / 2.68 / 3.76.
 int walk_lanes(const SegDesc &d, int64_t warps);
 int sm_count();
+inline int64_t spread_warps(const SegDesc &d) { return (int64_t)(d.walk_policy == 1 ? 9 : 8) * sm_count(); }
 
 // One compiled variant of the walk kernel.
 struct WalkVariant {

@@ -1003,7 +1003,7 @@ struct LinkShape {
 };
 inline LinkShape link_shape(const SegDesc &d, int grid, int block, size_t shared_bytes, size_t device_bytes) {
     auto lanes = [&](size_t bytes) {
-        return walk_lanes(d, std::min<int64_t>((int64_t)kSpreadWarps * sm_count(), link_resident(32 * bytes)));
+        return walk_lanes(d, std::min(spread_warps(d), link_resident(32 * bytes)));
     };
     const int ls = lanes(shared_bytes), lg = device_bytes ? lanes(device_bytes) : 32;
     const bool spread_device = 4 * lg <= ls && ls <= 8;
