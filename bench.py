@@ -28,7 +28,8 @@ sys.path.insert(0, ROOT)
 
 METRIC = "verified flips/sec and reductions per 1e9 flips at 1 GB300, learned vs uniform proposal"
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2511_20317_gb300", "csrc", f)
-               for f in ("walk_solo.cuh", "walk_group.cuh", "pterm.cuh", "walk_solo_zt32.cu", "walk_solo_z232.cu")]
+               for f in ("walk_link.cuh", "walk_thread.cuh", "walk_solo.cuh", "walk_group.cuh", "pterm.cuh",
+                         "walk_solo_zt32.cu", "walk_solo_z232.cu")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "walk_kernel_333_dram_traffic.txt")
 
 # Algorithmic integer work per walker-step (word operations on 32-bit words):
@@ -155,7 +156,7 @@ def mapping_name(pop):
     if pop["slots_per_lane"] == 0:
         return "warp per walker, shared-memory signature search"
     if pop["lanes"] == 1:
-        sliced = ", bit-sliced slot search" if pop.get("slice_len") else ""
+        sliced = ", bit-sliced slots or kept factor classes" if pop.get("slice_len") else ", kept factor classes"
         sliced += " (square factors compiled in)" if pop.get("square") else ""
         return f"thread per walker, {pop['slots_per_lane']} slots{sliced}, {pop['block_threads']} walkers per block"
     return f"{pop['lanes']} lanes x {pop['slots_per_lane']} slots, {pop['block_threads']} threads per block"

@@ -24,14 +24,14 @@
 // and 2); without it the plateau policy is compiled in alone.  CNT (window mode): lists
 // at any capacity, and every slot's number of matches (u, v and w) is kept too.
 //
-// What bounds it: the latency of a warp's step (550 to 1300 instructions, most of
-// them in the accepting lanes' short dependent loops, at 35% of the issue rate
-// with 7 to 9 warps an SM).  The kernel it replaces tested every slot in every
+// What bounds it: the latency of a warp's step (600 to 1300 instructions, most of them in
+// the accepting lanes' short dependent loops, 13 of 32 lanes active; at 62% of the issue
+// rate with 14 warps an SM, 35% with 7 to 9).  The kernel it replaces tested every slot in every
 // step (5500 instructions a warp-step at 83 slots, two thirds of the ALU pipe).
-// Measured, Z_T, steps/s before / now: (2,3,4) 65536 walkers 1.43e10 / 2.19e10, (3,3,4)
+// Measured, Z_T, steps/s before / now: (2,3,4) 65536 walkers 1.43e10 / 2.60e10, (3,3,4)
 // 40330 4.9e9 / 1.24e10, (3,4,5) 40330 4.3e9 / 1.12e10, (4,4,4) 80660 4.0e9 / 1.07e10,
 // (4,4,5) 80660 2.6e9 / 9.5e9; Z_2 (4,4,5) 2.4e9 / 6.8e9; Algorithm 1 policy (3,3,4)
-// 10007 walkers 6.9e8 / 2.5e9.
+// 10007 walkers 6.9e8 / 3.1e9; (2,2,2) 1024 walkers 8.9e8 / 1.7e9.
 //
 // Step order and every tie-break are those of the lane-group kernel and of the
 // CPU reference:
