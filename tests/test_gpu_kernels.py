@@ -331,3 +331,21 @@ def test_uniform_window_walk_in_few_lanes(fmt, nw):
     for x, y in zip(A.read_walkers(0, nw), B.read_walkers(0, nw)):
         assert np.array_equal(x, y)
     A.close(), B.close()
+
+
+def test_timeout_reaches_the_host_error_word():
+    """A completion wait that gives up raises from the call that made its own error word (in
+    host memory), and the next call is clean."""
+    import torch
+    from oracle import mlp
+    p = mlp.Params.random(np.random.default_rng(2))
+    blob = torch.from_numpy(np.frombuffer(p.blob(), dtype=np.uint8).copy()).cuda()
+    x = torch.zeros((1000, 32), dtype=torch.bfloat16, device="cuda")
+    want = tfg.tfg_mlp_score(blob, x)
+    tfg.tfg_test_set_wait_limit(0)
+    try:
+        with pytest.raises(tfg.TfgError):
+            tfg.tfg_mlp_score(blob, x)
+    finally:
+        tfg.tfg_test_set_wait_limit(-1)
+    assert torch.equal(tfg.tfg_mlp_score(blob, x), want)
