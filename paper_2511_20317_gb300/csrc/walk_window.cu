@@ -537,8 +537,9 @@ __device__ __forceinline__ void log_step(const WindowLog &log, int64_t w, const 
 // Bound by the latency of a step, most of it the walk over the counts (two slots a
 // word, 15 to 33 words a step on (4,4,4)).  Measured on (4,4,4), 262144 walkers: 2.17 ms a
 // step with a window kernel that lists all 256 rows and an apply kernel per step,
-// now 0.1 ms (20 steps, the last one by those kernels: 43.6, now 4.1 ms);
-// 4096 logged walkers (the training data), 500 steps: 28.4 ms, now 2.6.
+// now 0.1 ms (20 steps, the last one by those kernels: 43.6, now 2.55 ms);
+// 4096 logged walkers (the training data), 500 steps: 28.4 ms, now 2.6 with 32 walkers a
+// warp (the whole collection 5.2 ms; 4.6 with 4 walkers a warp).
 template <class Wd, int NW, bool GM>
 __global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int32_t steps, int32_t *__restrict__ choices,
                                                             int64_t choice_stride, WindowLog log) {
