@@ -284,9 +284,13 @@ __device__ __forceinline__ void window_of(const SegDesc &d, int64_t w, int lane,
             }
     }
     __syncwarp();
-    uint4 *dw = reinterpret_cast<uint4 *>(desc + (size_t)w * kWin);
-    const uint4 *sw = reinterpret_cast<const uint4 *>(srow);
-    for (int row = lane; row < K / 2; row += 32) dw[row] = sw[row];
+    uint2 *dw = desc + (size_t)w * kWin;
+    if (((uintptr_t)desc & 15u) == 0) {   // the scratch is; a dump's array may start at any 8 bytes
+        const uint4 *sw = reinterpret_cast<const uint4 *>(srow);
+        for (int row = lane; row < K / 2; row += 32) reinterpret_cast<uint4 *>(dw)[row] = sw[row];
+    } else {
+        for (int row = lane; row < K; row += 32) dw[row] = srow[row];
+    }
     if (feat) {
         __nv_bfloat16 *fw = feat + (size_t)w * kWin * kFeat;
         for (int row = lane; row < kWin; row += 32) {

@@ -349,3 +349,26 @@ def test_timeout_reaches_the_host_error_word():
     finally:
         tfg.tfg_test_set_wait_limit(-1)
     assert torch.equal(tfg.tfg_mlp_score(blob, x), want)
+
+
+@pytest.mark.parametrize("fmt,nw", [((2, 2, 2), 5), ((4, 4, 5), 33)])
+def test_window_dump_rows_at_an_8_byte_boundary(fmt, nw):
+    """The dump takes descriptors at any 8-byte boundary: the same rows and sizes as at a
+    16-byte one, nothing written before, after or past a window."""
+    import ctypes
+    import torch
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=5, params=tfg.tfg_default_params(plateau_len=100))
+    W.walk(200)
+    _, want, sizes = W.window_dump(features=False)
+    words = nw * tfg.WINDOW * 2
+    room = torch.full((words + 8,), -7, dtype=torch.int32, device="cuda")
+    kwin = torch.zeros(nw, dtype=torch.int32, device="cuda")
+    assert room.data_ptr() % 16 == 0
+    rc = tfg.lib().tfg_window_dump(W.ctx, None, ctypes.c_void_p(room.data_ptr() + 8), ctypes.c_void_p(kwin.data_ptr()))
+    assert rc == tfg.TFG_OK
+    W.sync()
+    got = room[2:2 + words].view(nw, tfg.WINDOW, 2)
+    inside = (torch.arange(tfg.WINDOW, device="cuda")[None, :, None] < sizes[:, None, None]).expand(-1, -1, 2)
+    assert torch.equal(kwin, sizes) and torch.equal(got[inside], want[inside]) and (got[~inside] == -7).all()
+    assert (room[:2] == -7).all() and (room[2 + words:] == -7).all()
+    W.close()
