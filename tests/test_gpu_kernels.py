@@ -372,3 +372,49 @@ def test_window_dump_rows_at_an_8_byte_boundary(fmt, nw):
     assert torch.equal(kwin, sizes) and torch.equal(got[inside], want[inside]) and (got[~inside] == -7).all()
     assert (room[:2] == -7).all() and (room[2 + words:] == -7).all()
     W.close()
+
+
+def _raised_start(fmt, seed=3):
+    """A scheme two expansions above the naive one, which walks without expansions come down from."""
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), 64)], seed=seed, params=tfg.tfg_default_params(plateau_len=2))
+    W.walk(8).sync()
+    info, slots, _ = W.read_walkers(0, 64)
+    W.close()
+    w = int(np.argmax(info["r"]))
+    assert info["r"][w] > naive_start(*fmt).shape[0]
+    return slots[w, : info["r"][w]]
+
+
+@pytest.mark.parametrize("mapping", [1, 32])
+@pytest.mark.parametrize("fmt,mode", [((2, 2, 3), 0), ((2, 3, 4), 1), ((3, 3, 4), 0), ((3, 3, 4), 1)])
+@pytest.mark.parametrize("L", [2**63 - 1, 2**63 - 700])
+def test_plateaus_beyond_the_step_counter(fmt, mode, L, mapping):
+    """A plateau length of 2^63 - 1 (never) and one just below: no expansion, over launches that
+    start before and after the first better scheme, with every kind of mapping."""
+    start, nw, steps = _raised_start(fmt), 70, 1800
+    if mode:
+        start = np.abs(start).astype(np.int8)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=18, params=tfg.tfg_default_params(plateau_len=L, mapping=mapping))
+    for part in (40, 760, 1000):
+        W.walk(part)
+    W.sync()
+    info, slots, best = W.read_walkers(0, nw)
+    ref = oracle.Walkers(fmt, start, np.arange(nw), seed=18, mode=mode, plateau_len=L).walk(steps, THREADS)
+    assert (ref.info["plus"] == 0).all() and (ref.info["best_t"] > 0).any()
+    assert_parity(info, slots, best, ref, range(nw), f"{fmt} mode {mode} plateau {L}")
+    W.close()
+
+
+def test_uniform_window_walk_without_plateaus():
+    """The joint launch of uniform window steps with a plateau length of 2^63 - 1."""
+    fmt, nw, steps, L = (3, 3, 4), 70, 900, 2**63 - 1
+    start = _raised_start(fmt)
+    W = tfg.Walkers([(fmt, 0, start, nw)], seed=19, params=tfg.tfg_default_params(plateau_len=L))
+    for part in (400, 500):
+        W.walk_window(part, policy=0)
+    W.sync()
+    info, slots, best = W.read_walkers(0, nw)
+    ref = oracle.Walkers(fmt, start, np.arange(nw), seed=19, plateau_len=L).walk_window(steps)
+    assert (ref.info["plus"] == 0).all() and (ref.info["best_t"] > 0).any()
+    assert_parity(info, slots, best, ref, range(nw), "window")
+    W.close()
