@@ -50,6 +50,14 @@ namespace dev {
 constexpr int kHashBits = 8;
 constexpr int kLane = 32;   // stride of a thread's rows in its warp's shared memory
 
+// The lanes of this thread's warp that hold walkers (the first ones), taken by all threads of
+// a block, of whole warps or of fewer than 32 threads, before those past the population
+// return.  Not read off the hardware where it is used: loading a walker runs loops of
+// different lengths, after which a warp need not be together.
+__device__ __forceinline__ unsigned walker_lanes(const SegDesc &d, int64_t w) {
+    return __ballot_sync(blockDim.x < 32 ? (1u << blockDim.x) - 1u : ~0u, w < d.n_walkers);
+}
+
 // all four bytes = the sign of byte B (compile-time) of x: a word of 0 or of ones
 template <int B>
 __device__ __forceinline__ uint32_t sign_spread(uint32_t x) {
@@ -541,7 +549,8 @@ struct LinkWalker {
     // requesting walker to its best buffer (coalesced stores).
     __device__ __forceinline__ void coop_snapshot(unsigned wmask, int lane, int nl, bool want, Wd *bestp) const {
         unsigned pend = __ballot_sync(wmask, want);
-        if constexpr (GM) __syncwarp(wmask);
+        if (pend == 0u) return;
+        __syncwarp(wmask);   // the slots as their owners left them, and (below) left alone until they are read
 #pragma unroll 1
         while (pend) {
             const int a = __ffs(pend) - 1;
@@ -564,6 +573,7 @@ struct LinkWalker {
                 }
             }
         }
+        __syncwarp(wmask);
     }
 
     // Expansion (Section 3.3.1): plus (three terms from the pair) or, under
@@ -874,12 +884,11 @@ struct LinkWalker {
         return true;
     }
 
-    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, int32_t steps) {
+    // wmask: walker_lanes
+    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, unsigned wmask, int32_t steps) {
         load(d, w);
+        __syncwarp(wmask);
         Wd *bestp = reinterpret_cast<Wd *>(d.best) + (size_t)w * R * NWS;
-        // threads past the population returned already; the live lanes of a
-        // warp are 0 .. nl-1 (walkers are assigned to consecutive threads)
-        const unsigned wmask = __activemask();
         const int lane = threadIdx.x & 31;
         const int nl = __popc(wmask);
         const int policy = PG ? d.walk_policy : 0;
@@ -944,11 +953,12 @@ template <int MODE, class Wd, int NW, bool GM, bool PG, bool LIST = false>
 __global__ void __launch_bounds__(kLinkMaxBlock, 3) walk_link_kernel(const SegDesc d, const int32_t steps) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned wmask = walker_lanes(d, w);
     if (w >= d.n_walkers) return;   // no block-wide barrier is used
     using LW = LinkWalker<MODE, Wd, NW, GM, PG, false, LIST>;
     LW wk;
     link_rows<LW, Wd>(wk, d, w, GM, smem_raw);
-    wk.run(d, w, steps);
+    wk.run(d, w, wmask, steps);
 }
 
 }  // namespace dev

@@ -549,6 +549,7 @@ __global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int
                                                             int64_t choice_stride, WindowLog log) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned wmask = walker_lanes(d, w);
     if (w >= d.n_walkers) return;   // no block-wide barrier is used
     using LW = LinkWalker<TFG_MODE_ZT, Wd, NW, GM, false, true>;
     using T = typename LW::T;
@@ -556,7 +557,7 @@ __global__ void __launch_bounds__(64, 7) window_walk_kernel(const SegDesc d, int
     link_rows<LW, Wd>(wk, d, w, GM, smem_raw);
     wk.load(d, w);
     Wd *bestp = reinterpret_cast<Wd *>(d.best) + (size_t)w * d.R * 2;
-    const unsigned wmask = __activemask();
+    __syncwarp(wmask);
     const int lane = threadIdx.x & 31;
     const int nl = __popc(wmask);
     U4 x = philox10((uint32_t)wk.t, (uint32_t)(wk.t >> 32), wk.wid, 0u, wk.key0, wk.key1);
