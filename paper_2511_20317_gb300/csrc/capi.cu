@@ -214,7 +214,8 @@ struct tfg_ctx {
             }
         d.key0 = (uint32_t)seed;
         d.key1 = (uint32_t)(seed >> 32);
-        d.plateau_len = prm.plateau_len;
+        // a plateau of 2^62 steps is never reached, and kernels may add one to a step counter
+        d.plateau_len = std::min<int64_t>(prm.plateau_len, (int64_t)1 << 62);
         d.refresh_thresh = prm.refresh_thresh;
         d.plus_attempts = prm.plus_attempts;
         d.plus_enabled = prm.plus_enabled;

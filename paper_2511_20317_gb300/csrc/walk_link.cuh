@@ -648,7 +648,7 @@ struct LinkWalker {
         best_r = H->best_r;
         t = H->t; best_t = H->best_t;
         t_zero = t - H->plateau - 1;
-        t_exp = plateau_end(d);
+        t_exp = t_zero + d.plateau_len;
         dig = H->digest; wid = H->walker_id;
         key0 = d.key0; key1 = d.key1;
         best_nnz = H->best_nnz;
@@ -702,14 +702,10 @@ struct LinkWalker {
         H->best_nnz = best_nnz;
     }
 
-    // t_zero + plateau_len; a plateau that the step counter cannot reach has no end
-    __device__ __forceinline__ int64_t plateau_end(const SegDesc &d) const {
-        return t_zero > INT64_MAX - d.plateau_len ? INT64_MAX : t_zero + d.plateau_len;
-    }
     // plateau := 0 by the step at t
     __device__ __forceinline__ void restart(const SegDesc &d) {
         t_zero = t;
-        t_exp = plateau_end(d);
+        t_exp = t + d.plateau_len;
     }
 
     // The sampled term of the next step, fetched ahead: its slot, its words and
