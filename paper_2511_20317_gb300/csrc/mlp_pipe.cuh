@@ -155,8 +155,10 @@ __device__ __forceinline__ void load_weights(const uint8_t *__restrict__ params,
                     const int c = 8 * kg + u;
                     float f = first ? b1[c] : b2[c];
                     if (first) f += __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(params)[31 * kHid + c]);
-                    const float hi = __bfloat162float(bf(f)), mid = __bfloat162float(bf(f - hi));
-                    f = piece == 0 ? hi : (piece == 1 ? mid : f - hi - mid);
+                    float hi = __bfloat162float(bf(f));
+                    if (isinf(hi)) hi = __bfloat162float(__float2bfloat16_rz(f));   // finite, unless f is not
+                    const float rest = isinf(hi) ? 0.f : f - hi, mid = __bfloat162float(bf(rest));
+                    f = piece == 0 ? hi : (piece == 1 ? mid : rest - mid);
                     h[u >> 1] |= (uint32_t)__bfloat16_as_ushort(bf(f)) << (16 * (u & 1));
                 }
             }

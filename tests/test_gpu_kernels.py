@@ -418,3 +418,30 @@ def test_uniform_window_walk_without_plateaus():
     assert (ref.info["plus"] == 0).all() and (ref.info["best_t"] > 0).any()
     assert_parity(info, slots, best, ref, range(nw), "window")
     W.close()
+
+
+@pytest.mark.parametrize("b2", [np.inf, -np.inf, 3.4e38, -3.4e38, 1e-3])
+def test_scores_with_an_extreme_bias(b2):
+    """An output bias of the second layer that is infinite, or finite beyond the largest BF16 value:
+    the score is the FP32 sum's.  Bound: the FP32 sum of 128 products and the bf16 flip of
+    a hidden unit, as for row scoring."""
+    import torch
+    from oracle import mlp
+    rng = np.random.default_rng(4)
+    p = mlp.Params.random(rng)
+    unit = 5
+    p.w3[unit] = np.float32(1e-32 if np.isfinite(b2) and abs(b2) > 1 else 0.5)
+    p.b2[unit] = np.float32(b2)
+    x = mlp.bf16_round(rng.integers(0, 9, size=(300, mlp.IN)).astype(np.float32))
+    y, _ = mlp.forward(p, x)
+    blob = torch.from_numpy(np.frombuffer(p.blob(), dtype=np.uint8).copy()).cuda()
+    xs = torch.from_numpy(mlp.bf16_bits(x).view(np.int16).copy()).cuda().view(torch.bfloat16)
+    got = tfg.tfg_mlp_score(blob, xs).cpu().numpy().astype(np.float64)
+    if np.isinf(y).any():
+        assert np.isinf(y).all() and np.array_equal(got, y)
+        return
+    z1 = mlp.bf16_round(x).astype(np.float64) @ p.W1 + p.b1
+    h1 = np.maximum(mlp.bf16_round(np.maximum(z1, 0)), 0).astype(np.float64)
+    path = np.abs(p.W2) @ np.abs(p.w3)
+    bound = 2 * ((h1 * 2.0 ** -8) * path).max(1) + 1e-5 * (1 + np.abs(y))
+    assert (np.abs(got - y) <= bound).all()
