@@ -347,6 +347,7 @@ void launch_replicate(const SegDesc &d, const void *start_words, int32_t r0, uin
 
 namespace {
 
+constexpr int64_t kWarpWords = 3072, kSlabWords = 40960;   // accumulators of a warp's tensor / a block's slab
 template <class Wd, bool BLOCK, int FB, bool WIDE>
 void verify_variant(const SegDesc &d, int64_t first, int64_t count, int slab_rows, int slab_words, int sms,
                     unsigned long long *fail, cudaStream_t st) {
@@ -354,7 +355,8 @@ void verify_variant(const SegDesc &d, int64_t first, int64_t count, int slab_row
     const int threads = BLOCK ? kVerifyTeam : kVerifyWarpBlock;
     const size_t smem = (size_t)teams * slab_words * 4;
     auto kernel = verify_best_kernel<Wd, BLOCK, FB, WIDE>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the most of any launch: another thread may be about to launch the same kernel with more
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabWords * 4);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     const int64_t blocks = std::min<int64_t>((count + teams - 1) / teams, (int64_t)sms * std::max(per_sm, 1));
@@ -374,7 +376,6 @@ void verify_teams(const SegDesc &d, int64_t first, int64_t count, unsigned long 
     // then leave room for several blocks on an SM); a block per walker beyond, in one
     // slab up to kSlabWords, else in even ones.  A slab of one u-index has at most 128 x
     // 128 entries.
-    constexpr int64_t kWarpWords = 3072, kSlabWords = 40960;
     // Few walkers (a collected best scheme): a block each, whose warps share the terms.
     if (words <= kWarpWords && !wide && count > 2 * sms) {
         verify_variant<Wd, false, FB, false>(d, first, count, lu, (int)words, sms, fail, st);

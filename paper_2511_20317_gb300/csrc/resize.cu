@@ -471,7 +471,10 @@ void launch_resize(const SegDesc &src, int64_t src_first, const SegDesc &dst, in
     if (count <= 0) return;
     const size_t smem = (size_t)2 * kMaxLT * sizeof(int16_t) + (plan.aux_rank > kResizeMaxTerms ? (size_t)0 : (size_t)plan.aux_rank * 2 * ((plan.lt_aux + 31) / 32) * 4) +
                         (size_t)dst.nws * dst.word_bits / 32 * 4 * kResizeThreads;
-    cudaFuncSetAttribute(resize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the most of any launch: another thread may be about to launch the kernel with more
+    constexpr int most_smem = 2 * kMaxLT * (int)sizeof(int16_t) + kResizeMaxTerms * 2 * (kMaxLT / 32) * 4 +
+                              2 * (kMaxLT / 32) * 4 * kResizeThreads;
+    cudaFuncSetAttribute(resize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);
     int dev = 0, sms = 1, per_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -445,3 +445,72 @@ def test_scores_with_an_extreme_bias(b2):
     path = np.abs(p.W2) @ np.abs(p.w3)
     bound = 2 * ((h1 * 2.0 ** -8) * path).max(1) + 1e-5 * (1 + np.abs(y))
     assert (np.abs(got - y) <= bound).all()
+
+
+def test_verification_from_two_threads():
+    """Two threads verify populations whose accumulators need different shared memory by the same
+    kernel: no call fails."""
+    import threading
+    import torch
+    from paper_2511_20317_gb300 import starts
+    errors = []
+    walkers = []
+    for fmt, start in (((6, 7, 9), starts.start_6_7_9()[1]), ((5, 5, 5), naive_start(5, 5, 5))):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            walkers.append((tfg.Walkers([(fmt, 0, start, 2)], seed=1, stream=st), torch.zeros(1, dtype=torch.int64, device="cuda")))
+    torch.cuda.synchronize()
+
+    def verify(W, fails):
+        import ctypes
+        torch.cuda.set_device(0)
+        for _ in range(2000):
+            if tfg.lib().tfg_verify_all_async(W.ctx, ctypes.c_void_p(fails.data_ptr())) != tfg.TFG_OK:
+                errors.append(tfg.lib().tfg_last_error())
+                return
+
+    threads = [threading.Thread(target=verify, args=a) for a in walkers]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert all(int(f.item()) == 0 for _, f in walkers)
+    for W, _ in walkers:
+        W.close()
+
+
+def test_resizes_from_two_threads():
+    """Two threads resize into populations whose terms need different shared memory: no call fails."""
+    import threading
+    import torch
+    errors, jobs = [], []
+    for src, dst, aux in (((2, 2, 2), (2, 2, 3), None), ((1, 1, 1), (8, 9, 9), (8, 9, 9))):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            W = tfg.Walkers([(src, 0, naive_start(*src), 4), (dst, 0, naive_start(*dst), 4)], seed=1, stream=st)
+        jobs.append((W, aux))
+    torch.cuda.synchronize()
+
+    def resize(W, aux):
+        torch.cuda.set_device(0)
+        try:
+            for _ in range(1000):
+                if aux:
+                    skipped = W.resize(tfg.TFG_RESIZE_PRODUCT, 0, 4, 4, aux=(aux, naive_start(*aux)))
+                else:
+                    skipped = W.resize(tfg.TFG_RESIZE_EXTEND, 0, 4, 4, axis=2)
+                assert skipped == 0
+        except Exception as e:
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=resize, args=a) for a in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for W, _ in jobs:
+        assert W.verify_all() == 0
+        W.close()
