@@ -112,7 +112,9 @@ struct WideWalker {
     __device__ __forceinline__ bool owns(int f) const { return (lane >> (FW - 1)) == f; }   // holds a word of factor f
     __device__ __forceinline__ bool fown() const { return lane < 3 * FW; }
 
+    bool live;   // these lanes have a walker; without one they hold zero terms and read no one's slots or classes
     __device__ __forceinline__ DF dget(int s) const {
+        if (!live) return DF{0ull, 0ull};
         return DF{W[(size_t)s * NWG + fq], ZT ? W[(size_t)s * NWG + TW + fq] : 0ull};
     }
     // res = a with factor f := a_f + b_f (neg: a_f - b_f); false when a
@@ -401,7 +403,7 @@ struct WideWalker {
         const DF dv = dget(s);
         int k0 = kNone, k1 = kNone, k2 = kNone;
         bool n1 = false, n2 = false;
-        int k = next(s, 0);
+        int k = on ? (int)next(s, 0) : s;
         bool act = on && k != s;
 #pragma unroll 1
         for (int n = 0; n < R && any(act); ++n) {
@@ -412,7 +414,7 @@ struct WideWalker {
             k = act ? (int)next(k, 0) : k;
             act = act && k != s;
         }
-        k = next(s, 1);
+        k = on ? (int)next(s, 1) : s;
         act = on && k0 == kNone && k1 == kNone && k != s;
 #pragma unroll 1
         for (int n = 0; n < R && any(act); ++n) {
@@ -618,7 +620,7 @@ struct WideWalker {
     // the sampled term's class sizes and members below it, one factor per lane 0 .. 2
     __device__ __forceinline__ void classes(int i, int &n0, int &n1, int &n2, int &mine_below) const {
         int n = 0, b = 0;
-        if (lane < 3) {
+        if (live && lane < 3) {
             int p = next(i, lane);
 #pragma unroll 1
             for (; n < R && p != i; ++n) {
@@ -631,9 +633,8 @@ struct WideWalker {
         mine_below = b;
     }
 
-    // live: the lanes have a walker (w); the others read the first walker's rows and take part
-    // in the warp's votes only
-    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, bool live, int32_t steps) {
+    // w: the walker; lanes without one take part in the warp's votes only
+    __device__ __forceinline__ void run(const SegDesc &d, int64_t w, int32_t steps) {
         fq = lane < 3 * FW ? lane : 0;
         tfg_walker_info *H = d.hdr + w;
         r = live ? min(max(H->r, 0), R) : 0;   // in range whatever a restored state holds
@@ -842,10 +843,10 @@ __global__ void __launch_bounds__(kWideBlock, 10) walk_wide_kernel(const SegDesc
     }
     wk.lane = wl % WW::G;
     wk.gb = wl - wk.lane;
-    const bool live = group < here;
-    const int a = live ? group : 0;
+    wk.live = group < here;
+    const int a = wk.live ? group : 0;
     wk.attach(at + bytes * a, slots + (size_t)a * words);
-    wk.run(d, first + a, live, steps);
+    wk.run(d, first + a, steps);
     if constexpr (!GM) {
         __syncwarp();
 #pragma unroll 1
