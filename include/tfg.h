@@ -444,7 +444,9 @@ int tfg_mlp_train_step(void *d_state, void *d_params, const uint16_t *d_x, const
  * candidate).  log (optional): chosen features with label 1 when the step
  * lowered the rank (always kept) or 0 (kept when a Philox draw of sub-stream
  * 256 is below neg_thresh), appended at d_count (device int64, caller-zeroed)
- * up to capacity entries.  With horizon H > 1 each walker keeps a ring of the
+ * up to capacity entries; d_count goes on counting, and what a full log has no
+ * room for is lost, the latest steps first: no entry it holds was appended by a
+ * step 256 or more after one whose entry was lost.  With horizon H > 1 each walker keeps a ring of the
  * features of its last H chosen candidates; a step that lowers the rank
  * appends (label 1, each with its own step) every ring entry chosen at steps
  * t - H + 1 .. t since the walker's previous such step, in step order, and

@@ -514,3 +514,21 @@ def test_resizes_from_two_threads():
     for W, _ in jobs:
         assert W.verify_all() == 0
         W.close()
+
+
+def test_a_full_log_keeps_the_earliest_steps():
+    """A log that fills up during uniform window steps of more walkers than reside at once: no entry
+    is of a step 256 or more after one that is lost.  A sixteenth of the steps is kept
+    (3750 a step, standard deviation 59; a step of which a tenth is missing counts as lost)."""
+    fmt, nw, steps = (4, 4, 4), 60001, 640
+    W = tfg.Walkers([(fmt, 0, naive_start(*fmt), nw)], seed=20, params=tfg.tfg_default_params(plateau_len=10**6))
+    W.walk(100)
+    log = tfg.TransitionLog(nw * 240 // 16, neg_thresh=2**28)
+    W.walk_window(steps, policy=0, log=log)
+    W.sync()
+    e = log.read()
+    assert len(e) == log.capacity < int(log.count.item())
+    kept = np.bincount(e["step"] - 100, minlength=steps)
+    lost = int(np.argmax(kept < 0.9 * nw / 16))
+    assert lost >= 128 and (kept[lost + 256:] == 0).all()
+    W.close()
