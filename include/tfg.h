@@ -71,7 +71,9 @@ typedef struct {
     int32_t block_threads;    /* CUDA block size, multiple of 32, at most 256 (default 256), of the
                                  lane-group kernels; a thread-per-walker kernel takes it as its
                                  walkers per block when a variant with that block size is compiled
-                                 for its capacity (else its compiled default; see tfg_launch_shape) */
+                                 for its capacity (else its compiled default, and fewer walkers
+                                 a block for a population too small to fill the GPU; see
+                                 tfg_launch_shape) */
     uint32_t walker_id_base;  /* global id of this context's first walker (sharding across GPUs) */
     int32_t use_graph;        /* tfg_walk launches one captured CUDA graph of all populations' kernels:
                                  1 chained (default), 2 forked onto one stream per population

@@ -43,6 +43,7 @@ struct Segment {
     size_t off_hdr = 0, off_slots = 0, off_best = 0, off_start = 0;
     const tfg::WalkVariant *var = nullptr;
     int block = 0;   // threads per block for variants whose block size the caller chooses (0: default)
+    bool own_block = false;   // the variant's block size was chosen (block_threads, or by the autotuner)
     std::vector<int8_t> start_rows;
 };
 
@@ -221,6 +222,7 @@ struct tfg_ctx {
         d.plus_enabled = prm.plus_enabled;
         d.walk_policy = prm.walk_policy;
         d.expand_thresh = prm.expand_thresh;
+        d.own_block = s.own_block ? 1 : 0;
         return d;
     }
     Aux *aux() const { return reinterpret_cast<Aux *>(ws); }
@@ -408,6 +410,7 @@ static int plan_segments(int32_t n_formats, const tfg_format *fmts, const int32_
         s.var = prm.mapping ? pick_variant(s.fmt.mode, s.word_bits, s.tw, prm.mapping, s.R, s.fmt, true)
                             : default_variant(s.fmt.mode, s.word_bits, s.tw, s.R, s.fmt, s.n, prm.walk_policy);
         s.var = with_block(s.var, prm.block_threads);
+        s.own_block = s.var && s.var->block == prm.block_threads;
         if (!s.var) { set_error("no compiled kernel variant for this format/rank/mapping"); return TFG_EINVAL; }
     }
     *bytes = off;
@@ -688,7 +691,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
     // capacity, and for each every walkers-per-block choice (the block sizes compiled for a
     // thread-per-walker kernel of that capacity, whose shared memory per block depends on it;
     // 128 or 256 threads for the lane-group kernels)
-    struct Choice { const tfg::WalkVariant *var; int block; };
+    struct Choice { const tfg::WalkVariant *var; int block; bool own_block; };
     std::vector<std::vector<Choice>> cand(P);
     static const int lanes[5] = {1, 4, 8, 16, 32};
     for (size_t f = 0; f < P; ++f) {
@@ -701,8 +704,8 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
                 if (v.mode != base->mode || v.word_bits != base->word_bits || v.tw != base->tw || v.G != base->G ||
                     v.capacity() != base->capacity() || v.fl != base->fl || v.sq != base->sq)
                     continue;
-                if (v.block) cand[f].push_back({&v, 0});
-                else { cand[f].push_back({&v, 128}); cand[f].push_back({&v, 256}); }
+                if (v.block) cand[f].push_back({&v, 0, &v != base || v.block == ctx->prm.block_threads});
+                else { cand[f].push_back({&v, 128, false}); cand[f].push_back({&v, 256, false}); }
             }
         }
     }
@@ -744,7 +747,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
     for (size_t f = 0; f < P; ++f) {
         Segment &s = ctx->segs[f];
         if (full_n[f] == 0 || cand[f].empty()) continue;
-        const Choice cur{s.var, s.block};
+        const Choice cur{s.var, s.block, s.own_block};
         float base_ms = -1.f;
         if (trial((int32_t)std::min<int64_t>(trial_steps, 64)) < 0.f || restore_state() != cudaSuccess ||
             (base_ms = trial((int32_t)trial_steps)) < 0.f) {
@@ -757,12 +760,14 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
             if (c.var == cur.var && c.block == cur.block) continue;
             s.var = c.var;
             s.block = c.block;
+            s.own_block = c.own_block;
             float ms = trial((int32_t)std::min<int64_t>(trial_steps, 64));   // warm-up (first launch of a kernel)
             if (ms >= 0.f && restore_state() != cudaSuccess) ms = -1.f;
             if (ms >= 0.f) ms = trial((int32_t)trial_steps);
             if (ms < 0.f) {
                 s.var = cur.var;
                 s.block = cur.block;
+                s.own_block = cur.own_block;
                 restore_n();
                 return cuda_fail(cudaGetLastError(), "autotune trial");
             }
@@ -771,6 +776,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
         if (!(best_ms < 0.99f * base_ms)) best = cur;
         s.var = best.var;
         s.block = best.block;
+        s.own_block = best.own_block;
         if (lanes_out) lanes_out[f] = best.var->G;
     }
     restore_n();

@@ -37,7 +37,7 @@ struct SegDesc {
     int32_t fbase[3];     // bit offset of factor u, v, w in a packed term
     int32_t walk_policy;  // 0: plateau plus transitions; 1: Algorithm 1 expansions
     uint32_t expand_thresh;
-    int32_t pad3;
+    int32_t own_block;    // 1: the walkers per block were chosen, and are kept (0: a small population spreads out)
     int64_t beside;       // walkers of the populations whose kernels run at the same time, this one's included
 };
 

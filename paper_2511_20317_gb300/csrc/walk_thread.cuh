@@ -82,7 +82,8 @@ void launch_walk_sliced_zt(const SegDesc &d, int32_t steps, int grid, int block,
     if (slices_faster(d))
         launch_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>(d, steps, grid, block, st);
     else
-        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, (int)((d.n_walkers + 31) / 32), 32, st);
+        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, d.own_block ? grid : (int)((d.n_walkers + 31) / 32),
+                                             d.own_block ? block : 32, st);
 }
 
 }  // namespace tfg

@@ -532,3 +532,48 @@ def test_a_full_log_keeps_the_earliest_steps():
     lost = int(np.argmax(kept < 0.9 * nw / 16))
     assert lost >= 128 and (kept[lost + 256:] == 0).all()
     W.close()
+
+
+def _launches(call):
+    """(name, threads per block, blocks) of the walk kernels that call() launches."""
+    import json
+    import tempfile
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]):   # a process's first session may miss launches
+        torch.zeros(1, device="cuda").add_(1)
+        torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    with tempfile.TemporaryDirectory() as d:
+        prof.export_chrome_trace(os.path.join(d, "trace.json"))
+        with open(os.path.join(d, "trace.json")) as f:
+            events = json.load(f)["traceEvents"]
+    out = [(e["name"], int(np.prod(e["args"]["block"])), int(np.prod(e["args"]["grid"])))
+           for e in events if e.get("cat") == "kernel" and "walk_" in e["name"]]
+    if not out:
+        pytest.skip("no kernel records from the profiler here")
+    return out
+
+
+@pytest.mark.parametrize("fmt,block,mode", [((3, 3, 4), 96, 0), ((3, 4, 5), 128, 0), ((4, 4, 4), 128, 0), ((4, 4, 5), 160, 0),
+                                            ((4, 4, 5), 64, 0), ((4, 4, 5), 128, 1), ((3, 3, 3), 64, 0)])
+@pytest.mark.parametrize("nw", [700, 20001])
+def test_walkers_per_block_that_were_asked_for(fmt, block, mode, nw):
+    """block_threads that name a compiled choice are the walkers per block of the launch itself,
+    also of a population that would otherwise spread over more warps, and change no walk."""
+    start, steps, L = naive_start(*fmt), 400, 60
+    if mode:
+        start = np.abs(start).astype(np.int8)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=21,
+                    params=tfg.tfg_default_params(plateau_len=L, mapping=1, block_threads=block, use_graph=0))
+    launched = _launches(lambda: W.walk(steps // 4).walk(steps - steps // 4).sync())
+    assert {x[1:] for x in launched} == {(block, (nw + block - 1) // block)}
+    take = np.unique(np.linspace(0, nw - 1, 40).astype(int))
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=21, mode=mode, plateau_len=L).walk(steps, THREADS)
+    assert (ref.info["plus"] > 0).any()
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} block {block}")
+    W.close()
