@@ -350,9 +350,12 @@ int tfg_restore(tfg_ctx *ctx, const void *buf, size_t size);
  * per walker; tfg_launch_shape reports the whole launch shape.  Synchronous. */
 int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32_t *lanes_out);
 
-/* Launch shape of population f's walk kernel: lanes per walker, threads per
- * block (walkers per block = block_threads / lanes) and blocks.  Any output may
- * be NULL. */
+/* Launch shape of population f's walk kernel in a tfg_walk of many steps: lanes
+ * per walker, threads per block and blocks (walkers per block = block_threads /
+ * lanes, fewer where the wide-term kernel leaves lanes of a warp without a
+ * walker).  The lanes are tfg_mapping's but for the wide-term formats, whose
+ * one mapping (32) runs eight lanes per walker in populations large enough to
+ * keep factor classes.  Any output may be NULL. */
 int tfg_launch_shape(tfg_ctx *ctx, int32_t f, int32_t *lanes, int32_t *block_threads, int64_t *grid);
 
 /* Mapping chosen for population f: lanes per walker G, slots per lane S (the

@@ -794,9 +794,11 @@ int tfg_launch_shape(tfg_ctx *ctx, int32_t f, int32_t *lanes, int32_t *block_thr
     if (!ctx || f < 0 || f >= (int)ctx->segs.size()) { set_error("bad population index"); return TFG_EINVAL; }
     const Segment &s = ctx->segs[f];
     const int b = block_of(ctx, s);
-    if (lanes) *lanes = s.var->G;
-    if (block_threads) *block_threads = b;
-    if (grid) *grid = (s.n * s.var->G + b - 1) / b;
+    tfg::LaunchShape k{s.var->G, b, (s.n * s.var->G + b - 1) / b};
+    if (s.var->shape) k = s.var->shape(ctx->desc(s), b);
+    if (lanes) *lanes = k.lanes;
+    if (block_threads) *block_threads = k.block;
+    if (grid) *grid = k.grid;
     return TFG_OK;
 }
 

@@ -54,6 +54,12 @@ int walk_lanes(const SegDesc &d, int64_t warps);
 int sm_count();
 inline int64_t spread_warps(const SegDesc &d) { return (int64_t)(d.walk_policy == 1 ? 9 : 8) * sm_count(); }
 
+// A walk launch: lanes per walker, threads per block, blocks.
+struct LaunchShape {
+    int lanes, block;
+    int64_t grid;
+};
+
 // One compiled variant of the walk kernel.
 struct WalkVariant {
     int mode;       // TFG_MODE_ZT / TFG_MODE_Z2
@@ -65,6 +71,7 @@ struct WalkVariant {
     void (*launch)(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st);
     const void *kernel;  // for cudaFuncGetAttributes
     void (*prepare)();   // one-time kernel attribute set-up (may be null)
+    LaunchShape (*shape)(const SegDesc &d, int block) = nullptr;   // the shape that launch takes for many steps (null: G lanes a walker, `block` threads)
     int cap = 0;         // slot capacity when not given by G and S
     int fl = 0;          // > 0: formats whose factors have at most fl coefficients only (bit-sliced)
     int sq = 0;          // 1: formats whose three factors have exactly fl coefficients only

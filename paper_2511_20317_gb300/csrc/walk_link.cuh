@@ -1047,20 +1047,40 @@ inline bool link_lists_pay(const SegDesc &d, size_t rows_bytes, size_t lists_byt
     return d.walk_policy == 1 ? rows >= 2 * lists : 2 * rows >= 3 * lists;
 }
 
+struct LinkPlan {
+    LinkShape k;
+    bool lists;   // at most 32 slots: classes as lists
+};
 template <int MODE, class Wd, int NW>
-void launch_walk_link(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
-    prepare_walk_link<MODE, Wd, NW>();
+LinkPlan link_plan(const SegDesc &d, int block) {
     using Shared = dev::LinkWalker<MODE, Wd, NW, false, false>;
     using Device = dev::LinkWalker<MODE, Wd, NW, true, false>;
+    const int grid = (int)((d.n_walkers + block - 1) / block);
     const LinkShape k = link_shape(d, grid, block, Shared::thread_bytes(d.R),
                                    sizeof(Wd) == 8 ? Device::thread_bytes(d.R) : (size_t)0);
     if constexpr (NW == 1 && sizeof(Wd) == 4) {
         const size_t lists = dev::LinkWalker<MODE, Wd, NW, false, false, false, true>::thread_bytes(d.R) * block;
-        if (k.block == block && link_lists_pay(d, k.smem, lists, grid, block)) {
+        if (k.block == block && link_lists_pay(d, k.smem, lists, grid, block)) return {{grid, block, true, lists}, true};
+    }
+    return {k, false};
+}
+template <int MODE, class Wd, int NW>
+LaunchShape link_launch_shape(const SegDesc &d, int block) {
+    const LinkShape k = link_plan<MODE, Wd, NW>(d, block).k;
+    return {1, k.block, k.grid};
+}
+
+template <int MODE, class Wd, int NW>
+void launch_walk_link(const SegDesc &d, int32_t steps, int /*grid*/, int block, cudaStream_t st) {
+    prepare_walk_link<MODE, Wd, NW>();
+    const LinkPlan plan = link_plan<MODE, Wd, NW>(d, block);
+    const LinkShape &k = plan.k;
+    if constexpr (NW == 1 && sizeof(Wd) == 4) {
+        if (plan.lists) {
             if (d.walk_policy == 0)
-                dev::walk_link_kernel<MODE, Wd, NW, false, false, true><<<grid, block, lists, st>>>(d, steps);
+                dev::walk_link_kernel<MODE, Wd, NW, false, false, true><<<k.grid, k.block, k.smem, st>>>(d, steps);
             else
-                dev::walk_link_kernel<MODE, Wd, NW, false, true, true><<<grid, block, lists, st>>>(d, steps);
+                dev::walk_link_kernel<MODE, Wd, NW, false, true, true><<<k.grid, k.block, k.smem, st>>>(d, steps);
             return;
         }
     }

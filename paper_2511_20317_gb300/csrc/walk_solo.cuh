@@ -1094,8 +1094,7 @@ void prepare_walk_solo() {
 }
 
 template <int MODE, class Wd, int RMAX, int BT, int FL = 0, bool SQ = false>
-void launch_walk_solo(const SegDesc &d, int32_t steps, int grid, int /*block*/, cudaStream_t st) {
-    prepare_walk_solo<MODE, Wd, RMAX, BT, FL, SQ>();
+LaunchShape solo_shape(const SegDesc &d, int /*block*/) {
     // Small populations: one warp a block, walkers in few of its lanes; the rows are a full block's.
     // A step here is mostly the search, the same for every lane, so that a second warp on
     // a scheduler costs more than fewer lanes save: at most a warp a scheduler.  (16000
@@ -1106,14 +1105,21 @@ void launch_walk_solo(const SegDesc &d, int32_t steps, int grid, int /*block*/, 
     const int fit = std::min(4, (int)((size_t)227 * 1024 / (smem + 1024)));
     const int lanes = walk_lanes(d, (int64_t)fit * sm_count());
     const int block = lanes < 32 ? lanes : BT;
-    if (lanes < 32) grid = (int)((d.n_walkers + lanes - 1) / lanes);
-    dev::solo_kernel<MODE, Wd, RMAX, BT, FL, SQ>()<<<grid, block, smem, st>>>(d, steps);
+    return {1, block, (d.n_walkers + block - 1) / block};
+}
+
+template <int MODE, class Wd, int RMAX, int BT, int FL = 0, bool SQ = false>
+void launch_walk_solo(const SegDesc &d, int32_t steps, int /*grid*/, int block, cudaStream_t st) {
+    prepare_walk_solo<MODE, Wd, RMAX, BT, FL, SQ>();
+    const LaunchShape k = solo_shape<MODE, Wd, RMAX, BT, FL, SQ>(d, block);
+    dev::solo_kernel<MODE, Wd, RMAX, BT, FL, SQ>()<<<(unsigned)k.grid, k.block,
+                                                     solo_smem_bytes<MODE, Wd, RMAX, BT, FL>(), st>>>(d, steps);
 }
 
 // bit-sliced: formats whose factors have at most FL coefficients (SQ: exactly FL each)
 #define TFG_SOLO_SLICED_VARIANT(MODE, WD, BITS, RMAX, BT, FL, SQ) \
     WalkVariant{MODE, BITS, 1, 1, RMAX, BT, &launch_walk_solo<MODE, WD, RMAX, BT, FL, SQ>, \
                 reinterpret_cast<const void *>(dev::solo_kernel<MODE, WD, RMAX, BT, FL, SQ>()), \
-                &prepare_walk_solo<MODE, WD, RMAX, BT, FL, SQ>, 0, FL, SQ ? 1 : 0}
+                &prepare_walk_solo<MODE, WD, RMAX, BT, FL, SQ>, &solo_shape<MODE, WD, RMAX, BT, FL, SQ>, 0, FL, SQ ? 1 : 0}
 
 }  // namespace tfg

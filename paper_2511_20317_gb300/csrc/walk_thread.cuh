@@ -50,10 +50,16 @@ void prepare_walk_thread() {
 }
 
 template <int MODE, class Wd, int CAP>
+LaunchShape thread_shape(const SegDesc &d, int block) {
+    if constexpr (has_every_slot<MODE, Wd, CAP>())
+        if (every_slot_faster<MODE, Wd>(d)) return solo_shape<MODE, Wd, CAP, 128>(d, block);
+    return link_launch_shape<MODE, Wd, (CAP + 31) / 32>(d, block);
+}
+template <int MODE, class Wd, int CAP>
 void launch_walk_thread(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
     if constexpr (has_every_slot<MODE, Wd, CAP>()) {
         if (every_slot_faster<MODE, Wd>(d)) {
-            launch_walk_solo<MODE, Wd, CAP, 128>(d, steps, (int)((d.n_walkers + 127) / 128), 128, st);
+            launch_walk_solo<MODE, Wd, CAP, 128>(d, steps, grid, block, st);
             return;
         }
     }
@@ -77,13 +83,18 @@ void prepare_walk_sliced_zt() {
     prepare_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>();
     prepare_walk_link<TFG_MODE_ZT, Wd, 1>();
 }
+inline int sliced_class_block(const SegDesc &d, int block) { return d.own_block ? block : 32; }
+template <class Wd, int BT, int FL, bool SQ>
+LaunchShape sliced_zt_shape(const SegDesc &d, int block) {
+    if (slices_faster(d)) return solo_shape<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>(d, block);
+    return link_launch_shape<TFG_MODE_ZT, Wd, 1>(d, sliced_class_block(d, block));
+}
 template <class Wd, int BT, int FL, bool SQ>
 void launch_walk_sliced_zt(const SegDesc &d, int32_t steps, int grid, int block, cudaStream_t st) {
     if (slices_faster(d))
         launch_walk_solo<TFG_MODE_ZT, Wd, 32, BT, FL, SQ>(d, steps, grid, block, st);
     else
-        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, d.own_block ? grid : (int)((d.n_walkers + 31) / 32),
-                                             d.own_block ? block : 32, st);
+        launch_walk_link<TFG_MODE_ZT, Wd, 1>(d, steps, grid, sliced_class_block(d, block), st);
 }
 
 }  // namespace tfg
@@ -92,15 +103,15 @@ void launch_walk_sliced_zt(const SegDesc &d, int32_t steps, int grid, int block,
 #define TFG_THREAD_VARIANT(MODE, WD, BITS, CAP, BLOCK) \
     WalkVariant{MODE, BITS, 1, 1, CAP, BLOCK, &launch_walk_thread<MODE, WD, CAP>, \
                 reinterpret_cast<const void *>(&dev::walk_link_kernel<MODE, WD, (CAP + 31) / 32, BITS == 64, false>), \
-                &prepare_walk_thread<MODE, WD, CAP>}
+                &prepare_walk_thread<MODE, WD, CAP>, &thread_shape<MODE, WD, CAP>}
 // 32-bit terms beyond 32 slots: not selectable by tfg_params.mapping, and by default for large
 // populations (default_variant)
 #define TFG_THREAD_VARIANT_AUTO(MODE, WD, BITS, CAP, BLOCK) \
     WalkVariant{MODE, BITS, 1, 1, CAP, BLOCK, &launch_walk_link<MODE, WD, (CAP + 31) / 32>, \
                 reinterpret_cast<const void *>(&dev::walk_link_kernel<MODE, WD, (CAP + 31) / 32, BITS == 64, false>), \
-                &prepare_walk_link<MODE, WD, (CAP + 31) / 32>, 0, 0, 0, true}
+                &prepare_walk_link<MODE, WD, (CAP + 31) / 32>, &link_launch_shape<MODE, WD, (CAP + 31) / 32>, 0, 0, 0, true}
 // Z_T bit-sliced, 32 slots: factors of at most FL coefficients (SQ: exactly FL each)
 #define TFG_SLICED_ZT_VARIANT(WD, BITS, BT, FL, SQ) \
     WalkVariant{TFG_MODE_ZT, BITS, 1, 1, 32, BT, &launch_walk_sliced_zt<WD, BT, FL, SQ>, \
                 reinterpret_cast<const void *>(dev::solo_kernel<TFG_MODE_ZT, WD, 32, BT, FL, SQ>()), \
-                &prepare_walk_sliced_zt<WD, BT, FL, SQ>, 0, FL, SQ ? 1 : 0}
+                &prepare_walk_sliced_zt<WD, BT, FL, SQ>, &sliced_zt_shape<WD, BT, FL, SQ>, 0, FL, SQ ? 1 : 0}

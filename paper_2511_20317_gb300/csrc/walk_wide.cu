@@ -897,6 +897,29 @@ bool classes_pay(const SegDesc &d, int32_t steps) {
 // warp takes the changing part of a step when any of its walkers does, so a lone
 // walker's step is shorter.  The terms go to shared memory when the whole population
 // resides at once that way.
+struct WidePlan {
+    int per;   // walkers per warp
+    unsigned grid;
+    bool shared;
+    size_t smem;
+};
+template <int MODE, int FW>
+WidePlan wide_plan(const SegDesc &d) {
+    using Shared = dev::WideWalker<MODE, false, FW, false>;
+    using Device = dev::WideWalker<MODE, false, FW, true>;
+    int per = 32 / Shared::G;
+    while (per > 1 && (d.n_walkers + per - 1) / per < (int64_t)sm_count() * 8) per /= 2;
+    const int walkers = dev::kWideBlock / 32 * per;   // of a block
+    const unsigned grid = (unsigned)((d.n_walkers + walkers - 1) / walkers);
+    const bool shared = link_terms_shared(Shared::walker_bytes(d.R) * walkers, grid);
+    return {per, grid, shared, (shared ? Shared::walker_bytes(d.R) : Device::walker_bytes(d.R)) * walkers};
+}
+template <int MODE, int FW>
+LaunchShape wide_shape(const SegDesc &d, int /*block*/) {
+    if (!classes_pay<MODE>(d, INT32_MAX)) return search_shape(d);
+    return {dev::WideWalker<MODE, false, FW, true>::G, dev::kWideBlock, wide_plan<MODE, FW>(d).grid};
+}
+
 template <int MODE, int FW>
 void launch_walk_wide(const SegDesc &d, int32_t steps, int /*grid*/, int /*block*/, cudaStream_t st) {
     if (!classes_pay<MODE>(d, steps)) {
@@ -904,24 +927,14 @@ void launch_walk_wide(const SegDesc &d, int32_t steps, int /*grid*/, int /*block
         return;
     }
     prepare_walk_wide<MODE, FW>();
-    using Shared = dev::WideWalker<MODE, false, FW, false>;
-    using Device = dev::WideWalker<MODE, false, FW, true>;
     if (d.n_walkers <= 0) return;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per = 32 / Shared::G;
-    while (per > 1 && (d.n_walkers + per - 1) / per < (int64_t)sms * 8) per /= 2;
-    const int walkers = dev::kWideBlock / 32 * per;   // of a block
-    const unsigned grid = (unsigned)((d.n_walkers + walkers - 1) / walkers);
-    const bool shared = link_terms_shared(Shared::walker_bytes(d.R) * walkers, grid);
-    const size_t smem = (shared ? Shared::walker_bytes(d.R) : Device::walker_bytes(d.R)) * walkers;
-    if (shared) {
-        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, false><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
-        else dev::walk_wide_kernel<MODE, true, FW, false><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+    const WidePlan k = wide_plan<MODE, FW>(d);
+    if (k.shared) {
+        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, false><<<k.grid, dev::kWideBlock, k.smem, st>>>(d, steps, k.per);
+        else dev::walk_wide_kernel<MODE, true, FW, false><<<k.grid, dev::kWideBlock, k.smem, st>>>(d, steps, k.per);
     } else {
-        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, true><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
-        else dev::walk_wide_kernel<MODE, true, FW, true><<<grid, dev::kWideBlock, smem, st>>>(d, steps, per);
+        if (d.walk_policy == 0) dev::walk_wide_kernel<MODE, false, FW, true><<<k.grid, dev::kWideBlock, k.smem, st>>>(d, steps, k.per);
+        else dev::walk_wide_kernel<MODE, true, FW, true><<<k.grid, dev::kWideBlock, k.smem, st>>>(d, steps, k.per);
     }
 }
 
@@ -930,7 +943,7 @@ template <int MODE, int FW>
 WalkVariant wide_variant() {
     return WalkVariant{MODE, 64, 3 * FW, 32, 0, 0, &launch_walk_wide<MODE, FW>,
                        reinterpret_cast<const void *>(&dev::walk_wide_kernel<MODE, false, FW, true>),
-                       &prepare_walk_wide<MODE, FW>, 1023};
+                       &prepare_walk_wide<MODE, FW>, &wide_shape<MODE, FW>, 1023};
 }
 
 }  // namespace

@@ -797,15 +797,19 @@ void prepare_walk_search() {
     (void)attr;
 }
 
+inline LaunchShape search_shape(const SegDesc &d) {
+    return {32, 32 * dev::kSearchWarps, (d.n_walkers + dev::kSearchWarps - 1) / dev::kSearchWarps};
+}
+
 template <int MODE, bool GW, int FW>
 void launch_search_as(const SegDesc &d, int32_t steps, cudaStream_t st) {
     const size_t smem = dev::search_walker_bytes<MODE, GW, FW>(d.R) * dev::kSearchWarps;
     if (d.n_walkers <= 0 || smem > (size_t)kSearchMaxSmem) return;
-    const int64_t grid = (d.n_walkers + dev::kSearchWarps - 1) / dev::kSearchWarps;
+    const LaunchShape k = search_shape(d);
     if (d.walk_policy == 0)
-        dev::walk_search_kernel<MODE, GW, false, FW><<<(unsigned)grid, 32 * dev::kSearchWarps, smem, st>>>(d, steps);
+        dev::walk_search_kernel<MODE, GW, false, FW><<<(unsigned)k.grid, k.block, smem, st>>>(d, steps);
     else
-        dev::walk_search_kernel<MODE, GW, true, FW><<<(unsigned)grid, 32 * dev::kSearchWarps, smem, st>>>(d, steps);
+        dev::walk_search_kernel<MODE, GW, true, FW><<<(unsigned)k.grid, k.block, smem, st>>>(d, steps);
 }
 
 template <int MODE, int FW>

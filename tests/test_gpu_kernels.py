@@ -577,3 +577,20 @@ def test_walkers_per_block_that_were_asked_for(fmt, block, mode, nw):
     assert (ref.info["plus"] > 0).any()
     assert_parity(info, slots, best, ref, range(take.size), f"{fmt} block {block}")
     W.close()
+
+
+@pytest.mark.parametrize("fmt,mode,nw,policy", [
+    ((2, 2, 2), 0, 300, 0), ((2, 3, 4), 0, 5001, 0), ((2, 3, 4), 1, 5001, 2), ((2, 3, 4), 0, 70001, 0), ((3, 3, 3), 0, 1001, 0),
+    ((3, 3, 3), 0, 10001, 0), ((3, 3, 3), 0, 70001, 0), ((3, 3, 3), 1, 10001, 0), ((2, 4, 4), 0, 1001, 0), ((2, 4, 4), 1, 20001, 0),
+    ((4, 4, 5), 0, 1001, 0), ((4, 4, 5), 0, 30001, 0), ((4, 4, 5), 1, 3001, 2), ((4, 5, 5), 0, 301, 0), ((4, 5, 5), 0, 5001, 0),
+])
+def test_the_launch_shape_is_the_launch(fmt, mode, nw, policy):
+    """Threads per block and blocks that population() reports (tfg_launch_shape) are those of the
+    walk's launch: small populations, every-slot, bit-sliced, class, lane-group and wide kernels."""
+    start = naive_start(*fmt)
+    if mode:
+        start = np.abs(start).astype(np.int8)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=22, params=tfg.tfg_default_params(walk_policy=policy, use_graph=0))
+    launched = _launches(lambda: W.walk(200).sync())
+    assert [x[1:] for x in launched] == [(W.pop[0]["block_threads"], W.pop[0]["grid"])]
+    W.close()
