@@ -342,7 +342,8 @@ int tfg_restore(tfg_ctx *ctx, const void *buf, size_t size);
  * depends on it; 128 or 256 threads for the lane-group kernels).  Population
  * by population, each candidate is timed for trial_steps steps on the first
  * min(walkers, trial_walkers) walkers of every population, all populations
- * launched as tfg_walk launches them (concurrently for use_graph 2) with the
+ * launched as tfg_walk launches them (concurrently for use_graph 2; the kernel
+ * and block size that tfg_walk takes for the whole population) with the
  * others at their current choice; a candidate replaces the current choice
  * when it is more than 1% faster.  The trial walkers' state is restored bit for
  * bit afterwards (host copies; no device memory is allocated); the choice

@@ -40,6 +40,7 @@ struct Segment {
     int r0 = 0, R = 0, word_bits = 32, lt = 0, tw = 1, nws = 2;
     int fbase[3] = {0, 0, 0};   // bit offset of each factor in a packed term
     int64_t n = 0, first = 0;
+    int64_t population = 0;   // n, also while an autotuner's trial cuts n
     size_t off_hdr = 0, off_slots = 0, off_best = 0, off_start = 0;
     const tfg::WalkVariant *var = nullptr;
     int block = 0;   // threads per block for variants whose block size the caller chooses (0: default)
@@ -198,7 +199,8 @@ struct tfg_ctx {
         d.best = ws + s.off_best;
         d.hdr = reinterpret_cast<tfg_walker_info *>(ws + s.off_hdr);
         d.n_walkers = s.n;
-        d.beside = prm.use_graph == 2 ? total : s.n;   // forked: all populations at once
+        d.population = s.population;
+        d.beside = prm.use_graph == 2 ? total : s.population;   // forked: all populations at once
         d.R = s.R;
         d.m = s.fmt.m; d.n = s.fmt.n; d.p = s.fmt.p;
         d.lt = s.lt; d.tw = s.tw; d.nws = s.nws; d.word_bits = s.word_bits;
@@ -402,7 +404,7 @@ static int plan_segments(int32_t n_formats, const tfg_format *fmts, const int32_
         s.R = ranks[f] + prm.r_slack;
         if (s.R > kMaxSlots) { set_error("rank + slack exceeds the supported 1023 slots"); return TFG_EINVAL; }
         set_geometry(s);
-        s.n = walkers[f];
+        s.n = s.population = walkers[f];
         s.first = first;
         first += s.n;
         if (first > (int64_t)UINT32_MAX) { set_error("more than 2^32 walkers"); return TFG_EINVAL; }
@@ -704,7 +706,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
                 if (v.mode != base->mode || v.word_bits != base->word_bits || v.tw != base->tw || v.G != base->G ||
                     v.capacity() != base->capacity() || v.fl != base->fl || v.sq != base->sq)
                     continue;
-                if (v.block) cand[f].push_back({&v, 0, &v != base || v.block == ctx->prm.block_threads});
+                if (v.block || v.shape) cand[f].push_back({&v, 0, &v != base || v.block == ctx->prm.block_threads});
                 else { cand[f].push_back({&v, 128, false}); cand[f].push_back({&v, 256, false}); }
             }
         }
@@ -724,12 +726,11 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
         return r;
     };
     // One timed trial: `steps` steps of the trial walkers through tfg_walk itself (the
-    // graph rebuilt for the current choices), so a trial is timed in the launch shape the
-    // walk uses: milliseconds, or < 0 on error.  The populations are cut to their trial
-    // walkers meanwhile.
-    std::vector<int64_t> full_n(P);
-    for (size_t f = 0; f < P; ++f) { full_n[f] = ctx->segs[f].n; ctx->segs[f].n = saved[f].nt; }
-    auto restore_n = [&] { for (size_t f = 0; f < P; ++f) ctx->segs[f].n = full_n[f]; };
+    // graph rebuilt for the current choices): milliseconds, or < 0 on error.  The populations
+    // are cut to their trial walkers meanwhile; kernel and launch shape go by the whole
+    // population, so a trial runs the kernel that the walk will, on a part of its walkers.
+    for (size_t f = 0; f < P; ++f) ctx->segs[f].n = saved[f].nt;
+    auto restore_n = [&] { for (Segment &s : ctx->segs) s.n = s.population; };
     auto trial = [&](int32_t steps) -> float {
         for (tfg_ctx::Graph &g : ctx->graphs) cudaGraphExecDestroy(g.exec);
         ctx->graphs.clear();
@@ -746,7 +747,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
     // when it is more than 1% faster
     for (size_t f = 0; f < P; ++f) {
         Segment &s = ctx->segs[f];
-        if (full_n[f] == 0 || cand[f].empty()) continue;
+        if (s.population == 0 || cand[f].empty()) continue;
         const Choice cur{s.var, s.block, s.own_block};
         float base_ms = -1.f;
         if (trial((int32_t)std::min<int64_t>(trial_steps, 64)) < 0.f || restore_state() != cudaSuccess ||

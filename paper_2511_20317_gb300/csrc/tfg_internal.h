@@ -38,7 +38,10 @@ struct SegDesc {
     int32_t walk_policy;  // 0: plateau plus transitions; 1: Algorithm 1 expansions
     uint32_t expand_thresh;
     int32_t own_block;    // 1: the walkers per block were chosen, and are kept (0: a small population spreads out)
-    int64_t beside;       // walkers of the populations whose kernels run at the same time, this one's included
+    // What the choice of kernel and launch shape goes by: the whole population (an
+    // autotuner's trial walks its first n_walkers only, as a part of the walk it stands for),
+    // and all populations whose kernels run at the same time, this one included.
+    int64_t population, beside;
 };
 
 // Lanes of a warp that hold walkers, for the kernels of one walker per thread: the fewest (a

@@ -1011,18 +1011,19 @@ struct LinkShape {
     bool shared;
     size_t smem;
 };
-inline LinkShape link_shape(const SegDesc &d, int grid, int block, size_t shared_bytes, size_t device_bytes) {
+inline LinkShape link_shape(const SegDesc &d, int block, size_t shared_bytes, size_t device_bytes) {
+    auto blocks = [&](int walkers) { return (int)((d.n_walkers + walkers - 1) / walkers); };
     auto lanes = [&](size_t bytes) {
         return walk_lanes(d, std::min(spread_warps(d), link_resident(32 * bytes)));
     };
     const int ls = lanes(shared_bytes), lg = device_bytes ? lanes(device_bytes) : 32;
     const bool spread_device = 4 * lg <= ls && ls <= 8;
     const bool shared = device_bytes == 0 ||
-                        (!spread_device && (ls < 32 || link_terms_shared(shared_bytes * block, grid)));
+                        (!spread_device && (ls < 32 || link_terms_shared(shared_bytes * block, (d.population + block - 1) / block)));
     const int l = shared ? ls : lg;
     const size_t bytes = shared ? shared_bytes : device_bytes;
-    if (l == 32) return {grid, block, shared, bytes * block};
-    return {(int)((d.n_walkers + l - 1) / l), l, shared, bytes * 32};
+    if (l == 32) return {blocks(block), block, shared, bytes * block};
+    return {blocks(l), l, shared, bytes * 32};
 }
 
 // At most 32 slots: classes as rows (12 bytes a slot) or as lists (4).  A row is read at
@@ -1036,7 +1037,8 @@ inline LinkShape link_shape(const SegDesc &d, int grid, int block, size_t shared
 // Z_2 (two / one) 12.0 / 10.1, policy 2 Z_T 65536 3.13 / 2.20; (2,3,3) 65536 Z_T (two /
 // one) 2.79 / 2.32, 262144 (five / four) 7.3 / 7.8; (2,2,6) Z_T 65536 (two / one) 3.16 /
 // 3.17, 131072 (three / two) 5.02 / 5.62.
-inline bool link_lists_pay(const SegDesc &d, size_t rows_bytes, size_t lists_bytes, int64_t grid, int block) {
+inline bool link_lists_pay(const SegDesc &d, size_t rows_bytes, size_t lists_bytes, int block) {
+    const int64_t grid = (d.population + block - 1) / block;
     const int shortest = std::min(d.m * d.n, std::min(d.n * d.p, d.p * d.m));
     if (shortest < 6) return false;
     auto waves = [&](size_t bytes) {   // of at most 16 warps an SM
@@ -1055,12 +1057,11 @@ template <int MODE, class Wd, int NW>
 LinkPlan link_plan(const SegDesc &d, int block) {
     using Shared = dev::LinkWalker<MODE, Wd, NW, false, false>;
     using Device = dev::LinkWalker<MODE, Wd, NW, true, false>;
-    const int grid = (int)((d.n_walkers + block - 1) / block);
-    const LinkShape k = link_shape(d, grid, block, Shared::thread_bytes(d.R),
+    const LinkShape k = link_shape(d, block, Shared::thread_bytes(d.R),
                                    sizeof(Wd) == 8 ? Device::thread_bytes(d.R) : (size_t)0);
     if constexpr (NW == 1 && sizeof(Wd) == 4) {
         const size_t lists = dev::LinkWalker<MODE, Wd, NW, false, false, false, true>::thread_bytes(d.R) * block;
-        if (k.block == block && link_lists_pay(d, k.smem, lists, grid, block)) return {{grid, block, true, lists}, true};
+        if (k.block == block && link_lists_pay(d, k.smem, lists, block)) return {{k.grid, block, true, lists}, true};
     }
     return {k, false};
 }

@@ -54,7 +54,7 @@ int sm_count() {
 
 int walk_lanes(const SegDesc &d, int64_t warps) {
     if (d.own_block) return 32;
-    const int64_t n = std::max(d.beside, d.n_walkers);
+    const int64_t n = std::max(d.beside, d.population);
     int lanes = 32;
     while (lanes > 1 && (n + lanes / 2 - 1) / (lanes / 2) <= warps) lanes /= 2;
     return lanes;

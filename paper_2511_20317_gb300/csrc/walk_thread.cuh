@@ -10,7 +10,7 @@ namespace tfg {
 // Lanes a warp would get if the population kept classes: few for a small one.
 inline int class_lanes(const SegDesc &d) { return walk_lanes(d, (int64_t)8 * sm_count()); }
 // At most a full warp a scheduler: a step's latency counts, not its instructions.
-inline bool one_warp_each(const SegDesc &d) { return d.n_walkers <= (int64_t)128 * sm_count(); }
+inline bool one_warp_each(const SegDesc &d) { return d.population <= (int64_t)128 * sm_count(); }
 
 // Keeping the classes pays when most steps only read them, and when the rank is large.
 // It does not when nearly every step changes the scheme and nothing else in the step

@@ -888,9 +888,9 @@ void prepare_walk_wide() {
 template <int MODE>
 bool classes_pay(const SegDesc &d, int32_t steps) {
     const bool large = d.R >= 256;
-    if (d.walk_policy == 0) return d.n_walkers >= 4000 && steps >= (large ? 120 : 40);
-    if (d.walk_policy == 2) return d.n_walkers >= 8000 && steps >= (large ? 200 : 60);
-    return d.n_walkers >= 8000 && steps >= 300 && (MODE == TFG_MODE_ZT || d.R >= 128);
+    if (d.walk_policy == 0) return d.population >= 4000 && steps >= (large ? 120 : 40);
+    if (d.walk_policy == 2) return d.population >= 8000 && steps >= (large ? 200 : 60);
+    return d.population >= 8000 && steps >= 300 && (MODE == TFG_MODE_ZT || d.R >= 128);
 }
 
 // Walkers per warp: four, unless that leaves an SM's schedulers without two warps each; a
@@ -908,10 +908,10 @@ WidePlan wide_plan(const SegDesc &d) {
     using Shared = dev::WideWalker<MODE, false, FW, false>;
     using Device = dev::WideWalker<MODE, false, FW, true>;
     int per = 32 / Shared::G;
-    while (per > 1 && (d.n_walkers + per - 1) / per < (int64_t)sm_count() * 8) per /= 2;
+    while (per > 1 && (d.population + per - 1) / per < (int64_t)sm_count() * 8) per /= 2;
     const int walkers = dev::kWideBlock / 32 * per;   // of a block
     const unsigned grid = (unsigned)((d.n_walkers + walkers - 1) / walkers);
-    const bool shared = link_terms_shared(Shared::walker_bytes(d.R) * walkers, grid);
+    const bool shared = link_terms_shared(Shared::walker_bytes(d.R) * walkers, (d.population + walkers - 1) / walkers);
     return {per, grid, shared, (shared ? Shared::walker_bytes(d.R) : Device::walker_bytes(d.R)) * walkers};
 }
 template <int MODE, int FW>

@@ -828,7 +828,7 @@ static void window_walk_variant(const SegDesc &d, int32_t steps, int32_t *choice
     (void)attr;
     SegDesc free = d;
     free.own_block = 0;   // the walkers per block of tfg_walk
-    const LinkShape k = link_shape(free, (int)((d.n_walkers + kBlock - 1) / kBlock), kBlock, Shared::thread_bytes(d.R),
+    const LinkShape k = link_shape(free, kBlock, Shared::thread_bytes(d.R),
                                    sizeof(Wd) == 8 ? Device::thread_bytes(d.R) : (size_t)0);
     if (k.shared) {
         dev::window_walk_kernel<Wd, NW, false><<<k.grid, k.block, k.smem, st>>>(d, steps, choices, stride, log);

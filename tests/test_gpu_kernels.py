@@ -594,3 +594,19 @@ def test_the_launch_shape_is_the_launch(fmt, mode, nw, policy):
     launched = _launches(lambda: W.walk(200).sync())
     assert [x[1:] for x in launched] == [(W.pop[0]["block_threads"], W.pop[0]["grid"])]
     W.close()
+
+
+@pytest.mark.parametrize("fmt,mode,nw,policy", [((2, 2, 2), 0, 20001, 0), ((2, 3, 4), 0, 70001, 0), ((3, 3, 3), 0, 70001, 0),
+                                                ((3, 3, 3), 0, 10001, 1), ((2, 3, 4), 0, 20001, 2), ((4, 4, 5), 0, 30001, 0)])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_the_autotuner_times_the_kernel_of_the_walk(fmt, mode, nw, policy, graph):
+    """A trial on a few of a population's walkers runs the kernel, at the threads per block, that
+    the whole population's walk runs before it, and the choice's walk runs one that a trial ran."""
+    start = naive_start(*fmt)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=23, params=tfg.tfg_default_params(walk_policy=policy, use_graph=graph))
+    before = _launches(lambda: W.walk(100).sync())
+    trials = _launches(lambda: W.autotune(trial_steps=100, trial_walkers=1024))
+    after = _launches(lambda: W.walk(100).sync())
+    assert trials[0][:2] == before[0][:2] and trials[0][2] == -(-1024 // before[0][1])
+    assert after[0][:2] in [x[:2] for x in trials]
+    W.close()
