@@ -338,14 +338,15 @@ int tfg_restore(tfg_ctx *ctx, const void *buf, size_t size);
 /* Autotuner: the candidates of a population are its compiled kernel variants
  * -- every mapping (one thread per walker; 4, 8, 16 or 32 lanes per walker) and,
  * for each, every walkers-per-block choice (the block sizes compiled for the
- * thread-per-walker kernel of that capacity, whose shared memory per block
- * depends on it; 128 or 256 threads for the lane-group kernels).  Population
+ * thread-per-walker kernel of that capacity, when trial_walkers covers the
+ * population; 128 or 256 threads for the lane-group kernels).  Population
  * by population, each candidate is timed for trial_steps steps on the first
  * min(walkers, trial_walkers) walkers of every population, all populations
  * launched as tfg_walk launches them (concurrently for use_graph 2; the kernel
  * and block size that tfg_walk takes for the whole population) with the
- * others at their current choice; a candidate replaces the current choice
- * when it is more than 1% faster.  The trial walkers' state is restored bit for
+ * others at their current choice; of a larger population the time is
+ * extrapolated from the trial and its first half.  A candidate replaces the
+ * current choice when it is more than 1% faster (5% when extrapolated).  The trial walkers' state is restored bit for
  * bit afterwards (host copies; no device memory is allocated); the choice
  * changes no trajectory.  lanes_out[f] (optional) receives the chosen lanes
  * per walker; tfg_launch_shape reports the whole launch shape.  Synchronous. */

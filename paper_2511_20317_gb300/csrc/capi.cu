@@ -691,7 +691,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
     }
     // candidates of every population: every mapping (lanes per walker) at its smallest
     // capacity, and for each every walkers-per-block choice (the block sizes compiled for a
-    // thread-per-walker kernel of that capacity, whose shared memory per block depends on it;
+    // thread-per-walker kernel of that capacity, when the trial is the whole population;
     // 128 or 256 threads for the lane-group kernels)
     struct Choice { const tfg::WalkVariant *var; int block; bool own_block; };
     std::vector<std::vector<Choice>> cand(P);
@@ -706,6 +706,10 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
                 if (v.mode != base->mode || v.word_bits != base->word_bits || v.tw != base->tw || v.G != base->G ||
                     v.capacity() != base->capacity() || v.fl != base->fl || v.sq != base->sq)
                     continue;
+                // Walkers per block matter by what resides and by how the last blocks fall, which a
+                // part of the population does not show ((4,4,5) Z_T, 262144 walkers: 128 a block won
+                // on 16384 of them and took 26.4 ms where 64 take 24.1).
+                if (&v != base && v.block && s.population > saved[f].nt) continue;
                 if (v.block || v.shape) cand[f].push_back({&v, 0, &v != base || v.block == ctx->prm.block_threads});
                 else { cand[f].push_back({&v, 128, false}); cand[f].push_back({&v, 256, false}); }
             }
@@ -742,16 +746,42 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
         cudaEventElapsedTime(&ms, ev.a, ev.b);
         return ms;
     };
+    // The time of trial_steps steps with population f's current choice, or < 0 on error.  Of
+    // a population larger than its trial: the trial's, and what its second half added to it
+    // for each further walker.  A part of the population need not fill the GPU, and lanes that
+    // share a walker's step are the faster exactly while it does not (Algorithm 1 policy, (3,3,3)
+    // Z_2, 131072 walkers, steps timed on 16384: 16 lanes a walker chosen by the trial's time
+    // alone, 13.4 ms for 300 steps where one lane takes 9.4).
+    auto estimate = [&](size_t f) -> float {
+        Segment &s = ctx->segs[f];
+        const int64_t nt = saved[f].nt, half = nt / 2;
+        const bool part = s.population > nt && half > 0;
+        auto timed = [&](int64_t n) -> float {
+            float best = -1.f;
+            for (int k = 0; k < (part ? 2 : 1); ++k) {   // a difference of two times: the better of two each
+                if (restore_state() != cudaSuccess) return -1.f;
+                s.n = n;
+                const float ms = trial((int32_t)trial_steps);
+                s.n = nt;
+                if (ms < 0.f) return -1.f;
+                best = best < 0.f ? ms : std::min(best, ms);
+            }
+            return best;
+        };
+        if (trial((int32_t)std::min<int64_t>(trial_steps, 64)) < 0.f) return -1.f;   // warm-up (first launch of a kernel)
+        const float ms = timed(nt), less = part && ms >= 0.f ? timed(half) : ms;
+        if (ms < 0.f || less < 0.f) return -1.f;
+        return part ? ms + std::max(ms - less, 0.f) * (float)(s.population - nt) / (float)(nt - half) : ms;
+    };
     // coordinate descent: population by population, every candidate timed with the other
     // populations at their current choice; a candidate replaces the current choice only
-    // when it is more than 1% faster
+    // when it is more than 1% faster (5% where the time is extrapolated)
     for (size_t f = 0; f < P; ++f) {
         Segment &s = ctx->segs[f];
         if (s.population == 0 || cand[f].empty()) continue;
         const Choice cur{s.var, s.block, s.own_block};
-        float base_ms = -1.f;
-        if (trial((int32_t)std::min<int64_t>(trial_steps, 64)) < 0.f || restore_state() != cudaSuccess ||
-            (base_ms = trial((int32_t)trial_steps)) < 0.f) {
+        const float base_ms = estimate(f);
+        if (base_ms < 0.f) {
             restore_n();
             return cuda_fail(cudaGetLastError(), "autotune trial");
         }
@@ -762,9 +792,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
             s.var = c.var;
             s.block = c.block;
             s.own_block = c.own_block;
-            float ms = trial((int32_t)std::min<int64_t>(trial_steps, 64));   // warm-up (first launch of a kernel)
-            if (ms >= 0.f && restore_state() != cudaSuccess) ms = -1.f;
-            if (ms >= 0.f) ms = trial((int32_t)trial_steps);
+            const float ms = estimate(f);
             if (ms < 0.f) {
                 s.var = cur.var;
                 s.block = cur.block;
@@ -774,7 +802,7 @@ int tfg_autotune(tfg_ctx *ctx, int64_t trial_steps, int64_t trial_walkers, int32
             }
             if (ms < best_ms) { best_ms = ms; best = c; }
         }
-        if (!(best_ms < 0.99f * base_ms)) best = cur;
+        if (!(best_ms < (s.population > saved[f].nt ? 0.95f : 0.99f) * base_ms)) best = cur;
         s.var = best.var;
         s.block = best.block;
         s.own_block = best.own_block;

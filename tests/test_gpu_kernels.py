@@ -610,3 +610,14 @@ def test_the_autotuner_times_the_kernel_of_the_walk(fmt, mode, nw, policy, graph
     assert trials[0][:2] == before[0][:2] and trials[0][2] == -(-1024 // before[0][1])
     assert after[0][:2] in [x[:2] for x in trials]
     W.close()
+
+
+def test_the_autotuner_judges_the_whole_population():
+    """Sixteen lanes a walker are the fastest on a trial that leaves most of the GPU idle and take 1.4
+    times as long as one on the whole population: the choice is one."""
+    fmt, nw = (3, 3, 3), 131072
+    W = tfg.Walkers([(fmt, 1, np.abs(naive_start(*fmt)).astype(np.int8), nw)], seed=24,
+                    params=tfg.tfg_default_params(walk_policy=1, r_slack=6, expand_thresh=int(0.01 * 2**32)))
+    W.walk(500).sync()
+    assert W.autotune(trial_steps=300, trial_walkers=16384) == [1]
+    W.close()
