@@ -621,3 +621,34 @@ def test_the_autotuner_judges_the_whole_population():
     W.walk(500).sync()
     assert W.autotune(trial_steps=300, trial_walkers=16384) == [1]
     W.close()
+
+
+@pytest.mark.parametrize("fmt,mode,nw,policy,slack,kernel", [
+    *[((2, 4, 4), mode, nw, policy, 3, kernel) for mode in (0, 1) for nw, policy, kernel in
+      ((8193, 0, "walk_link"), (8191, 0, "walk_group"), (8193, 2, "walk_link"), (16385, 1, "walk_link"), (16383, 1, "walk_group"))],
+    ((2, 3, 5), 0, 8193, 0, 3, "walk_link"), ((2, 3, 5), 1, 8193, 2, 34, "walk_link"), ((2, 3, 5), 0, 16385, 1, 6, "walk_link"),
+    ((3, 3, 4), 1, 60001, 1, 6, "walk_link"), ((4, 4, 5), 1, 45001, 0, 3, "walk_link"),   # terms in device memory
+])
+def test_default_mapping_of_many_walkers(fmt, mode, nw, policy, slack, kernel):
+    """32-bit terms of more than 32 slots on either side of the population from which a thread takes
+    a walker by default, and Z_2 populations of more than reside at once, against the oracle."""
+    start, steps, L = naive_start(*fmt), 300, 60
+    if mode:
+        start = np.abs(start).astype(np.int8)
+    kw = dict(plateau_len=L if policy == 0 else 10**6, walk_policy=policy, r_slack=slack,
+              expand_thresh=int(0.03 * 2**32) if policy == 1 else 0)
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=25, params=tfg.tfg_default_params(use_graph=0, **kw))
+    launched = _launches(lambda: W.walk(steps // 2).walk(steps - steps // 2).sync())
+    assert all(kernel in x[0] for x in launched) and launched[0][1] == W.pop[0]["block_threads"]
+    if nw > 20000:   # the fourth template argument of the kernel: terms in the walker's device-memory slots
+        args = launched[0][0].split("<", 1)[1].split(",")
+        assert args[3].strip().replace("(bool)", "") in ("1", "true"), launched[0][0]
+    take = np.unique(np.concatenate([np.linspace(0, nw - 1, 40).astype(int), np.arange(nw - 4, nw)]))
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=25, mode=mode, plateau_len=kw["plateau_len"], r_slack=slack, policy=policy,
+                         expand_thresh=kw["expand_thresh"]).walk(steps, THREADS)
+    assert (ref.info["accepted"] > 0).any()
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} policy {policy} mode {mode}")
+    assert W.verify_all() == 0
+    W.close()
