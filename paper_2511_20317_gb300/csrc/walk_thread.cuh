@@ -2,6 +2,8 @@
 // (walk_link.cuh), and the one that tests every slot in every step (walk_solo.cuh) where
 // that is still the faster.
 #pragma once
+#include <algorithm>
+
 #include "walk_link.cuh"
 #include "walk_solo.cuh"
 
@@ -19,12 +21,15 @@ inline bool one_warp_each(const SegDesc &d) { return d.population <= (int64_t)12
 // expansions and reductions alternate.  Small populations keep classes all the same: their
 // short dependent loops are what few lanes a warp save most on.  Measured, 300 steps, ms
 // testing every slot / keeping classes (both in few lanes where that is faster):
-//   policy 1: Z_T (2,2,2) 1200 walkers 1.26 / 0.87, 10000 3.16 / 3.08, 18000 3.19 / 3.47;
-//     Z_2 (2,2,3) 1200 0.73 / 0.47, 2500 1.05 / 0.85, 5000 1.06 / 1.18; (2,3,3) 5000 1.71 / 1.08,
-//     10000 1.66 / 1.54, 18000 1.58 / 1.64; (2,3,4) 1200 1.05 / 0.46, 10000 1.75 / 1.35
-//   policy 2: Z_T (2,2,3) 1200 0.32 / 0.27, 5000 0.36 / 0.43; (2,3,4) 1200 0.40 / 0.26, 5000 0.45 /
-//     0.43, 18000 0.46 / 0.50, 30000 0.62 / 0.56; Z_2 (2,3,4) 1200 0.34 / 0.35, 18000 0.37 / 0.59;
-//     (4,4,5) 1200 0.68 / 0.51, 5000 0.70 / 0.74, 30000 1.04 / 1.42
+//   policy 1: Z_T (2,2,2) 11 slots, 7500 walkers 2.61 / 2.61, 10000 3.17 / 2.83, 14000 3.17 / 3.26, 30000 4.18 /
+//     4.35; 14 slots, 14000 4.65 / 4.34, 65536 12.4 / 8.1
+//     Z_2 (2,2,2) 11 slots, 2500 1.00 / 0.69, 5000 0.97 / 0.95, 7500 0.97 / 1.33, 65536 2.53 / 3.73; (2,2,3) 15
+//     slots, 2500 1.05 / 0.69, 5000 1.07 / 0.93, 7500 1.28 / 1.34, 30000 1.81 / 2.69
+//     Z_2 (2,2,3) 18 slots, 10000 1.75 / 1.48, 14000 1.71 / 2.04; (2,3,3) 21 slots, 10000 1.68 / 1.23, 14000 1.71 /
+//     1.61, 18000 1.60 / 1.69; 24 slots, 10000 1.70 / 1.41, 14000 1.69 / 1.89; (2,2,5) 26 slots, 14000 1.85 / 1.59
+//   policy 2: Z_T (2,2,3) 1200 0.31 / 0.26, 5000 0.35 / 0.43; (2,3,4) 1200 0.39 / 0.26, 5000 0.43 /
+//     0.42, 18000 0.45 / 0.51, 30000 0.62 / 0.56; Z_2 (2,3,4) 1200 0.33 / 0.34, 18000 0.35 / 0.58;
+//     (4,4,5) 1200 0.67 / 0.50, 5000 0.68 / 0.73, 30000 1.05 / 1.43
 template <int MODE, class Wd>
 inline bool every_slot_faster(const SegDesc &d) {
     constexpr bool z2 = MODE == TFG_MODE_Z2, small = sizeof(Wd) == 4;
@@ -33,7 +38,10 @@ inline bool every_slot_faster(const SegDesc &d) {
         if (z2) return small || lanes > 1;
         return small && (d.R <= 20 ? lanes > 2 : lanes > 4 && one_warp_each(d));
     }
-    if (d.walk_policy == 1) return small && (z2 ? d.R <= 24 && lanes > (d.R <= 16 ? 2 : 8) : d.R <= 12 && lanes > 8);
+    if (d.walk_policy == 1) {   // by walkers an SM
+        const int64_t walkers = std::max(d.beside, d.population);
+        return small && d.R <= (z2 ? 24 : 12) && walkers > (int64_t)(z2 && d.R <= 16 ? 40 : 80) * sm_count();
+    }
     return false;
 }
 

@@ -652,3 +652,28 @@ def test_default_mapping_of_many_walkers(fmt, mode, nw, policy, slack, kernel):
     assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} policy {policy} mode {mode}")
     assert W.verify_all() == 0
     W.close()
+
+
+@pytest.mark.parametrize("fmt,mode,nw,kernel", [((2, 2, 2), 0, 12001, "walk_link"), ((2, 2, 2), 0, 12301, "walk_solo"),
+                                                ((2, 2, 3), 1, 2500, "walk_link"), ((2, 2, 3), 1, 6201, "walk_solo"),
+                                                ((2, 3, 3), 1, 10001, "walk_link"), ((2, 3, 3), 1, 12301, "walk_solo")])
+def test_expansion_policy_on_few_slots(fmt, mode, nw, kernel):
+    """Walk policy 1 on the smallest ranks, on either side of the population (walkers an SM) from
+    which testing every slot is the faster, against the oracle."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes of a GPU of 152 SMs")
+    start, steps = naive_start(*fmt), 300
+    if mode:
+        start = np.abs(start).astype(np.int8)
+    kw = dict(plateau_len=10**6, walk_policy=1, expand_thresh=int(0.03 * 2**32))
+    W = tfg.Walkers([(fmt, mode, start, nw)], seed=26, params=tfg.tfg_default_params(use_graph=0, **kw))
+    launched = _launches(lambda: W.walk(steps).sync())
+    assert kernel in launched[0][0]
+    take = np.unique(np.concatenate([np.linspace(0, nw - 1, 40).astype(int), np.arange(nw - 4, nw)]))
+    rows = [W.read_walkers(int(w), 1) for w in take]
+    info, slots, best = (np.concatenate([x[k] for x in rows]) for k in range(3))
+    ref = oracle.Walkers(fmt, start, take, seed=26, mode=mode, plateau_len=10**6, policy=1,
+                         expand_thresh=kw["expand_thresh"]).walk(steps, THREADS)
+    assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} mode {mode}")
+    W.close()
