@@ -341,6 +341,9 @@ def run_ours(args):
                      "collected_best_ranks": best_ranks},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
                      "frac": achieved / alu_peak, "traffic": traffic,
+                     "counts": "word operations of a walk that tests every slot in every step, over the launches' "
+                               "time; a kernel that keeps factor classes executes fewer, so this is the rate of the "
+                               "method's work and no fraction of what the ALU did",
                      "frac_excluding_philox": ops_nophilox / walk_s / 1e12 / alu_peak,
                      "kernel": "walk kernels of the step (" + "; ".join(p["mapping"] for p in per_mode.values()) + ")",
                      "walk_ms_per_step": sum(walk_ms) / len(walk_ms)},

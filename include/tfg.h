@@ -386,8 +386,9 @@ void tfg_destroy(tfg_ctx *ctx);
 size_t tfg_mlp_param_bytes(void);
 
 /* Scores n candidate feature rows d_x (bf16 [n][32], device, 16-byte aligned)
- * into d_out (f32 [n], device).  Asynchronous on cuda_stream; *d_err (device
- * int32, caller-zeroed) is set to 1 if a tensor-core completion wait gave up. */
+ * into d_out (f32 [n], device).  Asynchronous on cuda_stream; *d_err (an int32
+ * in device memory or in pinned host memory, caller-zeroed) is set to 1 if a
+ * tensor-core completion wait gave up. */
 int tfg_mlp_score(const void *d_params, const uint16_t *d_x, int64_t n, float *d_out, int32_t *d_err,
                   void *cuda_stream);
 
@@ -409,7 +410,7 @@ int tfg_mlp_score(const void *d_params, const uint16_t *d_x, int64_t n, float *d
  * the parameter blob.
  * tfg_mlp_train_step: one Adam step (beta1 0.9, beta2 0.999, eps 1e-8, step
  * counted from 1) on the samples; rewrites d_params (bf16 W1, W2, f32 rest).
- * Its gradient adds the per-CTA rows in CTA order: the same inputs give the
+ * Its gradient adds the per-CTA rows in a fixed order: the same inputs give the
  * same bits on every run (on a GPU of the same SM count). */
 int tfg_mlp_grad(const void *d_params, const uint16_t *d_x, const float *d_label, const float *d_weight, int64_t n,
                  float *d_grad, int32_t *d_err, void *cuda_stream);

@@ -24,7 +24,7 @@
 // snapshots and the build as they are now).
 //
 // Bound by the latency of a step, the reads of terms from L2 and memory first; 3.3 KB
-// of shared memory per walker at 354 slots let 68 walkers reside on an SM (17 warps).
+// of shared memory per walker at 354 slots let 64 walkers reside on an SM (8 blocks, 16 warps).
 // The kernel it replaces searched all slots' 32-bit signatures with a warp per walker in
 // every step (1186 instructions a walker-step at 351 terms, now 280).  Measured, Z_T, 32768
 // walkers, 400 steps (classes built at each launch), before / now: (4,5,12) 10.7 / 5.4 ms,
