@@ -341,7 +341,7 @@ def tfg_mlp_score(params, x, out=None, err=None, stream=None):
                                ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(err.data_ptr()),
                                ctypes.c_void_p(st.cuda_stream)))
     if own_err:
-        st.synchronize()
+        _wait(st)
         if int(err) != 0:
             raise TfgError(TFG_ETIMEOUT, "tensor-core completion wait gave up")
     return out
@@ -353,6 +353,12 @@ def _host_error_word():
     read it (20000 rows scored: 53 us with a word on the device, 39 so)."""
     import torch
     return torch.zeros(1, dtype=torch.int32, pin_memory=True)
+
+
+def _wait(stream):
+    """Until the stream's work is done; a stream is anything with a cuda_stream handle."""
+    import torch
+    getattr(stream, "synchronize", torch.cuda.synchronize)()
 
 
 def _vp(t):
@@ -368,7 +374,7 @@ def tfg_mlp_grad(params, x, label, weight, stream=None):
     st = stream if stream is not None else torch.cuda.current_stream()
     _check(lib().tfg_mlp_grad(_vp(params), _vp(x), _vp(label), _vp(weight), x.shape[0], _vp(grad), _vp(err),
                               ctypes.c_void_p(st.cuda_stream)))
-    st.synchronize()
+    _wait(st)
     if int(err) != 0:
         raise TfgError(TFG_ETIMEOUT, "tensor-core completion wait gave up")
     return grad[:P], float(grad[P].item())

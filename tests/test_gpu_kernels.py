@@ -677,3 +677,17 @@ def test_expansion_policy_on_few_slots(fmt, mode, nw, kernel):
                          expand_thresh=kw["expand_thresh"]).walk(steps, THREADS)
     assert_parity(info, slots, best, ref, range(take.size), f"{fmt} {nw} mode {mode}")
     W.close()
+
+
+def test_network_calls_take_any_stream_handle():
+    """Scores and gradients on a stream given as an object that has only its handle."""
+    import types
+    import torch
+    from oracle import mlp
+    p = mlp.Params.random(np.random.default_rng(3))
+    blob = torch.from_numpy(np.frombuffer(p.blob(), dtype=np.uint8).copy()).cuda()
+    x = torch.ones((300, 32), dtype=torch.bfloat16, device="cuda")
+    label = torch.ones(300, device="cuda")
+    stream = types.SimpleNamespace(cuda_stream=torch.cuda.current_stream().cuda_stream)
+    assert torch.equal(tfg.tfg_mlp_score(blob, x, stream=stream), tfg.tfg_mlp_score(blob, x))
+    assert abs(tfg.tfg_mlp_grad(blob, x, label, label, stream=stream)[1] - tfg.tfg_mlp_grad(blob, x, label, label)[1]) < 1e-2
